@@ -45,37 +45,12 @@ struct BatchSys {
   double rel_res;
 };
 
-// Block-wide sums of NV values, broadcast to every thread.  GB300 issues about two FP64
-// operations per clock per SM with a 64-cycle latency, so the sum is done by one warp: every
-// thread stages its values in shared memory, each lane of warp 0 adds blockDim/32 of them
-// with four interleaved accumulators (fixed order), and a butterfly finishes (both partners
-// of a pair add the same two values, so every lane ends with the same bits).
+// Block-wide sums of NV values, broadcast to every thread: warp sums in integer arithmetic
+// (warp_sum; the FP64 pipe stays with the row products), then warp k adds the warps' sums.
 template <int NV>
 __device__ __forceinline__ void cta_sum(double (&v)[NV]) {
-  __shared__ double buf[NV][1024];
   __shared__ double bc[NV];
-  const int lane = threadIdx.x & 31, per = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) buf[k][threadIdx.x] = v[k];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-      int m = 0;
-      for (; m + 4 <= per; m += 4) {
-        a0 += buf[k][(m + 0) * 32 + lane];
-        a1 += buf[k][(m + 1) * 32 + lane];
-        a2 += buf[k][(m + 2) * 32 + lane];
-        a3 += buf[k][(m + 3) * 32 + lane];
-      }
-      for (; m < per; ++m) a0 += buf[k][m * 32 + lane];
-      double t = (a0 + a1) + (a2 + a3);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) bc[k] = t;
-    }
-  }
+  block_sums<NV, 32>(v, [&](int k, double t) { bc[k] = t; });
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = bc[k];
@@ -236,8 +211,7 @@ __device__ int cta_cg64(BatchSys& S, double tol, int maxit, int G) {
       if (!isfinite(v[0]) || !isfinite(v[1])) sc.status = PK_ERR_NAN;
       else if (v[1] <= 0.0) sc.status = PK_NOT_SPD;
       else {
-        sc.a = rr / v[1];
-        sc.b = sc.a * sc.a * v[0] / rr - 1.0;
+        cg_coefficients(rr, v[0], v[1], sc.a, sc.b);
       }
     }
     __syncthreads();
@@ -334,8 +308,7 @@ __device__ int cta_cg_mixed(BatchSys& S, double tol, int maxit, double tol_in, i
         if (!isfinite(u[0]) || !isfinite(u[1])) sc.status = PK_ERR_NAN;
         else if (u[1] <= 0.0) sc.status = PK_NOT_SPD;
         else {
-          sc.a = rr / u[1];
-          sc.b = sc.a * sc.a * u[0] / rr - 1.0;
+          cg_coefficients(rr, u[0], u[1], sc.a, sc.b);
         }
       }
       __syncthreads();
@@ -394,32 +367,6 @@ __global__ void __launch_bounds__(1024, 1) k_batched(BatchSys* sys, int nsys, in
 // loads per row; in the update phase x, r, p, Ap stream through the same region.  One block
 // runs 288 threads and two blocks share an SM.  Every reduction is a fixed-order block sum.
 
-// Fixed-order sum of NV values over all threads of a tile block, broadcast to every thread.
-template <int NV>
-__device__ __forceinline__ void tile_block_sum(double (&v)[NV]) {
-  __shared__ double sm[NV][kTileThreads / 32];
-  __shared__ double bc[NV];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sm[k][warp] = v[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = lane < kTileThreads / 32 ? sm[k][lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) bc[k] = t;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = bc[k];
-}
-
 __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
@@ -468,7 +415,7 @@ __device__ int tile_cg64(BatchSys& S, double tol, int maxit, DevState* st, unsig
   });
   if (consumer) fence_proxy_async_global();
   inval(bars_s, 2 * kCsrStages);
-  tile_block_sum<2>(v);
+  cta_sum<2>(v);
   if (__ldcg(&st->timeout)) return PK_TIMEOUT;  // a wait gave up: the sums are incomplete
   double rr = v[0];
   const double bb = v[1], thr2 = tol * tol * bb;
@@ -497,15 +444,14 @@ __device__ int tile_cg64(BatchSys& S, double tol, int maxit, DevState* st, unsig
     });
     if (consumer) fence_proxy_async_global();  // Ap is read back by bulk copies
     inval(bars_s, 2 * kCsrStages);
-    tile_block_sum<2>(v);
+    cta_sum<2>(v);
     if (threadIdx.x == 0) {
       s_status = kRunning;
       if (__ldcg(&st->timeout)) s_status = PK_TIMEOUT;
       else if (!isfinite(v[0]) || !isfinite(v[1])) s_status = PK_ERR_NAN;
       else if (v[1] <= 0.0) s_status = PK_NOT_SPD;
       else {
-        s_ab[0] = rr / v[1];
-        s_ab[1] = s_ab[0] * s_ab[0] * v[0] / rr - 1.0;
+        cg_coefficients(rr, v[0], v[1], s_ab[0], s_ab[1]);
       }
     }
     __syncthreads();
@@ -531,7 +477,7 @@ __device__ int tile_cg64(BatchSys& S, double tol, int maxit, DevState* st, unsig
     for (int row = ne + (int)threadIdx.x; row < n; row += blockDim.x)
       upd(row, __ldca(S.x + row), __ldca(S.r + row), __ldca(S.p + row), __ldca(S.ap + row));
     if (consumer) fence_proxy_async_global();  // x, r, p are read back by bulk copies
-    tile_block_sum<1>(w);
+    cta_sum<1>(w);
     rr = w[0];
     S.iters = it + 1;
     S.rel_res = sqrt(rr / bb);

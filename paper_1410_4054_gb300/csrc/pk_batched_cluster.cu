@@ -38,10 +38,10 @@ struct BatchClArgs {
 constexpr int kBcSlots = 4;  // block sums per CTA: <Ap,Ap>, <p,Ap> | <r,r>
 
 // Shared memory of a CTA of NT threads and up to MAXR rows: p, x, r, Ap, the slots, the
-// reduction buffer (2 NT) and MAXR + 1 row pointers (padded).
+// reduction buffer (two values per warp) and MAXR + 1 row pointers (padded).
 template <int NT, int MAXR>
 constexpr size_t bc_smem() {
-  return sizeof(double) * (4 * (size_t)MAXR + kBcSlots + 2 * NT) + sizeof(int) * (MAXR + 4);
+  return sizeof(double) * (4 * (size_t)MAXR + kBcSlots + 2 * NT / 32) + sizeof(int) * (MAXR + 4);
 }
 
 // Row l of this CTA (row pointers staged in srp) times p.
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
   __shared__ int scs;
   double* slots = sm + 4 * MAXR;
   double* buf = slots + kBcSlots;
-  int* srp = reinterpret_cast<int*>(buf + 2 * NT);  // this CTA's row pointers
+  int* srp = reinterpret_cast<int*>(buf + 2 * NT / 32);  // this CTA's row pointers
   for (;;) {
     if (rank == 0 && threadIdx.x == 0) s_sys = atomicAdd(a.queue, 1);
     cl.sync();
@@ -102,16 +102,19 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       v[0] = fma(ri, ri, v[0]);
       v[1] = fma(bi, bi, v[1]);
     }
-    double t[2];
-    cluster_block_sum<NT, 2>(v, buf, t);
-    if (threadIdx.x == 0) {
-      slots[0] = t[0];
-      slots[1] = t[1];
-    }
+    double t[2] = {0.0, 0.0};
+    cluster_block_slots<NT, 2>(v, buf, slots);
     cl.sync();  // (also: no CTA reads sp any more)
-    cluster_total<2>(cl, slots, 0, t);
-    double rr = t[0];
-    const double bb = t[1], thr2 = a.tol * a.tol * bb;
+    if (threadIdx.x < 32) {
+      cluster_total<2>(cl, slots, 0, t);
+      if (threadIdx.x == 0) {
+        sc[0] = t[0];
+        sc[1] = t[1];
+      }
+    }
+    __syncthreads();
+    double rr = sc[0];
+    const double bb = sc[1], thr2 = a.tol * a.tol * bb;
     for (int l = threadIdx.x; l < nown; l += NT) sp[l] = sr[l];  // p0 = r0
     int status = kRunning, iters = 0;
     if (!isfinite(rr) || !isfinite(bb)) status = PK_ERR_NAN;
@@ -130,21 +133,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
         v[0] = fma(y, y, v[0]);
         v[1] = fma(sp[l], y, v[1]);
       }
-      cluster_block_sum<NT, 2>(v, buf, t);
-      if (threadIdx.x == 0) {
-        slots[0] = t[0];
-        slots[1] = t[1];
-      }
+      cluster_block_slots<NT, 2>(v, buf, slots);
       cl.sync();
-      cluster_total<2>(cl, slots, 0, t);
+      if (threadIdx.x < 32) cluster_total<2>(cl, slots, 0, t);
       if (threadIdx.x == 0) {
         int sts = kRunning;
         double al = 0.0, be = 0.0;
         if (!isfinite(t[0]) || !isfinite(t[1])) sts = PK_ERR_NAN;
         else if (t[1] <= 0.0) sts = PK_NOT_SPD;
         else {
-          al = rr / t[1];
-          be = al * al * t[0] / rr - 1.0;
+          cg_coefficients(rr, t[0], t[1], al, be);
         }
         sc[0] = al;
         sc[1] = be;
@@ -166,16 +164,19 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
         sp[l] = fma(beta, pk, rn);
         w[0] = fma(rn, rn, w[0]);
       }
-      double u[1];
-      cluster_block_sum<NT, 1>(w, buf, u);
-      if (threadIdx.x == 0) slots[2] = u[0];
+      cluster_block_slots<NT, 1>(w, buf, slots + 2);
       cl.sync();
-      cluster_total<1>(cl, slots, 2, u);
-      rr = u[0];
       iters = i + 1;
-      if (!isfinite(rr)) status = PK_ERR_NAN;
-      else if (rr <= thr2) status = PK_OK;
-      else if (i + 1 >= a.maxit) status = PK_NOT_CONVERGED;
+      if (threadIdx.x < 32) {
+        double u[1];
+        cluster_total<1>(cl, slots, 2, u);
+        if (threadIdx.x == 0) {
+          rr = u[0];  // (thread 0 alone needs it from here on)
+          scs = !isfinite(rr) ? PK_ERR_NAN : rr <= thr2 ? PK_OK : i + 1 >= a.maxit ? PK_NOT_CONVERGED : kRunning;
+        }
+      }
+      __syncthreads();
+      status = scs;
     }
     for (int l = threadIdx.x; l < nown; l += NT) S.x[row0 + l] = sx[l];
     if (rank == 0 && threadIdx.x == 0) {

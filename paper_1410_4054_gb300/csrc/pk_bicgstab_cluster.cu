@@ -41,8 +41,8 @@ struct BiClusterArgs {
   DevState* st;
 };
 
-// p, s, r, Ap, As, r0* (rows each), the slots and the block-sum buffer (4 values x kBiCT).
-size_t bi_cluster_smem(int rows) { return sizeof(double) * ((size_t)6 * rows + kBiSlots + 4 * kBiCT); }
+// p, s, r, Ap, As, r0* (rows each), the slots and the block-sum buffer (3 values per warp).
+size_t bi_cluster_smem(int rows) { return sizeof(double) * ((size_t)6 * rows + kBiSlots + 3 * kBiCT / 32); }
 
 }  // namespace
 
@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
   double* const trace = st->trace;
   const int trace_cap = st->trace_cap;
   double alpha = 0.0, beta = 0.0, omega = 0.0;
+  double apr0s = 0.0;  // <Ap_i, r0*> (thread 0)
   int iters = 0;
   int status = kRunning;
   __shared__ double sc[3];  // alpha | omega, beta
@@ -91,12 +92,11 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
       w[0] = fma(y, sz[l], w[0]);
     }
     double t1[1];
-    cluster_block_sum<kBiCT, 1>(w, buf, t1);
-    if (threadIdx.x == 0) slots[0] = t1[0];
+    cluster_block_slots<kBiCT, 1>(w, buf, slots);
     cl.sync();
-    cluster_total<1>(cl, slots, 0, t1);
-    const double apr0s = t1[0];
+    if (threadIdx.x < 32) cluster_total<1>(cl, slots, 0, t1);
     if (threadIdx.x == 0) {
+      apr0s = t1[0];
       int sts = kRunning;
       double al = 0.0;
       if (!isfinite(apr0s)) sts = PK_ERR_NAN;
@@ -118,16 +118,18 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
       ss[l] = sv;
       w[0] = fma(sv, sv, w[0]);
     }
-    cluster_block_sum<kBiCT, 1>(w, buf, t1);
-    if (threadIdx.x == 0) slots[4] = t1[0];
+    cluster_block_slots<kBiCT, 1>(w, buf, slots + 4);
     cl.sync();  // (also: every CTA's s is in place for phase 3)
-    cluster_total<1>(cl, slots, 4, t1);
-    const double sn = t1[0];
-    if (!isfinite(sn)) { status = PK_ERR_NAN; break; }
-    if (sn <= thr2) {  // ||s|| small: x += alpha p ends the solve (the early exit of Alg. 3)
+    if (threadIdx.x < 32) {
+      cluster_total<1>(cl, slots, 4, t1);
+      if (threadIdx.x == 0) scs = !isfinite(t1[0]) ? PK_ERR_NAN : t1[0] <= thr2 ? PK_OK : kRunning;
+    }
+    __syncthreads();
+    if (scs == PK_ERR_NAN) { status = PK_ERR_NAN; break; }
+    if (scs == PK_OK) {  // ||s|| small: x += alpha p ends the solve (the early exit of Alg. 3)
       for (int l = threadIdx.x; l < nown; l += kBiCT) a.x[row0 + l] = fma(alpha, sp[l], a.x[row0 + l]);
-      if (lead && trace && i < trace_cap) trace[(size_t)i * 4 + 3] = sn;
-      rr = sn;
+      if (threadIdx.x == 0) rr = t1[0];
+      if (lead && trace && i < trace_cap) trace[(size_t)i * 4 + 3] = rr;
       iters = i + 1;
       status = PK_OK;
       break;
@@ -143,14 +145,9 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
       v[2] = fma(y, sz[l], v[2]);
     }
     double t3[3];
-    cluster_block_sum<kBiCT, 3>(v, buf, t3);
-    if (threadIdx.x == 0) {
-      slots[0] = t3[0];
-      slots[1] = t3[1];
-      slots[2] = t3[2];
-    }
+    cluster_block_slots<kBiCT, 3>(v, buf, slots);
     cl.sync();
-    cluster_total<3>(cl, slots, 0, t3);
+    if (threadIdx.x < 32) cluster_total<3>(cl, slots, 0, t3);
     if (threadIdx.x == 0) {
       int sts = kRunning;
       double om = 0.0, be = 0.0;
@@ -185,21 +182,24 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
       u[0] = fma(rn, sz[l], u[0]);
       u[1] = fma(rn, rn, u[1]);
     }
-    double t2[2];
-    cluster_block_sum<kBiCT, 2>(u, buf, t2);
-    if (threadIdx.x == 0) {
-      slots[4] = t2[0];
-      slots[5] = t2[1];
-    }
+    cluster_block_slots<kBiCT, 2>(u, buf, slots + 4);
     cl.sync();
-    cluster_total<2>(cl, slots, 4, t2);
-    rr0s = t2[0];
-    rr = t2[1];
     iters = i + 1;
-    if (lead && trace && i < trace_cap) trace[(size_t)i * 4 + 3] = rr;
-    if (!isfinite(rr) || !isfinite(rr0s)) { status = PK_ERR_NAN; break; }
-    if (rr <= thr2) { status = PK_OK; break; }
-    if (i + 1 >= maxit) { status = PK_NOT_CONVERGED; break; }
+    if (threadIdx.x < 32) {
+      double t2[2];
+      cluster_total<2>(cl, slots, 4, t2);
+      if (threadIdx.x == 0) {  // (thread 0 alone needs the scalars)
+        rr0s = t2[0];
+        rr = t2[1];
+        if (lead && trace && i < trace_cap) trace[(size_t)i * 4 + 3] = rr;
+        scs = !isfinite(rr) || !isfinite(rr0s) ? PK_ERR_NAN
+              : rr <= thr2                     ? PK_OK
+              : i + 1 >= maxit                 ? PK_NOT_CONVERGED
+                                               : kRunning;
+      }
+    }
+    __syncthreads();
+    if (scs != kRunning) { status = scs; break; }
   }
   if (lead && !done0) {
     st->iter = iters;

@@ -79,8 +79,8 @@ __device__ __forceinline__ void cg_alpha_beta(DevState* st, double apap, double 
   } else if (pap <= 0.0) {
     finish(st, PK_NOT_SPD);
   } else {
-    const double alpha = rr / pap;
-    const double beta = alpha * alpha * apap / rr - 1.0;
+    double alpha, beta;
+    cg_coefficients(rr, apap, pap, alpha, beta);
     st->alpha = alpha;
     st->beta = beta;
     trace_put(st, i, 0, alpha);

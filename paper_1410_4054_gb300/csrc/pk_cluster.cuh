@@ -17,70 +17,37 @@ namespace pk {
 
 namespace cg = cooperative_groups;
 
-// Fixed-order block sum of NV values over NT threads, broadcast to every thread.  GB300
-// issues about two FP64 operations per clock per SM and an FP64 add has a long latency, so the
-// sum is done by one warp with short dependency chains: every thread stages its values in buf
-// (NV * NT doubles), each lane of warp 0 adds NT/32 of them as a pairwise tree (the NV sums
-// interleaved), and a butterfly finishes (both partners of a pair add the same two values, so
-// every lane ends with the same bits).
+// Block sums of NV values over NT threads into slots[0 .. NV): warp sums (integer arithmetic,
+// pk_internal.cuh: the FP64 pipe belongs to the row products), then warp k adds the warps' values
+// of sum k.  The caller's cluster barrier publishes the slots and frees buf (NV * NT / 32 doubles).
 template <int NT, int NV>
-__device__ __forceinline__ void cluster_block_sum(const double (&v)[NV], double* buf, double (&out)[NV]) {
-  constexpr int PER = NT / 32;
-  static_assert(PER == 4 || PER == 8 || PER == 16, "4, 8 or 16 values per lane");
-  __shared__ double bc[NV];
+__device__ __forceinline__ void cluster_block_slots(double (&v)[NV], double* buf, double* slots) {
+  constexpr int NW = NT / 32;
+  static_assert(NW >= NV && NW <= 32, "one warp per sum");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) buf[k * NT + threadIdx.x] = v[k];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t[NV][PER];
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
-#pragma unroll
-      for (int m = 0; m < PER; ++m) t[k][m] = buf[k * NT + m * 32 + threadIdx.x];
-#pragma unroll
-    for (int h = PER / 2; h >= 1; h >>= 1)
-#pragma unroll
-      for (int m = 0; m < h; ++m)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) t[k][m] = t[k][m] + t[k][m + h];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) t[k][0] += __shfl_xor_sync(0xffffffffu, t[k][0], o);
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) bc[k] = t[k][0];
-    }
+  for (int k = 0; k < NV; ++k) {
+    const double t = warp_sum(v[k]);
+    if (lane == 0) buf[k * NW + warp] = t;
   }
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = bc[k];
+  if (warp < NV) {
+    const double t = warp_sum(lane < NW ? buf[warp * NW + lane] : 0.0);
+    if (lane == 0) slots[warp] = t;
+  }
 }
 
-// Cluster total of slots [s0, s0 + NV) of every CTA (after a cluster barrier): lane c of warp
-// 0 reads CTA c's values from distributed shared memory, then a butterfly over the lanes (the
-// NV sums interleaved); every CTA runs the same additions on the same values.
+// Cluster totals of slots [s0, s0 + NV) of every CTA, in warp 0 (after a cluster barrier): lane c
+// reads CTA c's values from distributed shared memory; every CTA adds the same values, so all hold
+// the same bits.  Thread 0 goes on with the scalar work and broadcasts its result.
 template <int NV>
 __device__ __forceinline__ void cluster_total(cg::cluster_group& cl, double* slots, int s0, double (&out)[NV]) {
-  __shared__ double bc[NV];
-  if (threadIdx.x < 32) {
-    const int C = (int)cl.num_blocks();
-    double t[NV];
-    const double* rem = threadIdx.x < C ? cl.map_shared_rank(slots, (int)threadIdx.x) : nullptr;
+  const int lane = threadIdx.x & 31;
+  const double* rem = lane < (int)cl.num_blocks() ? cl.map_shared_rank(slots, lane) : nullptr;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) t[k] = rem ? rem[s0 + k] : 0.0;
+  for (int k = 0; k < NV; ++k) out[k] = rem ? rem[s0 + k] : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) bc[k] = t[k];
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = bc[k];
+  for (int k = 0; k < NV; ++k) out[k] = warp_sum(out[k]);
 }
 
 // Element `c` of a vector distributed over the cluster, R = 2^lg rows per CTA, each CTA's part

@@ -62,6 +62,27 @@ struct GmArgs {
   DevState* st;
 };
 
+// The reductions of this file stay FP64 trees (TREE, warp_sum_tree): classical Gram-Schmidt
+// divides their rounding by R_{i,i}, so any other rounding of equal quality moves xi_i of a badly
+// scaled matrix by as much as its parity bar (1.7e-12 against 1e-12 on rows of 9,000 nonzeros
+// among rows of 3), and the integer sums gain only 2 % of a step here.
+template <int NV>
+__device__ __forceinline__ void gm_final_sums(const double* partials, double (&out)[NV]) {
+  __shared__ double sm[NV];
+  if (threadIdx.x < 32) {
+    double t[NV];
+    lane_slot_sums<NV, (NV <= 2 ? 6 : 4)>(partials, gridDim.x, threadIdx.x, t);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const double u = warp_sum_tree(t[k]);
+      if (threadIdx.x == 0) sm[k] = u;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) out[k] = sm[k];
+}
+
 __device__ __forceinline__ void cond2_set(DevState* st, unsigned v) {
   if (st->use_cond) cudaGraphSetConditional(st->cond2, v);
 }
@@ -100,10 +121,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm_start(CsrTiles T, GmArgs
     }
     return;
   }
-  tile_block_partials<2>(v, g.partials);
+  tile_block_partials<2, true>(v, g.partials);
   if (arrive_last(&st->counter)) {
     double t[2];
-    final_sums<2>(g.partials, t);
+    gm_final_sums<2>(g.partials, t);
     if (threadIdx.x == 0) {
       if (st->gm_cycle == 0) {
         const double tol = st->thr2;
@@ -186,10 +207,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm1(CsrTiles T, GmArgs g) {
     }
   });
   if (!__syncthreads_or(threadIdx.x < kConsumers && live)) return;
-  tile_block_partials<NV>(v, g.partials);
+  tile_block_partials<NV, true>(v, g.partials);
   if (arrive_last(&st->counter)) {
     double t[NV];
-    final_sums<NV>(g.partials, t);
+    gm_final_sums<NV>(g.partials, t);
     if (threadIdx.x == 0) {
       if (i >= 2) g.R[(i - 1) * kRld + i] = t[0];
       if (SHIFT) {
@@ -406,7 +427,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm2(GmArgs g, int pass) {
         for (int q = 0; q < 8; ++q)
           if (base + 32 * q < G) t += v[q];
       }
-      t = warp_sum(t);
+      t = warp_sum_tree(t);
       if (lane == 0) {
         if (pass) g.C[j] = t;
         else g.R[j * kRld + i] = t;
@@ -536,11 +557,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm3(GmArgs g, int mode) {
     }
   }
   if (mode == 1) return;
-  tile_block_partials<1>(v, g.partials);
+  tile_block_partials<1, true>(v, g.partials);
   if (shift) {
     if (arrive_last(&st->counter)) {
       double t[1];
-      final_sums<1>(g.partials, t);
+      gm_final_sums<1>(g.partials, t);
       if (threadIdx.x == 0) {
         if (__ldcg(&st->timeout)) {
           gm_finish(st, PK_TIMEOUT);
@@ -564,7 +585,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm3(GmArgs g, int mode) {
   }
   if (arrive_last(&st->counter)) {
     double t[1];
-    final_sums<1>(g.partials, t);
+    gm_final_sums<1>(g.partials, t);
     if (threadIdx.x == 0) {
       const double nrm2 = t[0];
       double col2 = nrm2;
@@ -618,10 +639,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_gm4(GmArgs g) {
     }
   });
   if (!__syncthreads_or(threadIdx.x < kConsumers && live)) return;
-  tile_block_partials<1>(v, g.partials);
+  tile_block_partials<1, true>(v, g.partials);
   if (arrive_last(&st->counter)) {
     double t[1];
-    final_sums<1>(g.partials, t);
+    gm_final_sums<1>(g.partials, t);
     if (threadIdx.x == 0) {
       const double xi_i = t[0];
       st->s[1] += xi_i * xi_i;
@@ -654,10 +675,10 @@ __global__ void __launch_bounds__(kBlock) k_gmc_xi(GmArgs g) {
   ew_range(g.n, r0, r1);
   double v[1] = {0.0};
   for (int row = r0 + threadIdx.x; row < r1; row += blockDim.x) v[0] = fma(g.r[row], vi[row], v[0]);
-  block_partials<1>(v, g.partials);
+  block_partials<1, true>(v, g.partials);
   if (arrive_last(&st->counter)) {
     double t[1];
-    final_sums<1>(g.partials, t);
+    gm_final_sums<1>(g.partials, t);
     if (threadIdx.x == 0) {
       g.xi[i] = t[0];
       st->counter = 0;
@@ -686,10 +707,10 @@ __global__ void __launch_bounds__(kBlock) k_gmc_rnorm(GmArgs g) {
   ew_range(g.n, r0, r1);
   double v[1] = {0.0};
   for (int row = r0 + threadIdx.x; row < r1; row += blockDim.x) v[0] = fma(g.r[row], g.r[row], v[0]);
-  block_partials<1>(v, g.partials);
+  block_partials<1, true>(v, g.partials);
   if (arrive_last(&st->counter)) {
     double t[1];
-    final_sums<1>(g.partials, t);
+    gm_final_sums<1>(g.partials, t);
     if (threadIdx.x == 0) {
       gm_step_done(st, g, i, g.xi[i], t[0]);
       st->counter = 0;
@@ -709,7 +730,7 @@ __global__ void __launch_bounds__(kBlock) k_gm_end(GmArgs g) {
     for (int ii = k; ii >= 1; --ii) {
       double s = 0.0;
       for (int j = ii + 1 + lane; j <= k; j += 32) s = fma(ld_cg(g.R + ii * kRld + j), eta[j], s);
-      s = warp_sum(s);
+      s = warp_sum_tree(s);
       if (lane == 0) eta[ii] = (ld_cg(g.xi + ii) - s) / ld_cg(g.R + ii * kRld + ii);
       __syncwarp();
     }

@@ -55,18 +55,15 @@ size_t gc_smem(int rows) {
   return sizeof(double) * ((size_t)2 * rows + (size_t)kGcLd * kGcLd + 2 * kGcLd + 2 * kGcSlots + kGcWarps);
 }
 
-// Sum of one value over the CTA, valid in thread 0: a fixed xor butterfly per warp, then
-// thread 0 adds the warp partials in warp order.  (On GB300 an FP64 operation repeated by
-// every thread of the CTA costs the narrow FP64 pipe, so scalar work stays in thread 0.)
+// Sum of one value over the CTA, valid in warp 0: warp sums, then warp 0 adds them.  (On GB300
+// an FP64 operation repeated by every thread of the CTA costs the narrow FP64 pipe, so scalar
+// work stays in thread 0.)
 __device__ __forceinline__ double gc_block_sum(double v, double* wp) {
   v = warp_sum(v);
   if ((threadIdx.x & 31) == 0) wp[threadIdx.x >> 5] = v;
   __syncthreads();
   double t = 0.0;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int w = 0; w < kGcWarps; ++w) t += wp[w];
-  }
+  if (threadIdx.x < 32) t = warp_sum((int)threadIdx.x < kGcWarps ? wp[threadIdx.x] : 0.0);
   __syncthreads();  // (wp is reused by the next sum)
   return t;
 }

@@ -56,33 +56,79 @@ struct DevState {
 __device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ int ld_cg(const int* p) { return __ldcg(p); }
 
-// Warp sum with a fixed xor tree: every lane ends with the same, order-fixed sum.
-__device__ __forceinline__ double warp_sum(double v) {
+// Warp sum by the fixed xor tree in FP64: every lane ends with the same, order-fixed sum.
+__device__ __forceinline__ double warp_sum_tree(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// First reduction stage: block sum of NV per-thread values into partials[k * G + block].
-template <int NV>
-__device__ __forceinline__ void block_partials(double (&v)[NV], double* partials) {
-  __shared__ double sm[NV][kBlock / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Sum of a warp's 32 values, the same in every lane, in integer arithmetic.  GB300 issues an
+// FP64 warp instruction every 64 clocks per scheduler, so the five adds of a butterfly cost
+// 320 clocks of a pipe that the row products need, and a block's reduction of three inner
+// products by nine warps took about 1.9 us at the end of every fused kernel.  Here every value
+// becomes a 64-bit integer in units of 2^-5 of the largest value's last place, the integers are
+// added exactly (three limbs, one redux.sync each), and the total is rounded once to FP64: about
+// forty integer instructions.  The error is at most half a last place of the largest value
+// (32 roundings of 2^-6) plus the final rounding, below the tree's bound of five roundings of
+// partial sums, and the result does not depend on the order of the lanes.  Values near the ends
+// of the exponent range (and Inf, NaN) take the tree.
+__device__ __forceinline__ double warp_sum(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int e = (int)(b >> 52) & 0x7ff;
+  const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (em < 64 || em > 0x7f0) return warp_sum_tree(v);  // the same branch in every lane
+  // |v| = m 2^(e - 1075); m << 5 < 2^58, so 32 of them fit a signed 64-bit sum.  (em >= 64: a
+  // subnormal v, whose implicit bit is not set in m, is shifted out either way.)
+  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 5;
+  const int sh = min(em - e, 62);
+  long long q = (long long)((m + ((1ull << sh) >> 1)) >> sh);
+  if ((long long)b < 0) q = -q;
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3ffffffu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26) & 0x3ffffffu);
+  const int l2 = __reduce_add_sync(0xffffffffu, (int)(q >> 52));
+  const long long t = ((long long)l2 << 52) + ((long long)l1 << 26) + (long long)l0;
+  // t 2^(em - 1080): the exponent of a nonzero t is at least 1023, so it stays in range
+  const long long r = __double_as_longlong((double)t);
+  return t ? __longlong_as_double(r + ((long long)(em - 1080) << 52)) : 0.0;
+}
+
+// Eq. (3): alpha_i = <r_i,r_i>/<p_i,Ap_i>, beta_i = alpha_i^2 <Ap_i,Ap_i>/<r_i,r_i> - 1, the
+// quotient of beta formed beside alpha's instead of after it (an FP64 division is about 550
+// clocks on GB300, and this is on every iteration's critical path).  The product is rounded
+// before 1 is taken off: fused, beta p would cancel r exactly once a 1 x 1 system is solved, and
+// a fixed-count run would end with p = 0 instead of going on.
+__device__ __forceinline__ void cg_coefficients(double rr, double apap, double pap, double& alpha, double& beta) {
+  alpha = rr / pap;
+  const double q = apap / rr;
+  beta = __dadd_rn(__dmul_rn(__dmul_rn(alpha, alpha), q), -1.0);
+}
+
+// Block sums of NV values per thread, sum k in every lane of warp k % warps; `put(k, total)` is
+// called once per sum, by one lane.  Warp sums first, then one warp per sum adds the warps'.
+// TREE: by FP64 trees, as the Gram-Schmidt kernels of GMRES want it (see there).
+template <int NV, int MAXW, bool TREE = false, class Put>
+__device__ __forceinline__ void block_sums(double (&v)[NV], Put&& put) {
+  __shared__ double sm[NV][MAXW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
+  for (int k = 0; k < NV; ++k) v[k] = TREE ? warp_sum_tree(v[k]) : warp_sum(v[k]);
   if (lane == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) sm[k][warp] = v[k];
   }
   __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = lane < (int)(blockDim.x >> 5) ? sm[k][lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) partials[(size_t)k * gridDim.x + blockIdx.x] = t;
-    }
+  for (int k = warp; k < NV; k += nw) {
+    const double u = lane < nw ? sm[k][lane] : 0.0;
+    const double t = TREE ? warp_sum_tree(u) : warp_sum(u);
+    if (lane == 0) put(k, t);
   }
+}
+
+// First reduction stage: block sum of NV per-thread values into partials[k * G + block].
+template <int NV, bool TREE = false>
+__device__ __forceinline__ void block_partials(double (&v)[NV], double* partials) {
+  block_sums<NV, kBlock / 32, TREE>(v, [&](int k, double t) { partials[(size_t)k * gridDim.x + blockIdx.x] = t; });
 }
 
 // Float-float accumulator for FP32 inner products: s.hi + s.lo holds the running sum of the
@@ -153,25 +199,40 @@ __device__ __forceinline__ void lane_slot_sums(const double* partials, int G, in
 }
 
 // Second reduction stage in the last block: out[k] = sum over blocks of partials[k][.], in a
-// fixed order, broadcast to every thread.  One warp does it (two interleaved accumulators
-// per lane, loads issued in batches, then a butterfly): on GB300 every FP64 instruction that
-// all warps of the block would issue costs the SM's narrow FP64 pipe, and this runs on the
-// critical path.
+// fixed order, broadcast to every thread.  This runs on the critical path of every iteration.
+// The NV x G slots are cut into groups of 32; every warp takes groups, so all loads are in flight
+// at once (one L2 round trip), and adds each with warp_sum; then one warp per sum adds the
+// groups' sums.
+constexpr int kMaxSlotGroups = 64;  // G <= 2048 blocks
 template <int NV>
 __device__ __forceinline__ void final_sums(const double* partials, double (&out)[NV]) {
+  __shared__ double gs[NV][kMaxSlotGroups];
   __shared__ double sm[NV];
-  const int G = gridDim.x;
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    double t[NV];
-    lane_slot_sums<NV, (NV <= 2 ? 6 : 4)>(partials, G, lane, t);
+  const int G = gridDim.x, ng = (G + 31) >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+  constexpr int B = 4;  // groups a warp loads before it adds them
+  for (int q0 = warp; q0 < NV * ng; q0 += B * nw) {
+    double v[B];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double u = t[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-      if (lane == 0) sm[k] = u;
+    for (int u = 0; u < B; ++u) {
+      const int q = q0 + u * nw, k = q / ng, c = (q - k * ng) * 32 + lane;
+      v[u] = q < NV * ng && c < G ? ld_cg(partials + (size_t)k * G + c) : 0.0;
     }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      const int q = q0 + u * nw, k = q / ng;
+      if (q < NV * ng) {
+        const double t = warp_sum(v[u]);
+        if (lane == 0) gs[k][q - k * ng] = t;
+      }
+    }
+  }
+  __syncthreads();
+  for (int k = warp; k < NV; k += nw) {
+    double t = lane < ng ? gs[k][lane] : 0.0;
+    if (lane + 32 < ng) t += gs[k][lane + 32];
+    t = warp_sum(t);
+    if (lane == 0) sm[k] = t;
   }
   __syncthreads();
 #pragma unroll

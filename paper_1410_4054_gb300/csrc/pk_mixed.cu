@@ -178,8 +178,7 @@ __global__ void __launch_bounds__(kBlock) k_mx_spmv(MxArgs a) {
       if (!isfinite(t[0]) || !isfinite(t[1])) mx_finish(st, PK_ERR_NAN);
       else if (t[1] <= 0.0) mx_finish(st, PK_NOT_SPD);
       else {
-        st->alpha = rr / t[1];
-        st->beta = st->alpha * st->alpha * t[0] / rr - 1.0;
+        cg_coefficients(rr, t[0], t[1], st->alpha, st->beta);
       }
       st->counter = 0;
     }
@@ -254,8 +253,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_mx_spmv_tma(CsrTilesT<float
       else if (!isfinite(t[0]) || !isfinite(t[1])) mx_finish(st, PK_ERR_NAN);
       else if (t[1] <= 0.0) mx_finish(st, PK_NOT_SPD);
       else {
-        st->alpha = rr / t[1];
-        st->beta = st->alpha * st->alpha * t[0] / rr - 1.0;
+        cg_coefficients(rr, t[0], t[1], st->alpha, st->beta);
       }
       st->counter = 0;
     }

@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_pcg_spmv_dots_tma(CsrTiles 
       } else if (t[0] <= 0.0) {
         finish(st, PK_NOT_SPD);
       } else {
-        const double alpha = gamma / t[0];
-        const double beta = alpha * alpha * t[1] / gamma - 1.0;
+        double alpha, beta;
+        cg_coefficients(gamma, t[1], t[0], alpha, beta);
         st->alpha = alpha;
         st->beta = beta;
         trace_put(st, st->iter, 0, alpha);

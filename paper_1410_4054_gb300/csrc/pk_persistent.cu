@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
   double* sr = sm + 2 * R;
   double* sa = sm + 3 * R;    // Ap
   double* slots = sm + 4 * R; // kSlots block sums
-  double* buf = slots + kSlots; // 2 * kCT staging values of block_sum
+  double* buf = slots + kSlots; // warp sums of cluster_block_slots
   const int row0 = rank * R;
   const int nown = max(0, min(a.n - row0, R));
   DevState* st = a.st;
@@ -83,11 +83,10 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
       v[0] = fma(s, s, v[0]);
       v[1] = fma(sp[l], s, v[1]);
     }
-    double t[2];
-    cluster_block_sum<kCT, 2>(v, buf, t);
-    if (threadIdx.x == 0) { slots[0] = t[0]; slots[1] = t[1]; }
+    cluster_block_slots<kCT, 2>(v, buf, slots);
     cl.sync();
-    cluster_total<2>(cl, slots, 0, t);
+    double t[2];
+    if (threadIdx.x < 32) cluster_total<2>(cl, slots, 0, t);
     // the scalar work (two FP64 divisions) runs in one thread and is broadcast: on GB300 every
     // FP64 instruction issued by all warps of a CTA costs the SM's narrow FP64 pipe
     if (threadIdx.x == 0) {
@@ -97,8 +96,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
       else if (t[1] <= 0.0) sts = PK_NOT_SPD;
       else {
         // Eq. (3): alpha_i = <r_i,r_i>/<p_i,Ap_i>, beta_i = alpha_i^2 <Ap_i,Ap_i>/<r_i,r_i> - 1
-        al = rr / t[1];
-        be = al * al * t[0] / rr - 1.0;
+        cg_coefficients(rr, t[0], t[1], al, be);
         if (lead && trace && i < trace_cap) {
           trace[(size_t)i * 4 + 0] = al;
           trace[(size_t)i * 4 + 1] = be;
@@ -124,14 +122,13 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
       sp[l] = fma(beta, pk, rn);
       w[0] = fma(rn, rn, w[0]);
     }
-    double u[1];
-    cluster_block_sum<kCT, 1>(w, buf, u);
-    if (threadIdx.x == 0) slots[2] = u[0];
+    cluster_block_slots<kCT, 1>(w, buf, slots + 2);
     cl.sync();
-    cluster_total<1>(cl, slots, 2, u);
-    rr = u[0];
+    double u[1];
+    if (threadIdx.x < 32) cluster_total<1>(cl, slots, 2, u);
     iters = i + 1;
     if (threadIdx.x == 0) {
+      rr = u[0];  // (thread 0 alone needs it)
       int sts = kRunning;
       if (!isfinite(rr)) sts = PK_ERR_NAN;
       else if (rr <= thr2) sts = PK_OK;
@@ -160,7 +157,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
   cl.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-size_t cluster_smem(int rows) { return sizeof(double) * ((size_t)4 * rows + kSlots + 2 * kCT); }
+size_t cluster_smem(int rows) { return sizeof(double) * ((size_t)4 * rows + kSlots + 2 * kCT / 32); }
 
 // Cluster size the device runs with the largest shared-memory footprint (16, else 8); 0 if
 // neither.

@@ -195,8 +195,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cg_resident(ResArgs a) {
         else if (!isfinite(t[1]) || !isfinite(t[2])) status = PK_ERR_NAN;
         else if (t[2] <= 0.0) status = PK_NOT_SPD;
         else {
-          alpha = rr / t[2];
-          beta = alpha * alpha * t[1] / rr - 1.0;
+          cg_coefficients(rr, t[1], t[2], alpha, beta);
         }
       }
       if (b == 0 && ok) {
@@ -292,8 +291,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cg_resident(ResArgs a) {
     });
     if (consumer) fence_proxy_async();  // Ap is read back by this block's bulk copies in U_{i+1}
     // ---- this block's part of iteration i's reductions: slot (i & 1), then its arrival
-    tile_block_partials<3>(v, a.partials + (size_t)(i & 1) * 3 * G);  // written by thread 0
+    tile_block_partials<3>(v, a.partials + (size_t)(i & 1) * 3 * G);
     inval_ring(bars_s, 2 * kCsrStages);  // (after the barrier inside: the CSR ring is idle)
+    __syncthreads();  // the three sums are written, one per warp, before thread 0's release
     if (threadIdx.x == 0) {
       st_release(&a.arrive[b], i + 1);
       s_stop = __ldcg(&st->timeout);

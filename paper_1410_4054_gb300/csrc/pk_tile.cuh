@@ -132,25 +132,9 @@ __device__ __forceinline__ void report_timeout(DevState* st) {
 
 // Reduction of NV values over the consumer threads of a tile block (the producer warp
 // contributes zeros), written to partials[k * gridDim.x + blockIdx.x].
-template <int NV>
+template <int NV, bool TREE = false>
 __device__ __forceinline__ void tile_block_partials(double (&v)[NV], double* partials) {
-  __shared__ double sm[NV][kTileThreads / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sm[k][warp] = v[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double t = lane < kTileThreads / 32 ? sm[k][lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) partials[(size_t)k * gridDim.x + blockIdx.x] = t;
-    }
-  }
+  block_sums<NV, kTileThreads / 32, TREE>(v, [&](int k, double t) { partials[(size_t)k * gridDim.x + blockIdx.x] = t; });
 }
 
 // ----------------------------------------------------------------------------------------
