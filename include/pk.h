@@ -78,7 +78,14 @@ enum {
                         the block partials itself in a fixed order; for n <=
                         PK_PERSISTENT_MAX_N.  Larger n, other variants, precisions, GMRES
                         with PK_FLAG_CGS2 or PK_FLAG_GM_SHIFT return PK_ERR_ARG */
-  PK_LOOP_AUTO = 3,  /* PK_LOOP_PERSISTENT for pipelined FP64 CG with n <= PK_PERSISTENT_AUTO_N
+  PK_LOOP_AUTO = 3,  /* by size.  The smallest pipelined FP64 CG and BiCGStab solves (nnz + 6 n up to
+                        120,000) and what fits nothing below run on one cluster; then, as long as
+                        the matrix and the solver vectors fit the GPU's shared memory (7-point
+                        stencils to about 270,000 rows), the whole loop runs in one cooperative
+                        launch that keeps them there (one solve at a time per process; a solve
+                        of another host thread meanwhile takes the graph).  Where CG's graph loop
+                        runs on more than 65,536 rows, both give the same bits.  In detail:
+                        PK_LOOP_PERSISTENT for pipelined FP64 CG with n <= PK_PERSISTENT_AUTO_N
                         and nnz <= PK_PERSISTENT_AUTO_NNZ, pipelined BiCGStab with n <=
                         PK_PERSISTENT_BICGSTAB_AUTO_N and nnz <= PK_PERSISTENT_BICGSTAB_AUTO_NNZ,
                         and pipelined GMRES (one Gram-Schmidt pass) with n <=

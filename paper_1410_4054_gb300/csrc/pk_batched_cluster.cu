@@ -135,18 +135,20 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       }
       cluster_block_slots<NT, 2>(v, buf, slots);
       cl.sync();
-      if (threadIdx.x < 32) cluster_total<2>(cl, slots, 0, t);
-      if (threadIdx.x == 0) {
+      if (threadIdx.x < 32) {
+        cluster_total<2>(cl, slots, 0, t);
         int sts = kRunning;
         double al = 0.0, be = 0.0;
         if (!isfinite(t[0]) || !isfinite(t[1])) sts = PK_ERR_NAN;
         else if (t[1] <= 0.0) sts = PK_NOT_SPD;
         else {
-          cg_coefficients(rr, t[0], t[1], al, be);
+          cg_coefficients_warp(rr, t[0], t[1], al, be);
         }
-        sc[0] = al;
-        sc[1] = be;
-        scs = sts;
+        if (threadIdx.x == 0) {
+          sc[0] = al;
+          sc[1] = be;
+          scs = sts;
+        }
       }
       __syncthreads();
       if (scs != kRunning) {
@@ -170,8 +172,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       if (threadIdx.x < 32) {
         double u[1];
         cluster_total<1>(cl, slots, 2, u);
+        rr = u[0];  // (warp 0 alone needs it from here on)
         if (threadIdx.x == 0) {
-          rr = u[0];  // (thread 0 alone needs it from here on)
           scs = !isfinite(rr) ? PK_ERR_NAN : rr <= thr2 ? PK_OK : i + 1 >= a.maxit ? PK_NOT_CONVERGED : kRunning;
         }
       }

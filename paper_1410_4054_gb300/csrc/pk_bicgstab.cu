@@ -15,7 +15,7 @@
 #include <cmath>
 
 #include "pk_guard.cuh"
-#include "pk_tile.cuh"
+#include "pk_sm.cuh"
 
 namespace pk {
 
@@ -427,6 +427,10 @@ static pk_status bi_tma_setup() {
 // pk_bicgstab_cluster.cu: the whole pipelined loop on one thread-block cluster
 bool bicgstab_persistent_usable(const pk_csr* A);
 pk_status launch_bicgstab_persistent(pk_csr* A, double* x, const double* r, const double* r0s, cudaStream_t s);
+// pk_sm_bicgstab.cu: the loop with the matrix in shared memory
+pk_status sm_bicgstab_usable(pk_csr* A, cudaStream_t s, bool* usable);
+pk_status launch_sm_bicgstab(pk_csr* A, double* x, const double* r, const double* r0s, double* as, int maxit,
+                             cudaStream_t s);
 
 pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_info* info,
                          cudaStream_t s) {
@@ -463,6 +467,16 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
                  A->nnz <= PK_PERSISTENT_BICGSTAB_AUTO_NNZ && A->stats.tiles_long == 0 &&
                  !(o->flags & PK_FLAG_TIMING) && bicgstab_persistent_usable(A);
   }
+  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
+  // other host thread's is running
+  bool sm = false;
+  SmTurn turn;
+  if (o->loop == PK_LOOP_AUTO && !(persistent && cluster_size_work(A)) && o->variant == PK_VARIANT_PIPELINED &&
+      !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
+    if ((e = sm_bicgstab_usable(A, s, &sm))) return e;
+    sm = sm && turn.take();
+    if (sm) persistent = false;
+  }
   cudaEvent_t e0, e1;
   PK_CUDA(cudaEventCreate(&e0));
   PK_CUDA(cudaEventCreate(&e1));
@@ -474,7 +488,7 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
   if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (e = work_vec(A, 2, &ap)) ||
       (e = work_vec(A, 3, &sv)) || (e = work_vec(A, 4, &as)) || (e = work_vec(A, 5, &r0s)))
     return e;
-  const bool tma = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && o->variant == PK_VARIANT_PIPELINED && !persistent;
+  const bool tma = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && o->variant == PK_VARIANT_PIPELINED && !persistent && !sm;
   // the classical form's SpMV runs on the same tile engine (only the fusion differs)
   const bool tma_spmv = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA);
   double* xd = v.x_dev;
@@ -509,17 +523,19 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
   launch_zero_x(A, xd, s);
   launches += 2;
   PK_CUDA(cudaGetLastError());
-  if (persistent) {
+  if (persistent || sm) {
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    if ((e = launch_bicgstab_persistent(A, xd, r, r0s, s))) return e;
+    if ((e = sm ? launch_sm_bicgstab(A, xd, r, r0s, as, o->maxit, s) : launch_bicgstab_persistent(A, xd, r, r0s, s)))
+      return e;
     if ((e = T.end())) return e;
-    launches += 1;
+    launches += sm ? 2 : 1;
     if ((e = T.flush())) return e;
     if (jac.A) {
       if ((e = jacobi_right_leave(&jac, xd, s))) return e;
       launches += 2;
     }
     if ((e = finish_info(A, o, info, s, v, e0, e1, launches))) return e;
+    if (sm && info->status != PK_TIMEOUT) sm_done(A, 2 * (uint64_t)info->iters + 6);
     for (int k = 0; k < PK_MAX_KERNEL_SLOTS; ++k) {
       info->kernel_count[k] = T.count[k];
       info->kernel_ms[k] = T.count[k] ? T.ms[k] / T.count[k] : 0.0;

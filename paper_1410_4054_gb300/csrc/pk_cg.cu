@@ -13,7 +13,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "pk_tile.cuh"
+#include "pk_sm.cuh"
 
 namespace pk {
 
@@ -70,17 +70,19 @@ __global__ void __launch_bounds__(kBlock) k_zero_x(RowArgs a, double* __restrict
   for (int row = r0 + threadIdx.x; row < r1; row += blockDim.x) x[row] = 0.0;
 }
 
-// Second stage shared by K-CG-S and the split dots kernel: alpha_i and beta_i (Eq. (3)).
+// Second stage shared by K-CG-S and the split dots kernel: alpha_i and beta_i (Eq. (3)), by one
+// warp of the last block.
 __device__ __forceinline__ void cg_alpha_beta(DevState* st, double apap, double pap) {
   const double rr = st->rr;
   const int i = st->iter;
+  double alpha, beta;
+  cg_coefficients_warp(rr, apap, pap, alpha, beta);
+  if (threadIdx.x) return;
   if (!isfinite(apap) || !isfinite(pap)) {
     finish(st, PK_ERR_NAN);
   } else if (pap <= 0.0) {
     finish(st, PK_NOT_SPD);
   } else {
-    double alpha, beta;
-    cg_coefficients(rr, apap, pap, alpha, beta);
     st->alpha = alpha;
     st->beta = beta;
     trace_put(st, i, 0, alpha);
@@ -104,10 +106,8 @@ __global__ void __launch_bounds__(kBlock, 8) k_cg_spmv_dots(RowArgs a, const dou
   if (arrive_last(&a.st->counter)) {
     double t[2];
     final_sums<2>(a.partials, t);
-    if (threadIdx.x == 0) {
-      cg_alpha_beta(a.st, t[0], t[1]);
-      a.st->counter = 0;
-    }
+    if (threadIdx.x < 32) cg_alpha_beta(a.st, t[0], t[1]);
+    if (threadIdx.x == 0) a.st->counter = 0;
   }
 }
 
@@ -126,10 +126,8 @@ __global__ void __launch_bounds__(kBlock) k_cg_dots(RowArgs a, const double* __r
   if (arrive_last(&a.st->counter)) {
     double t[2];
     final_sums<2>(a.partials, t);
-    if (threadIdx.x == 0) {
-      cg_alpha_beta(a.st, t[0], t[1]);
-      a.st->counter = 0;
-    }
+    if (threadIdx.x < 32) cg_alpha_beta(a.st, t[0], t[1]);
+    if (threadIdx.x == 0) a.st->counter = 0;
   }
 }
 
@@ -205,7 +203,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_update(RowArgs a, double* __restr
 
 // K-CG-U on the streaming tile engine: inputs p, x, Ap, r arrive in shared memory through
 // bulk copies; results are stored straight to global memory.
-__global__ void __launch_bounds__(kTileThreads, 2) k_cg_update_tma(int n, double* __restrict__ x,
+__global__ void __launch_bounds__(kTileThreads, 2) k_cg_update_tma(int n, const int32_t* rows, double* __restrict__ x,
                                                                    double* __restrict__ r,
                                                                    double* __restrict__ p,
                                                                    const double* __restrict__ ap,
@@ -213,7 +211,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cg_update_tma(int n, double
   extern __shared__ __align__(128) unsigned char smem[];
   count_pass(st);
   int r0, r1;
-  ew_range(n, r0, r1);
+  if (rows) {  // (see rows_by_tile_block)
+    r0 = __ldg(rows + blockIdx.x);
+    r1 = __ldg(rows + blockIdx.x + 1);
+  } else {
+    ew_range(n, r0, r1);
+  }
   double v[1] = {0.0};
   double alpha = 0.0, beta = 0.0;
   // x and r do not depend on the preceding K-CG-S: prefetched before the dependency wait
@@ -288,11 +291,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_cg_spmv_dots_tma(CsrTiles T
   if (arrive_last(&st->counter)) {
     double t[2];
     final_sums<2>(partials, t);
-    if (threadIdx.x == 0) {
-      if (__ldcg(&st->timeout)) finish(st, PK_TIMEOUT);
-      else cg_alpha_beta(st, t[0], t[1]);
-      st->counter = 0;
+    if (threadIdx.x < 32) {
+      if (!__ldcg(&st->timeout)) cg_alpha_beta(st, t[0], t[1]);
+      else if (threadIdx.x == 0) finish(st, PK_TIMEOUT);
     }
+    if (threadIdx.x == 0) st->counter = 0;
   }
 }
 
@@ -322,10 +325,8 @@ __global__ void __launch_bounds__(kBlock) k_cg_sell_spmv_dots(SellArgs s, const 
   if (arrive_last(&st->counter)) {
     double t[2];
     final_sums<2>(partials, t);
-    if (threadIdx.x == 0) {
-      cg_alpha_beta(st, t[0], t[1]);
-      st->counter = 0;
-    }
+    if (threadIdx.x < 32) cg_alpha_beta(st, t[0], t[1]);
+    if (threadIdx.x == 0) st->counter = 0;
   }
 }
 
@@ -443,6 +444,8 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
 pk_status launch_cg_persistent(pk_csr* A, double* x, double* r, double* p, double* ap,
                                cudaStream_t s);
 pk_status resident_prepare(pk_csr* A, cudaStream_t s, bool* usable);
+pk_status sm_cg_usable(pk_csr* A, cudaStream_t s, bool* usable);
+pk_status launch_sm_cg(pk_csr* A, double* x, const double* r, const double* p, int maxit, cudaStream_t s);
 pk_status launch_cg_resident(pk_csr* A, double* x, double* r, double* p, double* ap, cudaStream_t s);
 
 pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_info* info,
@@ -480,6 +483,16 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
                  A->nnz <= PK_PERSISTENT_AUTO_NNZ &&
                  !(o->flags & PK_FLAG_TIMING) && persistent_usable(A, o);
   }
+  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
+  // other host thread's is running
+  bool sm = false;
+  SmTurn turn;
+  if (o->loop == PK_LOOP_AUTO && !(persistent && cluster_size_work(A)) && !sell &&
+      o->variant == PK_VARIANT_PIPELINED && !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
+    if ((e = sm_cg_usable(A, s, &sm))) return e;
+    sm = sm && turn.take();
+    if (sm) persistent = false;
+  }
   bool resident = false;
   if (o->loop == PK_LOOP_RESIDENT) {
     if (o->variant != PK_VARIANT_PIPELINED || sell || (o->flags & PK_FLAG_NO_TMA)) {
@@ -506,7 +519,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   double* xd = v.x_dev;
   // The bulk-copy kernels read x in 16-byte units: a caller's x that is not 16-byte aligned or
   // has odd length is iterated in a padded library copy.
-  const bool tma_engine = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && !persistent;
+  const bool tma_engine = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && !persistent && !sm;
   double* x_copy_back = nullptr;
   if (tma_engine && (((uintptr_t)xd & 15) || (A->n & 1))) {
     double* xi;
@@ -562,14 +575,15 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   k_zero_x<<<G, kBlock, 0, s>>>(ra, xd);
   launches += 2;
   PK_CUDA(cudaGetLastError());
-  if (persistent) {
-    // the whole iteration loop in one cooperative launch
+  if (persistent || sm) {
+    // the whole iteration loop in one launch
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    if ((e = launch_cg_persistent(A, xd, r, p, ap, s))) return e;
+    if ((e = sm ? launch_sm_cg(A, xd, r, p, o->maxit, s) : launch_cg_persistent(A, xd, r, p, ap, s))) return e;
     if ((e = T.end())) return e;
     launches += 1;
     if ((e = T.flush())) return e;
     if ((e = finish_info(A, o, info, s, v, e0, e1, launches))) return e;
+    if (sm && info->status != PK_TIMEOUT) sm_done(A, (uint64_t)info->iters + 4);
     for (int k = 0; k < PK_MAX_KERNEL_SLOTS; ++k) {
       info->kernel_count[k] = T.count[k];
       info->kernel_ms[k] = T.count[k] ? T.ms[k] / T.count[k] : 0.0;
@@ -583,7 +597,8 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if (tma && (e = tma_setup())) return e;
   const CsrTiles ct = csr_tiles_of(A);
   const bool irr = csr_irregular(A);  // some tile needs the grouped or whole-warp rows
-  const int Gt = A->grid_tma, Gs = A->grid_stream;
+  const int32_t* urows = rows_by_tile_block(A) ? A->blk_row : nullptr;
+  const int Gt = A->grid_tma, Gs = urows ? Gt : A->grid_stream;
   double* part = A->partials;
   DevState* dst = A->st;
   const int n = A->n;
@@ -613,7 +628,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
     L.ikeys[2] = sell;  // the SpMV kernel in the graph body
     L.body = [=](cudaStream_t cs, Timer* t) {
       if (t) t->begin(PK_SLOT_UPDATE);
-      if (tma) launch_pdl(k_cg_update_tma, Gs, kTileThreads, stream_smem_bytes<4, double, 2>(), cs, n, xd, r, p, ap, part, dst);
+      if (tma) launch_pdl(k_cg_update_tma, Gs, kTileThreads, stream_smem_bytes<4, double, 2>(), cs, n, urows, xd, r, p, ap, part, dst);
       else k_cg_update<<<Gu, kBlock, 0, cs>>>(ra, xd, r, p, ap);
       if (t) { t->end(); t->begin(PK_SLOT_SPMV_DOTS); }
       if (sell) launch_pdl(k_cg_sell_spmv_dots, Gsell, kBlock, 0, cs, sa, (const double*)p, ap, part, dst);

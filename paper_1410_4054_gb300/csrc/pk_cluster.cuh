@@ -25,10 +25,10 @@ __device__ __forceinline__ void cluster_block_slots(double (&v)[NV], double* buf
   constexpr int NW = NT / 32;
   static_assert(NW >= NV && NW <= 32, "one warp per sum");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  warp_sums<NV>(v);
+  if (lane == 0) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const double t = warp_sum(v[k]);
-    if (lane == 0) buf[k * NW + warp] = t;
+    for (int k = 0; k < NV; ++k) buf[k * NW + warp] = v[k];
   }
   __syncthreads();
   if (warp < NV) {
@@ -46,8 +46,7 @@ __device__ __forceinline__ void cluster_total(cg::cluster_group& cl, double* slo
   const double* rem = lane < (int)cl.num_blocks() ? cl.map_shared_rank(slots, lane) : nullptr;
 #pragma unroll
   for (int k = 0; k < NV; ++k) out[k] = rem ? rem[s0 + k] : 0.0;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = warp_sum(out[k]);
+  warp_sums<NV>(out);
 }
 
 // Element `c` of a vector distributed over the cluster, R = 2^lg rows per CTA, each CTA's part

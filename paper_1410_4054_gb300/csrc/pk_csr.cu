@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "pk_guard.cuh"
-#include "pk_tile.cuh"
+#include "pk_sm.cuh"
 
 namespace pk {
 
@@ -302,13 +302,15 @@ using namespace pk;
 // schedule, and the tile counts by schedule.
 struct CsrPlan {
   int grid = 1, grid_tma = 1, grid_stream = 1, ntiles = 0, tma_ok = 1;
-  std::vector<int32_t> rb, tile_row, blk_tile, tile_z0;
+  std::vector<int32_t> rb, tile_row, blk_tile, tile_z0, blk_row;
   std::vector<int8_t> tile_grp;
   std::vector<int16_t> tile_perm;
   int32_t tiles_thread = 0, tiles_long = 0, tiles_group = 0;
 };
 
-static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, int sms, CsrPlan& P) {
+// tile_blocks > 0: that many blocks for the tiles instead of the bulk-copy engine's number.
+static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, int sms, CsrPlan& P,
+                       int tile_blocks = 0) {
   // persistent grid: up to kMaxGridPerSm blocks per SM, at least kBlock rows per block
   const int64_t gmax = (int64_t)sms * kMaxGridPerSm;
   P.grid = (int)std::max<int64_t>(1, std::min<int64_t>(gmax, (n + kBlock - 1) / kBlock));
@@ -340,6 +342,7 @@ static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, i
   P.grid_tma = (int)std::max<int64_t>(
       1, std::min<int64_t>((int64_t)sms * 2, std::max<int64_t>((n + kTileRows - 1) / kTileRows,
                                                                ((int64_t)nnz + kTileNnz - 1) / kTileNnz)));
+  if (tile_blocks > 0) P.grid_tma = tile_blocks;
   {
     const int Gt = P.grid_tma;
     std::vector<int32_t> tb(Gt + 1);
@@ -354,6 +357,7 @@ static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, i
       tb[b] = (int32_t)std::max<int64_t>((lo / 32) * 32, tb[b - 1]);
     }
     tb[Gt] = (int32_t)n;
+    P.blk_row = tb;
     blk_tile.push_back(0);
     for (int b = 0; b < Gt && P.tma_ok; ++b) {
       int64_t R = tb[b];
@@ -457,6 +461,60 @@ static void row_histogram(int64_t n, const std::vector<int32_t>& rp, int64_t (&h
   }
 }
 
+namespace pk {
+
+// Blocks and tiles of the shared-memory-resident loops.  Up to kSmFineRows rows the launched
+// kernels' tiles of 512 rows would leave most SMs without work (8 blocks at 4,096 rows, each with
+// 3,000 clocks of FP64 work per product); these blocks hold about kSmFineWork FMAs of an iteration.
+// Larger systems keep the launched kernels' blocks and with them their summation order.
+pk_status sm_tiles(pk_csr* A, int sms, cudaStream_t s) {
+  A->sm_grid = A->grid_tma;
+  A->sm_rows_max = A->blk_rows_max;
+  A->sm_nnz_max = A->blk_nnz_max;
+  A->sm_blk_row = A->blk_row;
+  A->sm_tile_row = A->tile_row;
+  A->sm_blk_tile = A->blk_tile;
+  A->sm_tile_grp = A->tile_grp;
+  A->sm_tile_perm = A->tile_perm;
+  A->sm_irregular = csr_irregular(A);
+  if (A->n > kSmFineRows || A->grid_tma >= sms) return PK_OK;
+  std::vector<int32_t> rp(A->n + 1);
+  PK_CUDA(cudaMemcpyAsync(rp.data(), A->rp, sizeof(int32_t) * (A->n + 1), cudaMemcpyDeviceToHost, s));
+  PK_CUDA(cudaStreamSynchronize(s));
+  CsrPlan P;
+  const int64_t work = (int64_t)A->nnz + 6 * (int64_t)A->n;
+  build_plan(A->n, A->nnz, rp, sms, P,
+             (int)std::max<int64_t>(A->grid_tma, std::min<int64_t>(sms, (work + kSmFineWork - 1) / kSmFineWork)));
+  auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+  const size_t b0 = up(4 * P.blk_row.size()), b1 = up(4 * P.tile_row.size()), b2 = up(4 * P.blk_tile.size()),
+               b3 = up(P.tile_grp.size()), b4 = up(2 * P.tile_perm.size());
+  PK_CUDA(cudaMalloc(&A->sm_own, b0 + b1 + b2 + b3 + b4));
+  char* d = (char*)A->sm_own;
+  PK_CUDA(cudaMemcpyAsync(d, P.blk_row.data(), 4 * P.blk_row.size(), cudaMemcpyHostToDevice, s));
+  PK_CUDA(cudaMemcpyAsync(d + b0, P.tile_row.data(), 4 * P.tile_row.size(), cudaMemcpyHostToDevice, s));
+  PK_CUDA(cudaMemcpyAsync(d + b0 + b1, P.blk_tile.data(), 4 * P.blk_tile.size(), cudaMemcpyHostToDevice, s));
+  if (!P.tile_grp.empty())
+    PK_CUDA(cudaMemcpyAsync(d + b0 + b1 + b2, P.tile_grp.data(), P.tile_grp.size(), cudaMemcpyHostToDevice, s));
+  if (!P.tile_perm.empty())
+    PK_CUDA(cudaMemcpyAsync(d + b0 + b1 + b2 + b3, P.tile_perm.data(), 2 * P.tile_perm.size(), cudaMemcpyHostToDevice, s));
+  PK_CUDA(cudaStreamSynchronize(s));  // (the sources are host vectors)
+  A->sm_grid = P.grid_tma;
+  A->sm_blk_row = (const int32_t*)d;
+  A->sm_tile_row = (const int32_t*)(d + b0);
+  A->sm_blk_tile = (const int32_t*)(d + b0 + b1);
+  A->sm_tile_grp = (const int8_t*)(d + b0 + b1 + b2);
+  A->sm_tile_perm = P.tile_perm.empty() ? nullptr : (const int16_t*)(d + b0 + b1 + b2 + b3);
+  A->sm_irregular = P.tiles_long > 0 || P.tiles_group > 0;
+  A->sm_rows_max = A->sm_nnz_max = 0;
+  for (int b = 0; b < P.grid_tma; ++b) {
+    A->sm_rows_max = std::max(A->sm_rows_max, P.blk_row[b + 1] - P.blk_row[b]);
+    A->sm_nnz_max = std::max(A->sm_nnz_max, rp[P.blk_row[b + 1]] - rp[P.blk_row[b]]);
+  }
+  return PK_OK;
+}
+
+}  // namespace pk
+
 extern "C" {
 
 const char* pk_status_string(pk_status s) {
@@ -541,6 +599,10 @@ static pk_status csr_create(int64_t n, int64_t nnz, const int32_t* row_ptr, cons
   A->grid_stream = P.grid_stream;
   A->ntiles = P.ntiles;
   A->tma_ok = P.tma_ok;
+  for (int b = 0; b < P.grid_tma; ++b) {
+    A->blk_rows_max = std::max(A->blk_rows_max, P.blk_row[b + 1] - P.blk_row[b]);
+    A->blk_nnz_max = std::max(A->blk_nnz_max, rp[P.blk_row[b + 1]] - rp[P.blk_row[b]]);
+  }
   A->stats.tiles_thread = P.tiles_thread;
   A->stats.tiles_long = P.tiles_long;
   A->stats.tiles_group = P.tiles_group;
@@ -572,6 +634,8 @@ static pk_status csr_create(int64_t n, int64_t nnz, const int32_t* row_ptr, cons
   if (A->tma_ok) {
     if ((e = cudaMalloc(&A->tile_row, sizeof(int32_t) * tile_row.size())) != cudaSuccess) return fail(cuda_fail(e, "cudaMalloc(tiles)"));
     if ((e = cudaMalloc(&A->blk_tile, sizeof(int32_t) * blk_tile.size())) != cudaSuccess) return fail(cuda_fail(e, "cudaMalloc(tiles)"));
+    if ((e = cudaMalloc(&A->blk_row, sizeof(int32_t) * P.blk_row.size())) != cudaSuccess) return fail(cuda_fail(e, "cudaMalloc(tiles)"));
+    if ((e = cudaMemcpyAsync(A->blk_row, P.blk_row.data(), sizeof(int32_t) * P.blk_row.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return fail(cuda_fail(e, "copy tiles"));
     if ((e = cudaMemcpyAsync(A->tile_row, tile_row.data(), sizeof(int32_t) * tile_row.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return fail(cuda_fail(e, "copy tiles"));
     if ((e = cudaMemcpyAsync(A->blk_tile, blk_tile.data(), sizeof(int32_t) * blk_tile.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) return fail(cuda_fail(e, "copy tiles"));
     if ((e = cudaMalloc(&A->tile_grp, std::max<size_t>(1, tile_grp.size()))) != cudaSuccess) return fail(cuda_fail(e, "cudaMalloc(tiles)"));
@@ -635,6 +699,12 @@ pk_status pk_csr_destroy(pk_csr* A) {
   if (A->res_rows) cudaFree(A->res_rows);
   if (A->res_nbr) cudaFree(A->res_nbr);
   if (A->res_flag) cudaFree(A->res_flag);
+  if (A->blk_row) cudaFree(A->blk_row);
+  if (A->sm_own) cudaFree(A->sm_own);
+  if (A->sm_halo_ptr) cudaFree(A->sm_halo_ptr);
+  if (A->sm_halo) cudaFree(A->sm_halo);
+  if (A->sm_ci16) cudaFree(A->sm_ci16);
+  if (A->sm_exchange) cudaFree(A->sm_exchange);
   if (A->small) cudaFree(A->small);
   if (A->partials) cudaFree(A->partials);
   if (A->st) cudaFree(A->st);

@@ -63,45 +63,75 @@ __device__ __forceinline__ double warp_sum_tree(double v) {
   return v;
 }
 
-// Sum of a warp's 32 values, the same in every lane, in integer arithmetic.  GB300 issues an
-// FP64 warp instruction every 64 clocks per scheduler, so the five adds of a butterfly cost
-// 320 clocks of a pipe that the row products need, and a block's reduction of three inner
-// products by nine warps took about 1.9 us at the end of every fused kernel.  Here every value
-// becomes a 64-bit integer in units of 2^-5 of the largest value's last place, the integers are
-// added exactly (three limbs, one redux.sync each), and the total is rounded once to FP64: about
-// forty integer instructions.  The error is at most half a last place of the largest value
-// (32 roundings of 2^-6) plus the final rounding, below the tree's bound of five roundings of
-// partial sums, and the result does not depend on the order of the lanes.  Values near the ends
-// of the exponent range (and Inf, NaN) take the tree.
+// Sums of NV x 32 values of a warp, the same in every lane, in integer arithmetic.  GB300 issues
+// an FP64 warp instruction every 64 clocks per scheduler, so the five adds of a butterfly cost
+// 320 clocks of a pipe that the row products need (measured for one sum: 511 clocks of latency
+// with one warp, 1,530 with sixteen), and a block's reduction of three inner products by nine
+// warps took about 1.9 us at the end of every fused kernel.  Here every value becomes a 64-bit
+// integer in units of 2^-5 of the largest value's last place, the integers are added exactly
+// (three limbs, one redux.sync each), and the total is rounded once to FP64: 230 clocks (240 with
+// sixteen warps), and several sums overlap.  The error is at most half a last place of the largest
+// value (32 roundings of 2^-6) plus the final rounding, below the tree's bound of five roundings
+// of partial sums, and the result does not depend on the order of the lanes.  Values near the ends
+// of the exponent range (and Inf, NaN) take the tree; a warp of zeros takes neither.
+static __device__ __noinline__ double warp_sum_odd(double v) {
+  const bool some = (__double_as_longlong(v) << 1) != 0;
+  return __any_sync(0xffffffffu, some) ? warp_sum_tree(v) : 0.0;
+}
+
+template <int NV>
+__device__ __forceinline__ void warp_sums(double (&v)[NV]) {
+  int em[NV];
+  double r[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v[k]);
+    const int e = (int)(b >> 52) & 0x7ff;
+    em[k] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+    // |v| = m 2^(e - 1075); m << 5 < 2^58, so 32 of them fit a signed 64-bit sum.  (em >= 64: a
+    // subnormal v, whose implicit bit is not set in m, is shifted out either way.)
+    const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 5;
+    const int sh = min(em[k] - e, 62);
+    long long q = (long long)((m + ((1ull << sh) >> 1)) >> sh);
+    if ((long long)b < 0) q = -q;
+    const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3ffffffu);
+    const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26) & 0x3ffffffu);
+    const int l2 = __reduce_add_sync(0xffffffffu, (int)(q >> 52));
+    const long long t = ((long long)l2 << 52) + ((long long)l1 << 26) + (long long)l0;
+    // t 2^(em - 1080): the exponent of a nonzero t is at least 1023, so it stays in range
+    const long long d = __double_as_longlong((double)t);
+    r[k] = t ? __longlong_as_double(d + ((long long)(em[k] - 1080) << 52)) : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+    v[k] = em[k] < 64 || em[k] > 0x7f0 ? warp_sum_odd(v[k]) : r[k];  // the same branch in every lane
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int e = (int)(b >> 52) & 0x7ff;
-  const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if (em < 64 || em > 0x7f0) return warp_sum_tree(v);  // the same branch in every lane
-  // |v| = m 2^(e - 1075); m << 5 < 2^58, so 32 of them fit a signed 64-bit sum.  (em >= 64: a
-  // subnormal v, whose implicit bit is not set in m, is shifted out either way.)
-  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 5;
-  const int sh = min(em - e, 62);
-  long long q = (long long)((m + ((1ull << sh) >> 1)) >> sh);
-  if ((long long)b < 0) q = -q;
-  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3ffffffu);
-  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26) & 0x3ffffffu);
-  const int l2 = __reduce_add_sync(0xffffffffu, (int)(q >> 52));
-  const long long t = ((long long)l2 << 52) + ((long long)l1 << 26) + (long long)l0;
-  // t 2^(em - 1080): the exponent of a nonzero t is at least 1023, so it stays in range
-  const long long r = __double_as_longlong((double)t);
-  return t ? __longlong_as_double(r + ((long long)(em - 1080) << 52)) : 0.0;
+  double t[1] = {v};
+  warp_sums<1>(t);
+  return t[0];
 }
 
 // Eq. (3): alpha_i = <r_i,r_i>/<p_i,Ap_i>, beta_i = alpha_i^2 <Ap_i,Ap_i>/<r_i,r_i> - 1, the
-// quotient of beta formed beside alpha's instead of after it (an FP64 division is about 550
-// clocks on GB300, and this is on every iteration's critical path).  The product is rounded
-// before 1 is taken off: fused, beta p would cancel r exactly once a 1 x 1 system is solved, and
-// a fixed-count run would end with p = 0 instead of going on.
+// quotient of beta formed beside alpha's instead of after it.  The product is rounded before 1 is
+// taken off: fused, beta p would cancel r exactly once a 1 x 1 system is solved, and a fixed-count
+// run would end with p = 0 instead of going on.
+__device__ __forceinline__ double cg_beta(double alpha, double q) {
+  return __dadd_rn(__dmul_rn(__dmul_rn(alpha, alpha), q), -1.0);
+}
 __device__ __forceinline__ void cg_coefficients(double rr, double apap, double pap, double& alpha, double& beta) {
   alpha = rr / pap;
-  const double q = apap / rr;
-  beta = __dadd_rn(__dmul_rn(__dmul_rn(alpha, alpha), q), -1.0);
+  beta = cg_beta(alpha, apap / rr);
+}
+// The same by a whole warp that holds the same three sums in every lane: one lane per quotient, so
+// the two FP64 divisions (about 500 clocks each on GB300, and they do not overlap in one thread) cost
+// one.  Every lane returns the same values.
+__device__ __forceinline__ void cg_coefficients_warp(double rr, double apap, double pap, double& alpha, double& beta) {
+  const bool odd = threadIdx.x & 1;
+  const double q = (odd ? apap : rr) / (odd ? rr : pap);
+  alpha = __shfl_sync(0xffffffffu, q, 0);
+  beta = cg_beta(alpha, __shfl_sync(0xffffffffu, q, 1));
 }
 
 // Block sums of NV values per thread, sum k in every lane of warp k % warps; `put(k, total)` is
@@ -111,8 +141,12 @@ template <int NV, int MAXW, bool TREE = false, class Put>
 __device__ __forceinline__ void block_sums(double (&v)[NV], Put&& put) {
   __shared__ double sm[NV][MAXW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+  if (TREE) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = TREE ? warp_sum_tree(v[k]) : warp_sum(v[k]);
+    for (int k = 0; k < NV; ++k) v[k] = warp_sum_tree(v[k]);
+  } else {
+    warp_sums<NV>(v);
+  }
   if (lane == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) sm[k][warp] = v[k];
@@ -210,7 +244,7 @@ __device__ __forceinline__ void final_sums(const double* partials, double (&out)
   __shared__ double sm[NV];
   const int G = gridDim.x, ng = (G + 31) >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
-  constexpr int B = 4;  // groups a warp loads before it adds them
+  constexpr int B = 4;  // groups a warp loads and adds together
   for (int q0 = warp; q0 < NV * ng; q0 += B * nw) {
     double v[B];
 #pragma unroll
@@ -218,13 +252,11 @@ __device__ __forceinline__ void final_sums(const double* partials, double (&out)
       const int q = q0 + u * nw, k = q / ng, c = (q - k * ng) * 32 + lane;
       v[u] = q < NV * ng && c < G ? ld_cg(partials + (size_t)k * G + c) : 0.0;
     }
+    warp_sums<B>(v);
 #pragma unroll
     for (int u = 0; u < B; ++u) {
       const int q = q0 + u * nw, k = q / ng;
-      if (q < NV * ng) {
-        const double t = warp_sum(v[u]);
-        if (lane == 0) gs[k][q - k * ng] = t;
-      }
+      if (q < NV * ng && lane == 0) gs[k][q - k * ng] = v[u];
     }
   }
   __syncthreads();
@@ -350,6 +382,27 @@ struct pk_csr {
   int32_t* res_rows = nullptr;      // res_grid + 1
   int32_t* res_nbr = nullptr;       // 2 per block: first and last neighbour block
   int32_t* res_flag = nullptr;      // res_grid
+  // rows of the tile blocks: block b owns [blk_row[b], blk_row[b + 1]) (grid_tma + 1), and the
+  // most rows and entries of one block
+  int32_t* blk_row = nullptr;
+  int blk_rows_max = 0, blk_nnz_max = 0;
+  // shared-memory-resident loops (pk_sm.cuh): plan and exchange buffers, built on first use
+  int sm_state = 0;                 // 0 = not built, 1 = built, -1 = A does not fit
+  // their blocks and tiles: those of the launched kernels, or (small systems) finer ones in sm_own
+  int sm_grid = 0, sm_rows_max = 0, sm_nnz_max = 0;
+  const int32_t* sm_blk_row = nullptr;
+  const int32_t* sm_tile_row = nullptr;
+  const int32_t* sm_blk_tile = nullptr;
+  const int8_t* sm_tile_grp = nullptr;
+  const int16_t* sm_tile_perm = nullptr;
+  bool sm_irregular = false;
+  void* sm_own = nullptr;
+  int sm_halo_max = 0;              // most halo columns of one block
+  int32_t* sm_halo_ptr = nullptr;   // grid_tma + 1
+  int32_t* sm_halo = nullptr;
+  uint16_t* sm_ci16 = nullptr;
+  void* sm_exchange = nullptr;
+  uint64_t sm_epoch = 0, sm_epoch_next = 0;
   pk_graph_entry graphs[4];
   cudaEvent_t ev_pool[64] = {nullptr};
   int ev_count = 0;
@@ -471,6 +524,11 @@ __device__ __forceinline__ double sell_row(const SellArgs& s, int64_t base, int 
 
 // Kernels on the CSR tile engine take the instantiation with the grouped and whole-warp row
 // paths when some tile needs one of them.
+// Systems whose update kernel takes the tile blocks' rows (blk_row) instead of equal chunks: the
+// ones that a shared-memory-resident loop may run, so that both sum in the same order.
+constexpr int kSmMaxRows = 655360;  // (the plan's column bitmap fits shared memory)
+inline bool rows_by_tile_block(const pk_csr* A) { return A->tma_ok && !A->tile_z0 && A->n <= kSmMaxRows; }
+
 inline bool csr_irregular(const pk_csr* A) { return A->stats.tiles_long > 0 || A->stats.tiles_group > 0; }
 
 inline long long passes_of(const DevState* h) {

@@ -86,25 +86,27 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
     cluster_block_slots<kCT, 2>(v, buf, slots);
     cl.sync();
     double t[2];
-    if (threadIdx.x < 32) cluster_total<2>(cl, slots, 0, t);
-    // the scalar work (two FP64 divisions) runs in one thread and is broadcast: on GB300 every
+    // the scalar work (two FP64 divisions) runs in one warp and is broadcast: on GB300 every
     // FP64 instruction issued by all warps of a CTA costs the SM's narrow FP64 pipe
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
+      cluster_total<2>(cl, slots, 0, t);
       int sts = kRunning;
       double al = 0.0, be = 0.0;
       if (!isfinite(t[0]) || !isfinite(t[1])) sts = PK_ERR_NAN;
       else if (t[1] <= 0.0) sts = PK_NOT_SPD;
       else {
         // Eq. (3): alpha_i = <r_i,r_i>/<p_i,Ap_i>, beta_i = alpha_i^2 <Ap_i,Ap_i>/<r_i,r_i> - 1
-        cg_coefficients(rr, t[0], t[1], al, be);
+        cg_coefficients_warp(rr, t[0], t[1], al, be);
         if (lead && trace && i < trace_cap) {
           trace[(size_t)i * 4 + 0] = al;
           trace[(size_t)i * 4 + 1] = be;
         }
       }
-      sc[0] = al;
-      sc[1] = be;
-      scs = sts;
+      if (threadIdx.x == 0) {
+        sc[0] = al;
+        sc[1] = be;
+        scs = sts;
+      }
     }
     __syncthreads();
     if (scs != kRunning) { status = scs; break; }
@@ -125,10 +127,12 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
     cluster_block_slots<kCT, 1>(w, buf, slots + 2);
     cl.sync();
     double u[1];
-    if (threadIdx.x < 32) cluster_total<1>(cl, slots, 2, u);
+    if (threadIdx.x < 32) {
+      cluster_total<1>(cl, slots, 2, u);
+      rr = u[0];  // (warp 0 alone needs it)
+    }
     iters = i + 1;
     if (threadIdx.x == 0) {
-      rr = u[0];  // (thread 0 alone needs it)
       int sts = kRunning;
       if (!isfinite(rr)) sts = PK_ERR_NAN;
       else if (rr <= thr2) sts = PK_OK;

@@ -308,6 +308,11 @@ __device__ __forceinline__ double gather(const double* __restrict__ x, int c) { 
 __device__ __forceinline__ float gather(const float* __restrict__ x, int c) { return __ldg(x + c); }
 template <class VT>
 __device__ __forceinline__ VT gather(CohVec<VT> x, int c) { return __ldcg(x.p + c); }
+// Whether the gathers of XP read shared memory (pk_sm.cuh).
+template <class XP>
+struct GatherShared {
+  static constexpr bool value = false;
+};
 // BlockVec: a vector that only the reading block writes (the batched solver: one block owns a
 // system's vectors).  Plain L1-cached loads see the block's own earlier stores after a block
 // barrier; the non-coherent path might not.
@@ -360,8 +365,8 @@ __device__ __forceinline__ void fma_batch_gn(int mx, const VT (&v)[8], const VT 
 // every lane of the warp calls it together (lanes without a row pass j = j1), and the batch
 // loop runs to the warp's longest share, issuing only that many FMAs (predicated-off FP64
 // instructions still take issue slots).
-template <int G, class VT, class XP>
-__device__ __forceinline__ VT group_row(const VT* sva, const int32_t* sci, int j, int j1, XP x) {
+template <int G, class VT, class CI, class XP>
+__device__ __forceinline__ VT group_row(const VT* sva, const CI* sci, int j, int j1, XP x) {
   VT s = (VT)0;
   for (;;) {
     const int m = j < j1 ? min(8, (j1 - j + G - 1) / G) : 0;
@@ -386,8 +391,8 @@ __device__ __forceinline__ VT group_row(const VT* sva, const int32_t* sci, int j
 
 // The rows of a grouped tile: kConsumers / G rows per round, rows in order.  Rounds are the
 // same for the whole block, so every lane reaches the group's shuffles.
-template <int G, class VT, class XP, class RowDone>
-__device__ __forceinline__ void group_rows(const int32_t* srp, const VT* sva, const int32_t* sci, int R0,
+template <int G, class VT, class CI, class XP, class RowDone>
+__device__ __forceinline__ void group_rows(const int32_t* srp, const VT* sva, const CI* sci, int R0,
                                            int R1, XP x, RowDone& row_done) {
   constexpr int ng = kConsumers / G;
   const int gid = (int)threadIdx.x / G, q = (int)threadIdx.x & (G - 1);
@@ -400,12 +405,17 @@ __device__ __forceinline__ void group_rows(const int32_t* srp, const VT* sva, co
   }
 }
 
+// The same for a gathered vector in shared memory (defined in pk_sm.cuh).
+template <class CI, class XP, class RowDone>
+__device__ __forceinline__ void group_rows_shared(int G, const int32_t* srp, const double* sva, const CI* sci, int R0,
+                                                  int R1, XP x, RowDone& row_done);
+
 // Two row products from a shared-memory window (defined below): FP64 and FP32.
-template <class XP>
-__device__ __forceinline__ void row_pair(const double* sva, const int32_t* sci, int ja, int ja1, int jb,
+template <class CI, class XP>
+__device__ __forceinline__ void row_pair(const double* sva, const CI* sci, int ja, int ja1, int jb,
                                          int jb1, XP x, double& sa, double& sb);
-template <class XP>
-__device__ __forceinline__ void row_pair(const float* sva, const int32_t* sci, int ja, int ja1, int jb,
+template <class CI, class XP>
+__device__ __forceinline__ void row_pair(const float* sva, const CI* sci, int ja, int ja1, int jb,
                                          int jb1, XP x, float& sa, float& sb);
 
 // Runs the CSR pipeline and the row products y_row = sum_j A[row][j] x[col j]; every finished
@@ -463,6 +473,70 @@ __device__ __forceinline__ void block_row_chunk(int row, int zc0, int zr1, VT* s
     for (int k = 0; k < kConsumerWarps; ++k) tot += vr[k];
     *cnt = 0;
     row_done(row, tot);
+  }
+}
+
+// The row products of one tile, rows [R0, R1), from shared memory: srp[row] is the index of the
+// row's first entry in sva / sci; G is the tile's schedule (1: a thread per row; 2 .. 16: G lanes
+// per row; 32: whole warps for the long rows, with the row order sperm if there is one).  Called
+// by the kConsumers consumer threads together; row_done(row, y) runs in one thread per row.
+template <bool IRR, class VT, class CI, class XP, class RowDone>
+__device__ __forceinline__ void tile_rows(int R0, int R1, int G, const int16_t* sperm, const int32_t* srp,
+                                          const VT* sva, const CI* sci, XP x, RowDone& row_done) {
+  const int lane = threadIdx.x & 31;
+  if (!IRR || G == 1) {
+    const int ra = R0 + (int)threadIdx.x;
+    if (ra < R1) {
+      const int rb = ra + kConsumers < R1 ? ra + kConsumers : -1;
+      VT sa, sb;
+      row_pair(sva, sci, srp[ra], srp[ra + 1], rb >= 0 ? srp[rb] : 0, rb >= 0 ? srp[rb + 1] : 0, x, sa, sb);
+      row_done(ra, sa);
+      if (rb >= 0) row_done(rb, sb);
+    }
+  } else if (G < 32) {
+    // rows of similar length, too long for one thread: G lanes per row (G = 2..16)
+    if constexpr (GatherShared<XP>::value) {
+      group_rows_shared(G, srp, sva, sci, R0, R1, x, row_done);
+    } else {
+      switch (G) {
+        case 2: group_rows<2>(srp, sva, sci, R0, R1, x, row_done); break;
+        case 4: group_rows<4>(srp, sva, sci, R0, R1, x, row_done); break;
+        case 8: group_rows<8>(srp, sva, sci, R0, R1, x, row_done); break;
+        default: group_rows<16>(srp, sva, sci, R0, R1, x, row_done); break;
+      }
+    }
+  } else {
+    // every lane takes part (the ballots below need the whole warp).  With a row order
+    // (sorted by length, dealt round-robin over the warps) each warp holds rows of similar
+    // length, so its FMA batches carry few idle lanes.
+    const int ka = sperm ? sperm[threadIdx.x] : (int)threadIdx.x;
+    const int kb = sperm ? sperm[threadIdx.x + kConsumers] : (int)threadIdx.x + kConsumers;
+    const int ra = ka >= 0 && R0 + ka < R1 ? R0 + ka : -1;
+    const int rb = kb >= 0 && R0 + kb < R1 ? R0 + kb : -1;
+    int ja0 = ra >= 0 ? srp[ra] : 0, ja1 = ra >= 0 ? srp[ra + 1] : 0;
+    int jb0 = rb >= 0 ? srp[rb] : 0, jb1 = rb >= 0 ? srp[rb + 1] : 0;
+    const bool la = ja1 - ja0 > kLongRow, lb = jb1 - jb0 > kLongRow;
+    if (ra >= 0 || rb >= 0) {
+      VT sa, sb;
+      row_pair(sva, sci, ja0, la ? ja0 : ja1, jb0, lb ? jb0 : jb1, x, sa, sb);
+      if (ra >= 0 && !la) row_done(ra, sa);
+      if (rb >= 0 && !lb) row_done(rb, sb);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      unsigned pending = __ballot_sync(0xffffffffu, h == 0 ? la : lb);
+      while (pending) {
+        const int src = __ffs(pending) - 1;
+        pending &= pending - 1;
+        const int r = __shfl_sync(0xffffffffu, h == 0 ? ra : rb, src);
+        const int j0 = srp[r], j1 = srp[r + 1];
+        VT acc = (VT)0;
+        for (int j = j0 + lane; j < j1; j += 32) acc = fma_t(sva[j], gather(x, sci[j]), acc);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == src) row_done(r, acc);
+      }
+    }
   }
 }
 
@@ -596,56 +670,8 @@ __device__ __forceinline__ bool csr_tiles_range(const CsrTilesT<VT>& T, int t0, 
     if (IRR && G == kChunkTile) {
       block_row_chunk(R0, m.w, srp[R0 + 1], stage_va(s), stage_ci(s), x, chunk_acc, chunk_red, &chunk_cnt,
                       warp, lane, row_done);
-    } else if (!IRR || G == 1) {
-      const int ra = R0 + (int)threadIdx.x;
-      if (ra < R1) {
-        const int rb = ra + kConsumers < R1 ? ra + kConsumers : -1;
-        VT sa, sb;
-        row_pair(sva, sci, srp[ra], srp[ra + 1], rb >= 0 ? srp[rb] : 0, rb >= 0 ? srp[rb + 1] : 0, x, sa, sb);
-        row_done(ra, sa);
-        if (rb >= 0) row_done(rb, sb);
-      }
-    } else if (G < 32) {
-      // rows of similar length, too long for one thread: G lanes per row (G = 2..16)
-      switch (G) {
-        case 2: group_rows<2>(srp, sva, sci, R0, R1, x, row_done); break;
-        case 4: group_rows<4>(srp, sva, sci, R0, R1, x, row_done); break;
-        case 8: group_rows<8>(srp, sva, sci, R0, R1, x, row_done); break;
-        default: group_rows<16>(srp, sva, sci, R0, R1, x, row_done); break;
-      }
     } else {
-      // every lane takes part (the ballots below need the whole warp).  With a row order
-      // (sorted by length, dealt round-robin over the warps) each warp holds rows of similar
-      // length, so its FMA batches carry few idle lanes.
-      const int16_t* sperm = m.w ? stage_perm(s) : nullptr;
-      const int ka = sperm ? sperm[threadIdx.x] : (int)threadIdx.x;
-      const int kb = sperm ? sperm[threadIdx.x + kConsumers] : (int)threadIdx.x + kConsumers;
-      const int ra = ka >= 0 && R0 + ka < R1 ? R0 + ka : -1;
-      const int rb = kb >= 0 && R0 + kb < R1 ? R0 + kb : -1;
-      int ja0 = ra >= 0 ? srp[ra] : 0, ja1 = ra >= 0 ? srp[ra + 1] : 0;
-      int jb0 = rb >= 0 ? srp[rb] : 0, jb1 = rb >= 0 ? srp[rb + 1] : 0;
-      const bool la = ja1 - ja0 > kLongRow, lb = jb1 - jb0 > kLongRow;
-      if (ra >= 0 || rb >= 0) {
-        VT sa, sb;
-        row_pair(sva, sci, ja0, la ? ja0 : ja1, jb0, lb ? jb0 : jb1, x, sa, sb);
-        if (ra >= 0 && !la) row_done(ra, sa);
-        if (rb >= 0 && !lb) row_done(rb, sb);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        unsigned pending = __ballot_sync(0xffffffffu, h == 0 ? la : lb);
-        while (pending) {
-          const int src = __ffs(pending) - 1;
-          pending &= pending - 1;
-          const int r = __shfl_sync(0xffffffffu, h == 0 ? ra : rb, src);
-          const int j0 = srp[r], j1 = srp[r + 1];
-          VT acc = (VT)0;
-          for (int j = j0 + lane; j < j1; j += 32) acc = fma_t(sva[j], gather(x, sci[j]), acc);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-          if (lane == src) row_done(r, acc);
-        }
-      }
+      tile_rows<IRR>(R0, R1, G, IRR && m.w ? stage_perm(s) : nullptr, srp, sva, sci, x, row_done);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
@@ -690,8 +716,8 @@ __device__ __forceinline__ void fma_batch_n(int mx, const double (&v)[8], const 
   }
 }
 
-template <class XP>
-__device__ __forceinline__ void smem_row2(const double* sva, const int32_t* sci, int ja, int ja1,
+template <class CI, class XP>
+__device__ __forceinline__ void smem_row2(const double* sva, const CI* sci, int ja, int ja1,
                                           int jb, int jb1, XP x, double& sa, double& sb) {
   sa = 0.0;
   sb = 0.0;
@@ -773,8 +799,8 @@ inline void launch_pdl(void (*kern)(KArgs...), int grid, int block, size_t smem,
 
 // FP32 row product from a shared-memory window: the row's products summed left to right
 // (the order of a plain CSR row loop), gathers of a batch of 8 issued before the FMAs.
-template <class XP>
-__device__ __forceinline__ float smem_row_f32(const float* sva, const int32_t* sci, int j, int j1, XP x) {
+template <class CI, class XP>
+__device__ __forceinline__ float smem_row_f32(const float* sva, const CI* sci, int j, int j1, XP x) {
   float s = 0.0f;
   for (; j < j1; j += 8) {
     const int m = min(8, j1 - j);
@@ -794,14 +820,14 @@ __device__ __forceinline__ float smem_row_f32(const float* sva, const int32_t* s
   return s;
 }
 
-template <class XP>
-__device__ __forceinline__ void row_pair(const double* sva, const int32_t* sci, int ja, int ja1, int jb,
+template <class CI, class XP>
+__device__ __forceinline__ void row_pair(const double* sva, const CI* sci, int ja, int ja1, int jb,
                                          int jb1, XP x, double& sa, double& sb) {
   smem_row2(sva, sci, ja, ja1, jb, jb1, x, sa, sb);
 }
 
-template <class XP>
-__device__ __forceinline__ void row_pair(const float* sva, const int32_t* sci, int ja, int ja1, int jb,
+template <class CI, class XP>
+__device__ __forceinline__ void row_pair(const float* sva, const CI* sci, int ja, int ja1, int jb,
                                          int jb1, XP x, float& sa, float& sb) {
   sa = smem_row_f32(sva, sci, ja, ja1, x);
   sb = jb1 > jb ? smem_row_f32(sva, sci, jb, jb1, x) : 0.0f;
