@@ -444,8 +444,9 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
 pk_status launch_cg_persistent(pk_csr* A, double* x, double* r, double* p, double* ap,
                                cudaStream_t s);
 pk_status resident_prepare(pk_csr* A, cudaStream_t s, bool* usable);
-pk_status sm_cg_usable(pk_csr* A, cudaStream_t s, bool* usable);
-pk_status launch_sm_cg(pk_csr* A, double* x, const double* r, const double* p, int maxit, cudaStream_t s);
+pk_status sm_cg_usable(pk_csr* A, bool jac, cudaStream_t s, bool* usable);
+pk_status launch_sm_cg(pk_csr* A, double* x, const double* r, const double* p, const double* dinv, int maxit,
+                       cudaStream_t s);
 pk_status launch_cg_resident(pk_csr* A, double* x, double* r, double* p, double* ap, cudaStream_t s);
 
 pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_info* info,
@@ -489,7 +490,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   SmTurn turn;
   if (o->loop == PK_LOOP_AUTO && !(persistent && cluster_size_work(A)) && !sell &&
       o->variant == PK_VARIANT_PIPELINED && !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
-    if ((e = sm_cg_usable(A, s, &sm))) return e;
+    if ((e = sm_cg_usable(A, false, s, &sm))) return e;
     sm = sm && turn.take();
     if (sm) persistent = false;
   }
@@ -578,7 +579,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if (persistent || sm) {
     // the whole iteration loop in one launch
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    if ((e = sm ? launch_sm_cg(A, xd, r, p, o->maxit, s) : launch_cg_persistent(A, xd, r, p, ap, s))) return e;
+    if ((e = sm ? launch_sm_cg(A, xd, r, p, nullptr, o->maxit, s) : launch_cg_persistent(A, xd, r, p, ap, s))) return e;
     if ((e = T.end())) return e;
     launches += 1;
     if ((e = T.flush())) return e;

@@ -33,7 +33,7 @@
 #include <vector>
 
 #include "pk_guard.cuh"
-#include "pk_tile.cuh"
+#include "pk_sm.cuh"
 
 namespace pk {
 
@@ -781,6 +781,11 @@ static pk_status gm_setup() {
 bool gmres_persistent_usable(const pk_csr* A, int m);
 pk_status launch_gmres_persistent(pk_csr* A, const double* b, double* x, int m, double* V, int64_t ld,
                                   double* Rout, double* xiout, cudaStream_t s);
+// pk_sm_gmres.cu: the loop with the matrix in shared memory
+pk_status sm_gmres_usable(pk_csr* A, cudaStream_t s, bool* usable);
+uint64_t sm_gmres_epochs(uint64_t iters, uint64_t cycles);
+pk_status launch_sm_gmres(pk_csr* A, const double* b, const double* r, double* x, int m, double* V, int64_t ld,
+                          double* Rout, double* xiout, int maxit, cudaStream_t s);
 
 pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_info* info,
                       cudaStream_t s) {
@@ -824,6 +829,16 @@ pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, p
     persistent = plain && A->n <= PK_PERSISTENT_GMRES_AUTO_N && A->nnz <= PK_PERSISTENT_GMRES_AUTO_NNZ &&
                  A->stats.tiles_long == 0 && !(o->flags & PK_FLAG_TIMING) && gmres_persistent_usable(A, m);
   }
+  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
+  // other host thread's is running
+  bool sm = false;
+  SmTurn turn;
+  if (o->loop == PK_LOOP_AUTO && plain && !(persistent && cluster_size_work(A)) &&
+      !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
+    if ((e = sm_gmres_usable(A, s, &sm))) return e;
+    sm = sm && turn.take();
+    if (sm) persistent = false;
+  }
   if (!A->tma_ok && !persistent) { set_error("GMRES needs the tile engine"); return PK_ERR_ARG; }
   if ((e = gm_setup())) return e;
   const int n = A->n;
@@ -847,16 +862,25 @@ pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, p
   // right Jacobi preconditioning: iterate on A M^-1 with y = M x (values swapped until leave)
   JacobiRight jac;
   if (o->precond == PK_PRECOND_JACOBI && (e = jacobi_right_enter(A, v.x_dev, s, &jac))) return e;
-  if (persistent) {
+  if (persistent || sm) {
     Timer T;
     T.A = A;
     T.on = (o->flags & PK_FLAG_TIMING) != 0;
     T.s = s;
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    if ((e = launch_gmres_persistent(A, v.b_dev, v.x_dev, m, A->basis, ld, A->small, A->small + kXiOff, s))) return e;
+    int launches = 3;  // state, the loop, the b = 0 case
+    if (sm) {
+      double* r;
+      if ((e = work_vec(A, 0, &r))) return e;
+      launch_residual_init(A, v.b_dev, v.x_dev, r, nullptr, nullptr, s);
+      e = launch_sm_gmres(A, v.b_dev, r, v.x_dev, m, A->basis, ld, A->small, A->small + kXiOff, o->maxit, s);
+      launches += 2;  // the setup kernel, r_0 to the exchange
+    } else {
+      e = launch_gmres_persistent(A, v.b_dev, v.x_dev, m, A->basis, ld, A->small, A->small + kXiOff, s);
+    }
+    if (e) return e;
     if ((e = T.end())) return e;
     launch_zero_x(A, v.x_dev, s);
-    int launches = 3;  // state, the loop, the b = 0 case
     if ((e = T.flush())) return e;
     if (jac.A) {
       if ((e = jacobi_right_leave(&jac, v.x_dev, s))) return e;
@@ -864,6 +888,7 @@ pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, p
     }
     if ((e = finish_info(A, o, info, s, v, e0, e1, launches))) return e;
     info->cycles = A->st_host->gm_cycle;
+    if (sm && info->status != PK_TIMEOUT) sm_done(A, sm_gmres_epochs(info->iters, info->cycles + 2));
     for (int k = 0; k < PK_MAX_KERNEL_SLOTS; ++k) {
       info->kernel_count[k] = T.count[k];
       info->kernel_ms[k] = T.count[k] ? T.ms[k] / T.count[k] : 0.0;

@@ -10,7 +10,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "pk_tile.cuh"
+#include "pk_sm.cuh"
 
 namespace pk {
 
@@ -202,6 +202,11 @@ pk_status pcg_setup() {
 
 }  // namespace
 
+// pk_sm_cg.cu: the loop with the matrix in shared memory
+pk_status sm_cg_usable(pk_csr* A, bool jac, cudaStream_t s, bool* usable);
+pk_status launch_sm_cg(pk_csr* A, double* x, const double* r, const double* p, const double* dinv, int maxit,
+                       cudaStream_t s);
+
 pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_info* info,
                            cudaStream_t s) {
   if (o->variant != PK_VARIANT_PIPELINED || o->precision != PK_PREC_FP64 || o->loop == PK_LOOP_PERSISTENT || o->loop == PK_LOOP_RESIDENT) {
@@ -214,6 +219,13 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
   }
   pk_status e;
   if ((e = pcg_setup())) return e;
+  // the shared-memory-resident loop, where the system fits it and no other host thread's is running
+  bool sm = false;
+  SmTurn turn;
+  if (o->loop == PK_LOOP_AUTO && !(o->flags & PK_FLAG_TIMING)) {
+    if ((e = sm_cg_usable(A, true, s, &sm))) return e;
+    sm = sm && turn.take();
+  }
   cudaEvent_t e0, e1;
   PK_CUDA(cudaEventCreate(&e0));
   PK_CUDA(cudaEventCreate(&e1));
@@ -227,7 +239,7 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
     return e;
   double* xd = v.x_dev;
   double* x_copy_back = nullptr;  // the bulk-copy kernels read x in 16-byte units
-  if (((uintptr_t)xd & 15) || (A->n & 1)) {
+  if (!sm && (((uintptr_t)xd & 15) || (A->n & 1))) {
     double* xi;
     if ((e = work_vec(A, 13, &xi))) return e;
     PK_CUDA(cudaMemcpyAsync(xi, xd, sizeof(double) * A->n, cudaMemcpyDeviceToDevice, s));
@@ -252,6 +264,15 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
   if ((e = T.end())) return e;
   launch_zero_x(A, xd, s);
   launches += 3;
+  if (sm) {
+    if ((e = launch_sm_cg(A, xd, r, p, dinv, o->maxit, s))) return e;
+    launches += 1;
+    if ((e = finish_info(A, o, info, s, v, e0, e1, launches))) return e;
+    if (info->status != PK_TIMEOUT) sm_done(A, (uint64_t)info->iters + 4);
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    return (pk_status)info->status;
+  }
   // A p0, alpha_0, beta_0
   if ((e = T.begin(PK_SLOT_SPMV_DOTS))) return e;
   (irr ? k_pcg_spmv_dots_tma<true> : k_pcg_spmv_dots_tma<false>)<<<Gt, kTileThreads, csr_smem_bytes(), s>>>(

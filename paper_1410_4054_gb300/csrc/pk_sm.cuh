@@ -33,6 +33,7 @@ constexpr int kSmWords = 4;             // scalars broadcast per reduction
 constexpr int kSmCopies = 16;           // copies of the broadcast (blocks share them out)
 constexpr size_t kSmSlotWords = (size_t)2 * kSmSums * kSmMaxBlocks;
 constexpr size_t kSmBcWords = (size_t)2 * kSmCopies * kSmWords;
+constexpr size_t kSmColWords = (size_t)2 * 65 * (kSmMaxBlocks + 8);
 
 struct SmArgs {
   CsrTiles T;
@@ -43,6 +44,7 @@ struct SmArgs {
   ulonglong2* vex;          // [2][n] published vector
   ulonglong2* slots;        // [2][kSmSums][kSmMaxBlocks]
   ulonglong2* bc;           // [2][kSmCopies][kSmWords]
+  ulonglong2* col;          // GMRES: column sums and their broadcast (kSmColWords)
   int32_t n;
   int32_t max_rows, max_nnz, max_halo;  // shared memory layout
   uint32_t ep0;             // epochs of this launch start above ep0
@@ -143,6 +145,13 @@ __device__ __forceinline__ SmLayout sm_layout(unsigned char* smem, const SmArgs&
   L.rp = reinterpret_cast<int32_t*>(d);
   L.ci = reinterpret_cast<uint16_t*>(L.rp + r + 4);
   return L;
+}
+
+// The last `missing` vectors have no room in shared memory: rp and ci follow the last one that has.
+__device__ __forceinline__ void sm_shorten(SmLayout& L, const SmArgs& a, int missing) {
+  const int skip = missing * sm_even(a.max_rows);
+  L.rp -= 2 * skip;
+  L.ci -= 4 * skip;
 }
 
 struct SmemVec {
@@ -290,9 +299,11 @@ __device__ __forceinline__ void sm_publish(const SmArgs& a, int row, double v, u
   ll_put(a.vex + (size_t)(ep & 1) * a.n + row, v, ep);
 }
 
-// The halo of exchange ep behind the own rows of v; a barrier must follow.  false: gave up (this
-// thread).
-__device__ __forceinline__ bool sm_fetch(const SmArgs& a, const SmBlock& B, double* v_own, uint32_t ep) {
+// The halo of exchange ep behind the own rows of v (SCALE: times `scale`); a barrier must follow.
+// false: gave up (this thread).
+template <bool SCALE = false>
+__device__ __forceinline__ bool sm_fetch(const SmArgs& a, const SmBlock& B, double* v_own, uint32_t ep,
+                                         double scale = 1.0) {
   constexpr int N = 4;
   double* dst = v_own + B.hoff;
   const ulonglong2* src = a.vex + (size_t)(ep & 1) * a.n;
@@ -302,7 +313,7 @@ __device__ __forceinline__ bool sm_fetch(const SmArgs& a, const SmBlock& B, doub
 #pragma unroll
     for (int u = 0; u < N; ++u) c[u] = k0 + u * kSmThreads < B.nh ? __ldg(B.halo + k0 + u * kSmThreads) : 0;
     if (!ll_wait<N>([&](int u) { return src + c[u]; }, min(N, (B.nh - k0 + kSmThreads - 1) / kSmThreads), ep, a.st,
-                    [&](int u, double v) { dst[k0 + u * kSmThreads] = v; }))
+                    [&](int u, double v) { dst[k0 + u * kSmThreads] = SCALE ? v * scale : v; }))
       return false;
   }
   return true;
@@ -412,6 +423,8 @@ pk_status sm_launch(pk_csr* A, Kernel kernel, size_t smem, const SmArgs& a, cons
   PK_CUDA(cudaLaunchKernelEx(&cfg, kernel, a, extra));
   return PK_OK;
 }
+// v as the first exchange of the launch (epoch a.ep0), by a kernel before the loop.
+void launch_sm_publish(const SmArgs& a, const double* v, cudaStream_t s);
 // After the solve: `epochs` were used (0: unknown, the exchange buffers are cleared next time).
 void sm_done(pk_csr* A, uint64_t epochs);
 

@@ -26,23 +26,13 @@ struct SmBi {
   int nvec;    // vectors in shared memory, kSmBiMin .. kSmBiMax
 };
 
-__global__ void __launch_bounds__(kBlock) k_sm_publish(SmArgs a, const double* v) {
-  if (state_done(a.st)) return;
-  for (int row = blockIdx.x * kBlock + threadIdx.x; row < a.n; row += gridDim.x * kBlock) sm_publish(a, row, v[row], a.ep0);
-}
-
 template <bool IRR>
 __global__ void __launch_bounds__(kSmThreads, 2) k_sm_bi(SmArgs a, SmBi g) {
   extern __shared__ __align__(16) unsigned char smem[];
   DevState* st = a.st;
   if (state_done(st)) return;  // decided by the setup kernel, the same for every block
-  // the layout's vectors beyond nvec have no room: rp and ci follow the last one that has
   SmLayout L = sm_layout<kSmBiMax, 1>(smem, a);
-  {
-    const int skip = (kSmBiMax - g.nvec) * sm_even(a.max_rows);
-    L.rp -= 2 * skip;
-    L.ci -= 4 * skip;
-  }
+  sm_shorten(L, a, kSmBiMax - g.nvec);
   const SmBlock B = sm_begin(a, L);
   double *sg = L.vec[0], *sp = L.vec[1], *sr = L.vec[2], *sap = L.vec[3];
   double* as = g.nvec > 4 ? L.vec[4] : g.as + B.r0;
@@ -210,7 +200,7 @@ pk_status launch_sm_bicgstab(pk_csr* A, double* x, const double* r, const double
   if (e) return e;
   size_t smem;
   const int nv = sm_bi_vectors(A, &smem);
-  k_sm_publish<<<(A->n + kBlock - 1) / kBlock, kBlock, 0, s>>>(a, r);
+  launch_sm_publish(a, r, s);
   PK_CUDA(cudaGetLastError());
   return sm_launch(A, A->sm_irregular ? k_sm_bi<true> : k_sm_bi<false>, smem, a, SmBi{x, r, r0s, as, nv}, s);
 }

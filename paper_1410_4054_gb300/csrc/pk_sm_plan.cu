@@ -72,10 +72,16 @@ __global__ void __launch_bounds__(kPlanThreads) k_sm_plan(const int32_t* rp, con
   }
 }
 
+__global__ void __launch_bounds__(kBlock) k_sm_publish(SmArgs a, const double* v) {
+  if (state_done(a.st)) return;
+  const int row = blockIdx.x * kBlock + threadIdx.x;
+  if (row < a.n) sm_publish(a, row, v[row], a.ep0);
+}
+
 std::atomic_flag g_turn = ATOMIC_FLAG_INIT;
 
 size_t exchange_bytes(const pk_csr* A) {
-  return sizeof(ulonglong2) * (2 * (size_t)A->n + kSmSlotWords + kSmBcWords);
+  return sizeof(ulonglong2) * (2 * (size_t)A->n + kSmSlotWords + kSmBcWords + kSmColWords);
 }
 
 pk_status build(pk_csr* A, cudaStream_t s) {
@@ -172,6 +178,7 @@ pk_status sm_args(pk_csr* A, uint64_t epochs, cudaStream_t s, SmArgs* out) {
   a.vex = reinterpret_cast<ulonglong2*>(A->sm_exchange);
   a.slots = a.vex + 2 * (size_t)A->n;
   a.bc = a.slots + kSmSlotWords;
+  a.col = a.bc + kSmBcWords;
   a.n = A->n;
   a.max_rows = A->sm_rows_max;
   a.max_nnz = A->sm_nnz_max;
@@ -182,6 +189,10 @@ pk_status sm_args(pk_csr* A, uint64_t epochs, cudaStream_t s, SmArgs* out) {
   A->sm_epoch_next = A->sm_epoch;
   A->sm_epoch = 0;  // unknown until sm_done
   return PK_OK;
+}
+
+void launch_sm_publish(const SmArgs& a, const double* v, cudaStream_t s) {
+  k_sm_publish<<<(a.n + kBlock - 1) / kBlock, kBlock, 0, s>>>(a, v);
 }
 
 void sm_done(pk_csr* A, uint64_t epochs) { A->sm_epoch = epochs ? A->sm_epoch_next + epochs : 0; }
