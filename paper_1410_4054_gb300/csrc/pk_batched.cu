@@ -596,11 +596,16 @@ static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterP
   return true;
 }
 
+// The class streams and events are shared by every caller: a batch is enqueued under the mutex
+// (stream waits refer to an event's state at the time of the call, so batches of other threads may
+// record the events again as soon as this one is enqueued).
+static std::mutex g_cl_mutex;
 static cudaStream_t g_cl_stream[kClClasses];
 static cudaEvent_t g_cl_fork, g_cl_join[kClClasses];
 
 static pk_status run_clusters(BatchClSys* dsys, const ClusterPlan& P, int* queues, double tol, int maxit,
                               cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(g_cl_mutex);
   static bool init = false;
   if (!init) {
     for (int j = 0; j < kClClasses; ++j) {
@@ -761,11 +766,16 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
   }
   const double mean_len = rows > 0 ? (double)nnz / (double)rows : 0.0;
   const int lanes_auto = mean_len <= 12 ? 1 : mean_len <= 24 ? 2 : mean_len <= 48 ? 4 : 8;
-  // lanes -1: the tile engine; -2: the cluster engine; otherwise the row kernel with the
-  // given (or automatic) lanes
-  TuneVal cfg = o->lanes == -1   ? TuneVal{kTileThreads, 2, -1, 0}
-                : o->lanes == -2 ? TuneVal{kClRowsDefault / 8, 4096 / kClRowsDefault, -2, kClRowsDefault}
-                                 : TuneVal{512, 2, o->lanes ? o->lanes : lanes_auto, 0};
+  // lanes -1: the tile engine; -2: the cluster engine; otherwise the row kernel with the given
+  // lanes.  Automatic: the cluster engine for FP64 batches of rows short enough for one thread each
+  // (512 shifted 2D Laplacians of 1,024 to 65,536 rows to 1e-10 on GB300: 16.9 ms a call, the row kernel at
+  // 512 threads x 2 37.5 ms, tuned 17.5 ms: a large system runs on up to 16 SMs instead of one
+  // block, and its vectors stay in shared memory); longer rows keep the row kernel's lanes.
+  const TuneVal cluster_cfg{kClRowsDefault / 8, 4096 / kClRowsDefault, -2, kClRowsDefault};
+  TuneVal cfg = o->lanes == -1                                          ? TuneVal{kTileThreads, 2, -1, 0}
+                : o->lanes == -2                                        ? cluster_cfg
+                : o->lanes == 0 && clusters_ok && lanes_auto == 1 ? cluster_cfg
+                                                                    : TuneVal{512, 2, o->lanes ? o->lanes : lanes_auto, 0};
   const TuneKey key{nsys, rows, nnz, mixed};
   bool have = false;
   if (o->lanes == 0) {
