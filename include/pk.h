@@ -499,6 +499,14 @@ pk_status pk_adam_step(int64_t count, float* p, const float* grad, float* m, flo
                        float beta1, float beta2, float eps, int32_t step, void* p_bf16,
                        void* stream);
 
+/* pk_adam_step of up to PK_ADAM_MAX_TENSORS tensors in one launch: HOST arrays of counts and device
+ * pointers; p_bf16 (the array or an entry may be NULL) receives the BF16 copies, flipped (the same;
+ * only for tensors of 27 x 16 x 16 weights) the flipped BF16 copies that pk_conv3d_flip makes. */
+#define PK_ADAM_MAX_TENSORS 16
+pk_status pk_adam_step_many(int32_t tensors, const int64_t* counts, float* const* p, const float* const* grad,
+                            float* const* m, float* const* v, void* const* p_bf16, void* const* flipped, float lr,
+                            float beta1, float beta2, float eps, int32_t step, void* stream);
+
 /* Human-readable name of a status code (static string). */
 const char* pk_status_string(pk_status s);
 

@@ -6,13 +6,13 @@
 // zero padding of 1 at the grid boundary.
 //
 // Forward / backward-data (conv3d_fwd): the tcgen05 tensor-core kernel below (TMA-staged
-// input blocks, one M128 N16 K16 MMA per tap, FP32 accumulators in tensor memory).  The
-// backward-data pass is the same kernel on flipped, transposed weights with the ReLU mask of
-// the layer input applied in the epilogue.
-// Weight gradient (conv3d_wgrad): tcgen05 as well, the taps stacked into M (8 taps x 16 input
-// channels per M128 tile), N = 16 output channels, K = voxels; the K-major operands are
-// written per 64-voxel segment with ldmatrix.trans / stmatrix (see k_conv3d_wgrad_tc), then a
-// fixed-order reduction over blocks (deterministic).
+// input planes, one M128 N48 K16 MMA per (dy, dx) for the three dz, FP32 accumulators in tensor
+// memory).  The backward-data pass is the same kernel on flipped, transposed weights with the ReLU
+// mask of the layer input applied in the epilogue.
+// Weight gradient (conv3d_wgrad): tcgen05 as well, (dy, dz, input channel) stacked into M and (dx,
+// output channel) into N, K = voxels; each row's K-major operand is written once per run of rows
+// with ldmatrix.trans / stmatrix (see k_conv3d_wgrad_tc), then a fixed-order reduction over blocks
+// (deterministic).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -24,6 +24,12 @@ namespace pk {
 
 constexpr int kCh = 16;         // channels (padded)
 
+// Units [u, u1) of block b of G: equal shares, the first `units % G` blocks one more.
+__device__ __forceinline__ void unit_share(int units, int& u, int& u1) {
+  const int b = blockIdx.x, G = gridDim.x, base = units / G, rem = units - base * G;
+  u = b * base + min(b, rem);
+  u1 = u + base + (b < rem ? 1 : 0);
+}
 
 struct ConvArgs {
   const __nv_bfloat16* X;     // input activations [D][H][W][16]
@@ -38,37 +44,49 @@ struct ConvArgs {
 };
 
 // ---------------------------------------------------------------- tcgen05 forward kernel
-// Implicit GEMM on the 5th-generation tensor cores: an M = 128 tile of output voxels (8 along
-// x by 16 along y at one z) times N = 16 output channels, K = 27 taps x 16 input channels,
-// one tcgen05.mma (M128 N16 K16, BF16 operands, FP32 accumulator in tensor memory) per tap.
-// The input block around a tile -- 3 planes x 18 rows x 10 voxels, each voxel's 16 channels
-// as two 8-channel halves -- arrives by TMA: six cp.async.bulk.tensor copies of an
-// [18][10][8] box per tile, the halo outside the grid filled with zeros by the copy engine.
-// Each box lands in the no-swizzle K-major layout of the MMA's A operand: a core matrix is 8
+// Implicit GEMM on the 5th-generation tensor cores: an M = 128 tile of voxels (8 along x by 16 along
+// y at one z), K = 16 input channels per tap.  Input-stationary in z: the tile's input plane z (18
+// rows x 10 voxels with the halo) is multiplied once with the taps of all three dz, N = 48 columns =
+// (dz = -1, 0, +1) x 16 output channels, nine MMAs (dy, dx) per plane; column block dz is that
+// plane's share of the outputs at z + 1, z and z - 1, and an output tile is the sum of three blocks
+// of three neighbouring planes, added in the order dz = -1, 0, +1 (each block accumulates its nine
+// taps in order: the same products and sums as one MMA per tap).  So a plane is staged once and its
+// operand rows are read by 9 MMAs, where one MMA per tap and output tile staged every plane three
+// times and read it 27 times: an M128 MMA reads 4 KB of A whatever N is, 32 clocks of shared-memory
+// bandwidth, which bounds so narrow a product.
+// A block takes a run of (column tile, z) units in z order; warp 0 issues the TMA copies (two
+// [18][10][8] boxes per plane, the halo outside the grid filled with zeros), warps 1 and 2 the MMAs
+// of every other plane (one warp's waits between two planes left the tensor pipe idle for as long as
+// the nine MMAs take: 930 clocks per plane where the MMAs are 480), and two groups of four warps take
+// the output tiles in turn (tcgen05.ld, bias, ReLU or mask, BF16 store).  Planes pass through
+// kTcStages staging buffers and kTcSlots accumulator slots in tensor memory; a slot is free once the
+// (up to three) output tiles that read it have.  One block per SM.
+// Measured (64^3, launches back to back): 18.6 us before (one MMA per tap, two blocks per SM), 12.2
+// us now (one MMA warp: 14.7); 72^3: 23.8 -> 14.5; 32^3: 10.7 -> 10.4, which is the launch, the
+// prologue (barriers, tensor memory, weights: 1.2 us) and one run's latency.  The 16.8 MB in and out
+// take 2.4 us of memory time.
+// A box lands in the no-swizzle K-major layout of the MMA's A operand: a core matrix is 8
 // voxels consecutive in x (8 x 16 bytes), the two K halves are kTcHalf bytes apart (leading
-// byte offset) and consecutive y rows kTcRow bytes apart (stride byte offset); a tap
-// (dz, dy, dx) is the same descriptor with its start moved by (dz, dy, dx) voxels; the taps
-// of each dz accumulate in their own tensor-memory accumulator (three independent MMA chains
-// per tile, summed in the epilogue).  Weights
-// [tap][half][co][8 ci] stay in shared memory for the whole launch.  A ring of kTcStages
-// staging buffers and two accumulators pipeline a persistent block's tiles: thread 0 issues
-// the copies and the MMAs of the next tile while all four warps run the epilogue of the
-// current one (tcgen05.ld, bias, ReLU or mask, BF16 store).  Every mbarrier wait is bounded
-// (2 s): a wait that runs out sets a device flag (pk_conv3d_check reports PK_TIMEOUT), the
-// block waits (bounded) for what it issued, frees its tensor memory and returns.
+// byte offset) and consecutive y rows kTcRow bytes apart (stride byte offset); a tap (dy, dx) is the
+// same descriptor with its start moved.  Every mbarrier wait is bounded (2 s): a wait that runs out
+// sets a device flag (pk_conv3d_check reports PK_TIMEOUT), and the block waits (bounded) for what it
+// issued, frees its tensor memory and returns.
 
 constexpr int kTcX = 8, kTcY = 16;                  // tile: 8 x 16 voxels = M 128
 constexpr int kTcBx = kTcX + 2, kTcBy = kTcY + 2;   // staged block with the halo
 constexpr int kTcRow = kTcBx * 16;                  // bytes between staged y rows (SBO)
 constexpr int kTcBox = kTcBy * kTcRow;              // bytes of one [18][10][8] box (2880)
 constexpr int kTcHalf = (kTcBox + 127) & ~127;      // box pitch, 128-byte aligned (LBO)
-constexpr int kTcPlane = 2 * kTcHalf;
-constexpr int kTcStage = 3 * kTcPlane;              // 17,664 bytes
-constexpr int kTcStages = 2;
-constexpr int kTcW = 27 * 512;                      // weights, 13,824 bytes
-constexpr int kTcSmem = kTcStages * kTcStage + kTcW;
-constexpr int kTcChains = 3;                        // independent accumulators per tile (9 taps each)
-constexpr uint32_t kTcCols = 128;                   // tensor memory: 2 tiles x 3 accumulators x 16 columns
+constexpr int kTcPlane = 2 * kTcHalf;               // one staged plane, 5,888 bytes
+constexpr int kTcStages = 16;
+constexpr int kTcN = 48;                            // (dz, output channel)
+constexpr int kTcWTap = kTcN * 32;                  // weights of one (dy, dx): 48 rows x 16 channels
+constexpr int kTcW = 9 * kTcWTap;                   // 13,824 bytes
+constexpr int kTcSmem = kTcStages * kTcPlane + kTcW;
+constexpr int kTcSlots = 10;                        // accumulators of 48 columns
+constexpr uint32_t kTcCols = 512;                   // tensor memory (480 columns in use)
+constexpr int kTcMma = 2;                            // MMA warps: planes in turn
+constexpr int kTcThreads = 32 * (1 + kTcMma + 8);   // copies, MMAs, two epilogue groups of four warps
 
 __device__ int g_conv_timeout = 0;
 
@@ -81,16 +99,31 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t lbo, uint32
 
 // instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 =
 // 1), both K-major (bits 15, 16 = 0), N >> 3 (bits 17-22), M >> 4 (bits 24-28)
-constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(16 >> 3) << 17) |
-                              ((uint32_t)(128 >> 4) << 24);
+template <int M>
+constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
+                              ((uint32_t)(M >> 4) << 24);
 
+template <int M = 128>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(kTcIdesc), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(kTcIdesc<M>), "r"(accumulate)
       : "memory");
+}
+
+// One lane of a converged warp.  The MMA warps run their loops converged and issue under this
+// predicate: descriptors and loop state then live in uniform registers, where a branch on the lane
+// number costs a move per operand (measured: 146 clocks per MMA issued, 5 times what it takes).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p)::"memory");
+  return p != 0;
 }
 
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
@@ -128,230 +161,260 @@ __device__ __forceinline__ void tc_tma_box(uint32_t dst, const CUtensorMap* map,
       : "memory");
 }
 
-__global__ void __launch_bounds__(128) k_conv3d_tc(const __grid_constant__ CUtensorMap xmap, ConvArgs a) {
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+
+// The runs of a block's units [u0, u1), unit = column tile * D + z: planes [za, zb) of one column.
+struct TcRuns {
+  int u, u1, D, col, za, zb;
+  __device__ __forceinline__ TcRuns(int units, int D_) : D(D_) { unit_share(units, u, u1); }
+  __device__ __forceinline__ bool next() {
+    if (u >= u1) return false;
+    col = u / D;
+    za = u - col * D;
+    zb = min(D, za + (u1 - u));
+    u += zb - za;
+    return true;
+  }
+};
+
+__global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_constant__ CUtensorMap xmap, ConvArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_tc[];
-  unsigned char* stg0 = smem_tc;                          // kTcStages staging buffers
-  unsigned char* wsm = smem_tc + kTcStages * kTcStage;    // weights
-  __shared__ __align__(8) uint64_t full_bar[kTcStages];   // staging buffer loaded
-  __shared__ __align__(8) uint64_t mma_bar[2];            // accumulator complete
+  unsigned char* wsm = smem_tc + kTcStages * kTcPlane;     // weights [dy dx][k half][dz, co][8 ci]
+  __shared__ __align__(8) uint64_t full_bar[kTcStages];    // plane loaded
+  __shared__ __align__(8) uint64_t empty_bar[kTcStages];   // plane read by its MMAs
+  __shared__ __align__(8) uint64_t done_bar[kTcSlots];     // accumulator complete
+  __shared__ __align__(8) uint64_t free_bar[kTcSlots];     // accumulator read by its output tiles
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tx = (a.W + kTcX - 1) / kTcX, ty = (a.H + kTcY - 1) / kTcY;
-  const int ntiles = tx * ty * a.D;
-  const int mine = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;  // my tiles
-  for (int e = threadIdx.x; e < 27 * kCh * 2; e += blockDim.x) {
-    const int half = e & 1, row = e >> 1, t = row / kCh, co = row % kCh;
-    *reinterpret_cast<uint4*>(wsm + t * 512 + half * 256 + co * 16) =
-        __ldg(reinterpret_cast<const uint4*>(a.Wt + row * kCh + 8 * half));
-  }
-  proxy_fence();  // the weights are read by the tensor core (async proxy)
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kTcStages; ++s) mbar_init(&full_bar[s], 1);
-    mbar_init(&mma_bar[0], 1);
-    mbar_init(&mma_bar[1], 1);
+  const int units = tx * ty * a.D;  // (< 2^31: checked by the host)
+  // (one barrier per thread: initialised one after the other they took 0.5 us of every launch)
+  if (threadIdx.x < kTcStages) {
+    mbar_init(&full_bar[threadIdx.x], 1);
+    mbar_init(&empty_bar[threadIdx.x], 1);
+    if (threadIdx.x < kTcSlots) {
+      mbar_init(&done_bar[threadIdx.x], 1);
+      mbar_init(&free_bar[threadIdx.x], 3 * 4);  // three output tiles, a warp of four each
+    }
     mbar_fence_init();
-    abort_flag = 0;
+    if (threadIdx.x == 0) abort_flag = 0;
   }
-  if (warp == 0) {
+  __syncthreads();  // the barriers are in place: the copies start while the other warps go on
+  if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
                  "r"(kTcCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  const uint32_t w_addr = smem_addr(wsm), s_base = smem_addr(stg0);
-  auto tile_of = [&](int k, int& z, int& y0, int& x0) {  // the block's k-th tile
-    const int t = blockIdx.x + k * gridDim.x;
-    x0 = (t % tx) * kTcX;
-    y0 = ((t / tx) % ty) * kTcY;
-    z = t / (tx * ty);
-  };
-  auto load = [&](int k) {  // thread 0: the six boxes of tile k into stage k % kTcStages
-    int z, y0, x0;
-    tile_of(k, z, y0, x0);
-    const int s = k % kTcStages;
-    mbar_expect_tx(&full_bar[s], 6 * kTcBox);
-    for (int pl = 0; pl < 3; ++pl)
-      for (int h = 0; h < 2; ++h)
-        tc_tma_box(s_base + s * kTcStage + pl * kTcPlane + h * kTcHalf, &xmap, 8 * h, x0 - 1, y0 - 1,
-                   z + pl - 1, &full_bar[s]);
-  };
-  bool ok = true;
-  auto issue = [&](int k) {  // thread 0: wait for tile k's data, 27 MMAs into accumulator k & 1
-    const int s = k % kTcStages;
-    if (!mbar_wait(&full_bar[s], (k / kTcStages) & 1)) return false;
+  for (int e = (int)threadIdx.x - 32; warp > 0 && e < 27 * kCh * 2; e += kTcThreads - 32) {
+    const int half = e & 1, row = e >> 1, t = row / kCh, co = row % kCh;
+    *reinterpret_cast<uint4*>(wsm + (t % 9) * kTcWTap + half * (kTcN * 16) + ((t / 9) * kCh + co) * 16) =
+        __ldg(reinterpret_cast<const uint4*>(a.Wt + row * kCh + 8 * half));
+  }
+  uint32_t tmem = 0;
+  if (warp > 0) {
+    proxy_fence();  // the weights are read by the tensor core (async proxy)
+    tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"r"(kTcThreads - 32) : "memory");
     tc_fence_after();
-    const uint32_t sa0 = s_base + s * kTcStage;
-    const uint32_t acc = tmem + (k & 1) * (kTcChains * 16);
-    // three chains of nine taps (dz = -1, 0, +1), issued interleaved: consecutive MMAs write
-    // different accumulators and overlap in the tensor pipe
-#pragma unroll 1
-    for (int i = 0; i < 9; ++i) {
-      const int dy = i / 3, dx = i % 3;
+    tmem = tmem_slot;
+  }
+  const uint32_t w_addr = smem_addr(wsm), s_base = smem_addr(smem_tc);
+  volatile int* const stop = &abort_flag;
+  TcRuns run(units, a.D);
+  if (warp == 0) {
+    if (lane == 0) {
+      int q = 0;
+      while (!*stop && run.next()) {
+        const int x0 = (run.col % tx) * kTcX, y0 = (run.col / tx) * kTcY;
+        for (int z = run.za - 1; z <= run.zb; ++z, ++q) {
+          const int s = q % kTcStages;
+          if (q >= kTcStages && !mbar_wait(&empty_bar[s], (q / kTcStages - 1) & 1)) {
+            *stop = 1;
+            break;
+          }
+          mbar_expect_tx(&full_bar[s], 2 * kTcBox);
+          for (int h = 0; h < 2; ++h)
+            tc_tma_box(s_base + s * kTcPlane + h * kTcHalf, &xmap, 8 * h, x0 - 1, y0 - 1, z, &full_bar[s]);
+        }
+      }
+      // bounded waits for the copies in flight before the block leaves
+      for (int p = max(0, q - kTcStages); p < q; ++p)
+        if (!mbar_wait(&full_bar[p % kTcStages], (p / kTcStages) & 1)) *stop = 1;
+    }
+  } else if (warp <= kTcMma) {
+    // descriptors differ by their start address (bits 0-13, in 16-byte units)
+    const uint64_t wd = tc_desc(w_addr, kTcN * 16, 128), xd = tc_desc(s_base, kTcHalf, kTcRow);
+    int q = 0, s = 0, d = 0, use_s = 0, use_d = 0;  // plane, its stage and slot and their uses so far
+    int mine = -1;                                  // this warp's last plane
+    bool ok = true;
+    while (ok && run.next()) {
+      for (int z = run.za - 1; z <= run.zb; ++z, ++q, s = s + 1 == kTcStages ? (++use_s, 0) : s + 1,
+               d = d + 1 == kTcSlots ? (++use_d, 0) : d + 1) {
+        if (q % kTcMma != warp - 1) continue;
+        ok = mbar_wait(&full_bar[s], use_s & 1) && (use_d == 0 || mbar_wait(&free_bar[d], (use_d - 1) & 1));
+        ok = !__any_sync(0xffffffffu, !ok || *stop);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t xs = xd + (uint64_t)(s * (kTcPlane >> 4));
+        const uint32_t acc = tmem + d * kTcN;
+        if (elect_one()) {
 #pragma unroll
-      for (int c = 0; c < kTcChains; ++c) {
-        const int tap = 9 * c + i;  // dz = c - 1
-        tc_mma(acc + c * 16, tc_desc(sa0 + c * kTcPlane + dy * kTcRow + dx * 16, kTcHalf, kTcRow),
-               tc_desc(w_addr + tap * 512, 256, 128), i > 0 ? 1u : 0u);
+          for (int i = 0; i < 9; ++i)
+            tc_mma(acc, xs + (((i / 3) * kTcRow + (i % 3) * 16) >> 4), wd + i * (kTcWTap >> 4), i > 0 ? 1u : 0u);
+          tc_commit(&empty_bar[s]);
+          tc_commit(&done_bar[d]);
+        }
+        __syncwarp();
+        mine = q;
       }
     }
-    tc_commit(&mma_bar[k & 1]);
-    return true;
-  };
-  float bias[16];
+    if (!ok) *stop = 1;
+    // the last commit covers every MMA this warp issued
+    if (mine >= 0 && !mbar_wait(&done_bar[mine % kTcSlots], (mine / kTcSlots) & 1)) *stop = 1;
+  } else {
+    const int grp = (warp - 1 - kTcMma) >> 2, quarter = warp & 3;  // a warp reads its quarter of the lanes
+    float bias[16];
 #pragma unroll
-  for (int c = 0; c < 16; ++c) bias[c] = a.bias ? a.bias[c] : 0.f;
-  if (threadIdx.x == 0 && mine > 0) {
-    for (int k = 0; k < min(kTcStages, mine); ++k) load(k);
-    ok = issue(0);
-  }
-  int issued_mma = threadIdx.x == 0 && mine > 0 && ok ? 1 : 0;
-  for (int k = 0; k < mine; ++k) {
-    // thread 0: the next tile's MMAs go out before this tile's epilogue (other accumulator)
-    if (threadIdx.x == 0 && ok && k + 1 < mine) {
-      ok = issue(k + 1);
-      issued_mma += ok;
-    }
-    if (!ok) abort_flag = 1;
-    if (!mbar_wait(&mma_bar[k & 1], (k >> 1) & 1)) abort_flag = 1;
-    tc_fence_after();
-    __syncthreads();
-    if (abort_flag) break;
-    // the stage of tile k is free: thread 0 refills it with tile k + kTcStages
-    if (threadIdx.x == 0 && k + kTcStages < mine) load(k + kTcStages);
-    int z, y0, x0;
-    tile_of(k, z, y0, x0);
-    float o[16];
-    {
-      // the three partial sums (taps with dz = -1, 0, +1), added in that order
-      const uint32_t row = tmem + ((uint32_t)(32 * warp) << 16) + (k & 1) * (kTcChains * 16);
-      float p1[16], p2[16];
-      tc_ld16(row, o);
-      tc_ld16(row + 16, p1);
-      tc_ld16(row + 32, p2);
+    for (int c = 0; c < 16; ++c) bias[c] = a.bias ? a.bias[c] : 0.f;
+    const int m = 32 * quarter + lane;
+    int q0 = 0, k = 0;  // first plane of the run, output tiles so far
+    while (!__any_sync(0xffffffffu, *stop) && run.next()) {
+      const int x = (run.col % tx) * kTcX + m % kTcX, y = (run.col / tx) * kTcY + m / kTcX;
+      const int c0 = q0 + 1, c1 = q0 + run.zb - run.za;  // planes at the centre of the output tiles
+      for (int c = c0; c <= c1; ++c, ++k) {
+        if ((k & 1) != grp) continue;
+        for (int p = c - 1; p <= c + 1; ++p)
+          if (!mbar_wait(&done_bar[p % kTcSlots], (p / kTcSlots) & 1)) *stop = 1;
+        if (__any_sync(0xffffffffu, *stop)) break;
+        tc_fence_after();
+        float o[16];
+        {
+          // the three partial sums (taps with dz = -1, 0, +1), added in that order
+          const uint32_t row = tmem + ((uint32_t)(32 * quarter) << 16);
+          float p1[16], p2[16];
+          tc_ld16(row + ((c - 1) % kTcSlots) * kTcN, o);
+          tc_ld16(row + (c % kTcSlots) * kTcN + 16, p1);
+          tc_ld16(row + ((c + 1) % kTcSlots) * kTcN + 32, p2);
 #pragma unroll
-      for (int c = 0; c < 16; ++c) o[c] = (o[c] + p1[c]) + p2[c];
-    }
-    const int m = 32 * warp + lane;
-    const int y = y0 + m / kTcX, x = x0 + m % kTcX;
-    if (y < a.H && x < a.W) {
-      const size_t v = ((size_t)z * a.H + y) * a.W + x;
-      if (a.out_f32) {
-        a.Yf[v] = o[0] + bias[0];
-      } else {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          o[c] += bias[c];
-          if (a.relu) o[c] = fmaxf(o[c], 0.f);
+          for (int j = 0; j < 16; ++j) o[j] = (o[j] + p1[j]) + p2[j];
         }
-        if (a.mask) {
-          const uint4 m0 = *reinterpret_cast<const uint4*>(a.mask + v * kCh);
-          const uint4 m1 = *reinterpret_cast<const uint4*>(a.mask + v * kCh + 8);
-          const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
-          const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
+        tc_fence_before();
+        __syncwarp();
+        if (lane < 3) {
+          // slot of plane p: read by the output tiles centred at p - 1, p, p + 1 of this run; the
+          // first of them arrives for those that the run does not have
+          const int p = c - 1 + lane, lo = max(c0, p - 1), hi = min(c1, p + 1);
+          mbar_arrive_n(&free_bar[p % kTcSlots], c == lo ? 1 + (3 - (hi - lo + 1)) : 1);
+        }
+        const int z = run.za + (c - c0);
+        if (y < a.H && x < a.W) {
+          const size_t v = ((size_t)z * a.H + y) * a.W + x;
+          if (a.out_f32) {
+            a.Yf[v] = o[0] + bias[0];
+          } else {
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            if (!(__bfloat162float(mb0[c]) > 0.f)) o[c] = 0.f;
-            if (!(__bfloat162float(mb1[c]) > 0.f)) o[8 + c] = 0.f;
+            for (int j = 0; j < 16; ++j) {
+              o[j] += bias[j];
+              if (a.relu) o[j] = fmaxf(o[j], 0.f);
+            }
+            if (a.mask) {
+              const uint4 m0 = *reinterpret_cast<const uint4*>(a.mask + v * kCh);
+              const uint4 m1 = *reinterpret_cast<const uint4*>(a.mask + v * kCh + 8);
+              const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
+              const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (!(__bfloat162float(mb0[j]) > 0.f)) o[j] = 0.f;
+                if (!(__bfloat162float(mb1[j]) > 0.f)) o[8 + j] = 0.f;
+              }
+            }
+            uint4 p0, p1;
+            __nv_bfloat162* r0 = reinterpret_cast<__nv_bfloat162*>(&p0);
+            __nv_bfloat162* r1 = reinterpret_cast<__nv_bfloat162*>(&p1);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              r0[j] = __floats2bfloat162_rn(o[2 * j], o[2 * j + 1]);
+              r1[j] = __floats2bfloat162_rn(o[8 + 2 * j], o[8 + 2 * j + 1]);
+            }
+            *reinterpret_cast<uint4*>(a.Y + v * kCh) = p0;
+            *reinterpret_cast<uint4*>(a.Y + v * kCh + 8) = p1;
           }
         }
-        uint4 p0, p1;
-        __nv_bfloat162* q0 = reinterpret_cast<__nv_bfloat162*>(&p0);
-        __nv_bfloat162* q1 = reinterpret_cast<__nv_bfloat162*>(&p1);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          q0[c] = __floats2bfloat162_rn(o[2 * c], o[2 * c + 1]);
-          q1[c] = __floats2bfloat162_rn(o[8 + 2 * c], o[8 + 2 * c + 1]);
-        }
-        *reinterpret_cast<uint4*>(a.Y + v * kCh) = p0;
-        *reinterpret_cast<uint4*>(a.Y + v * kCh + 8) = p1;
       }
+      q0 += run.zb - run.za + 2;
     }
-    tc_fence_before();
-    __syncthreads();  // accumulator k & 1 is free again
   }
-  if (abort_flag && threadIdx.x == 0) {
-    atomicExch(&g_conv_timeout, 1);
-    // bounded waits for what this block still has in flight before its tensor memory goes
-    for (int s = 0; s < kTcStages; ++s) mbar_wait(&full_bar[s], 0);
-    mbar_wait(&mma_bar[0], 0);
-    mbar_wait(&mma_bar[1], 0);
-  }
-  (void)issued_mma;
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x == 0 && abort_flag) atomicExch(&g_conv_timeout, 1);
+  if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols) : "memory");
   }
 }
 
 // ---------------------------------------------------------------- tcgen05 weight gradient
-// dW[tap][co][ci] = sum_v G[v][co] A[v + s][ci] (s the tap's shift) as one implicit GEMM per
-// 16 voxels on the tensor cores.  The shift is split between the operands: with
-// s = s_a + s_b, sum_v G[v] A[v + s] = sum_k A[k + s_a] G[k - s_b], so a product of
-//   M = 128 rows (s_a, ci): the 8 shifts s_a = (dz, dy, 0) other than (1, 1, 0), x 16 ci,
-//   N = 96 rows (s_b, co): the 6 shifts s_b = (0, 0, dx) and (1, 1, dx), x 16 co,
-// over K = voxels k holds every tap once: s_a + (0, 0, dx) for the 24 taps with (dz, dy) !=
-// (1, 1), and (0, 0, 0) + (1, 1, dx) for the other 3 (the remaining (s_a, s_b) pairs are not
-// taps and are not read).  One M128 N96 K16 MMA per 16 voxels covers all 27 taps.
-// A block takes 64-voxel x segments of (z, y) rows in turn.  For a segment, bulk copies bring
-// the 3 x 3 rows of A around it and the rows (z, y), (z-1, y-1) of G, 66 voxels each with the
-// x halo (one contiguous run of 32-byte voxels per row; the parts outside the grid are not
-// copied, and the operand writers read zeros for them), into one of five staging buffers,
-// four segments ahead.  Eight warps write the K-major operands -- the
-// shifted copies of A and of G, transposed -- with ldmatrix.trans / stmatrix: each 8 x 8
-// block of [voxel][channel] becomes the [channel][voxel] core matrix of the no-swizzle
-// K-major layout (8 rows of 16 bytes; K-adjacent core matrices kWgLboA / kWgLboB bytes apart,
-// M- or N-adjacent 128).  A loader warp issues the copies (one lane per row), and one thread
-// of another warp issues, per segment, 4 MMAs into one
-// FP32 accumulator of 96 columns in tensor memory that persists over all of the block's
-// segments; three operand buffers rotate, so the writers run up to two segments ahead of
-// the tensor core's completions (mbarriers: operands written by the 8 warps, operands read by
-// the MMAs).  Every wait is bounded (a wait that runs out sets the device
-// flag that pk_conv3d_check reports, and the block waits, bounded, for what it issued before
-// it frees its tensor memory).  At the end each thread reads its accumulator lane (one
-// (s_a, ci) row) into the block's partial; a fixed-order reduction over blocks follows.
+// dW[tap][co][ci] = sum_v G[v][co] A[v + s][ci] (s the tap's shift) as implicit GEMMs on the tensor
+// cores, K = voxels.  With s = (dz, dy, dx), sum_v G[v] A[v + s] = sum_k A[k + (dz, dy, 0)]
+// G[k - (0, 0, dx)]: a product of M rows (dy, dz, ci) and N = 48 columns (dx, co) per 16 voxels.
+// A block walks y along runs of rows (z, y) of a 64-voxel x segment.  A row of A is an operand row
+// group of 16 channels x 64 voxels (2 KB); the groups of a run lie in y order, three (dz) per y, so
+// the nine groups around row y are consecutive and the next y uses six of them again: each row of A
+// is transposed once per run where a separate operand per output row transposed eight.  One MMA of
+// M = 128 takes the first eight groups, a second one of M = 64 (whose other rows are not read) the
+// ninth, (1, 1); both accumulate in tensor memory over the block's rows.
+// A loader warp brings the rows (three of A and one of G per step, 66 voxels with the x halo, zeros
+// outside the grid) as two TMA boxes into a staging ring (a copy per row, issued by a lane each, took
+// 950 clocks per step and set the pace); two groups of eight warps take the steps in turn (a step is a
+// chain of some 1,200 clocks of waits, loads, stores, fence and arrivals, twice what its MMAs take) and
+// write the operands with ldmatrix.trans + stmatrix, which turn [voxel][channel] 8 x 8 blocks into the
+// [channel][voxel] core matrices of the no-swizzle K-major layout (K-adjacent core matrices 128 bytes
+// apart, M- or N-adjacent 1 KB).  (Loading the fragments from global memory instead, 4 bytes of a voxel
+// per thread, took 560 clocks of issue per step.)  Two warps issue the MMAs of every other output row,
+// each into accumulators of its own (one warp's waits and issue took 1,000 clocks per row).  Runs have
+// at most kWgRun rows: two run buffers alternate, and four buffers of G (its three dx shifts) rotate.
+// Every wait is bounded (a wait that runs out sets the device flag that pk_conv3d_check reports, and
+// the block waits, bounded, for what it issued before it frees its tensor memory).  At the end each
+// thread reads its accumulator lane into the block's partial; a fixed-order reduction over blocks
+// follows.
+// Measured with that reduction (64^3, launches back to back): 33.0 us before (an im2col operand per
+// 64-voxel segment), 22.9 us now; 72^3 (two segments per row, the second mostly empty): 69.0 -> 41.9;
+// 32^3: 14.7 -> 14.5.  The rest is issue and wait latency: tensor pipe and memory are idle for most
+// of it.
 constexpr int kWgSeg = 64;                       // voxels (K) per segment
-constexpr int kWgKg = kWgSeg / 8;                // K core matrices per segment
-constexpr int kWgSa = 8, kWgSb = 6;              // shifts on the A side and on the G side
-constexpr int kWgN = kWgSb * 16;                 // 96
-constexpr int kWgLboA = kWgSa * 2 * 128;         // bytes between K-adjacent core matrices of A (2 KB)
-constexpr int kWgLboB = kWgSb * 2 * 128;         // ... of G^T (1.5 KB)
-constexpr int kWgA = kWgKg * kWgLboA;            // 16 KB: A operand of one segment
-constexpr int kWgB = kWgKg * kWgLboB;            // 12 KB: G operand of one segment
-constexpr int kWgHx = kWgSeg + 2;                // staged x extent (halo of one)
-constexpr int kWgRow = kWgHx * 32;               // one staged row: 66 voxels x 16 channels BF16
-constexpr int kWgStageA = 9 * kWgRow;            // A rows (z + dz, y + dy), (dz + 1) 3 + (dy + 1)
-constexpr int kWgStage = (kWgStageA + 2 * kWgRow + 127) & ~127;  // + G rows (z-1, y-1), (z, y)
-constexpr int kWgOp = kWgA + kWgB;               // one operand buffer (28 KB)
-constexpr int kWgStages = 5;                     // staging buffers (copies four segments ahead)
-constexpr int kWgOps = 3;                        // operand buffers (the writers run 2 segments ahead)
-constexpr int kWgSmem = kWgOps * kWgOp + kWgStages * kWgStage;
+constexpr int kWgRun = 10;                       // output rows per run
+constexpr int kWgSlots = kWgRun + 2;             // y rows of A per run
+constexpr int kWgRowOp = 2048;                   // one operand row group: 16 channels x 64 voxels
+constexpr int kWgA = kWgSlots * 3 * kWgRowOp;    // a run's A operand (72 KB)
+constexpr int kWgG = 3 * kWgRowOp;               // G of a row, three dx shifts (6 KB)
+constexpr int kWgGs = 4;                         // (even: see below)
+constexpr int kWgRow = (kWgSeg + 2) * 32;        // a staged row: 66 voxels x 16 channels BF16
+constexpr int kWgStageG = (3 * kWgRow + 127) & ~127;  // A at dz = -1, 0, +1, then G, 128-byte aligned
+constexpr int kWgStage = (kWgStageG + kWgRow + 127) & ~127;
+constexpr int kWgStages = 6;
+constexpr int kWgSmem = 2 * kWgA + kWgGs * kWgG + kWgStages * kWgStage;  // (the second MMA reads 6 KB past a run)
+constexpr int kWgReady = 16;                     // ready barriers (the writers are at most 8 steps ahead)
 constexpr int kWgMaxBlocks = 256;
-constexpr uint32_t kWgCols = 128;                // tensor memory: one accumulator of 96 columns
-constexpr int kWgThreads = 256;                  // 8 warps write the operands
-// instruction descriptor, kind::f16: D FP32, A and B BF16, both K-major, N = 96, M = 128
-constexpr uint32_t kWgIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kWgN >> 3) << 17) |
-                              ((uint32_t)(128 >> 4) << 24);
-
-__device__ __forceinline__ void wg_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(kWgIdesc), "r"(accumulate)
-      : "memory");
-}
+constexpr int kWgMma = 2;                        // MMA warps: output rows in turn, accumulators of their own
+constexpr uint32_t kWgCols = 128 * kWgMma;       // tensor memory: 48 columns at 0 and at 64 for each
+constexpr int kWgWarps = 8;                      // warps that write a step's operands
+constexpr int kWgGroups = 2;                     // groups of them, fill steps in turn
+constexpr int kWgThreads = 32 * kWgWarps * kWgGroups;
+// A group's steps with an output row are every other row, the rows of one MMA warp, and an even number
+// of G buffers keeps a buffer with that pair: its phases complete in order, and no wait can take the
+// phase before the last for the one it needs.
+static_assert(kWgGroups == kWgMma && kWgGs % kWgGroups == 0 && kWgStages % kWgGroups == 0, "buffers and their pairs");
+static_assert(kWgGs * kWgG >= 3 * kWgRowOp && kWgSmem <= 226 * 1024, "the second MMA's unused rows stay in bounds");
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
+               : "r"(addr)
+               : "memory");
 }
 
 __device__ __forceinline__ void stsm4(uint32_t addr, const uint32_t (&r)[4]) {
@@ -360,39 +423,55 @@ __device__ __forceinline__ void stsm4(uint32_t addr, const uint32_t (&r)[4]) {
                : "memory");
 }
 
-__global__ void __launch_bounds__(kWgThreads + 64) k_conv3d_wgrad_tc(const __nv_bfloat16* __restrict__ A,
-                                                                   const __nv_bfloat16* __restrict__ G,
-                                                                   float* partial, float* partial_db, int D,
-                                                                   int H, int W) {
+// The fill steps of a block's units [u, u1), unit = (segment * D + z) * H + y: per run of L rows
+// from ya, steps t = 0 .. L + 1 bring row ya - 1 + t of A and, from t = 2 on, row ya + t - 2 of G,
+// after which that output row can be multiplied.
+struct WgSteps {
+  int u, u1, D, H;
+  int seg, z, ya, L, t, run;
+  __device__ __forceinline__ WgSteps(int units, int D_, int H_) : D(D_), H(H_), L(0), t(1), run(-1) {
+    unit_share(units, u, u1);
+  }
+  __device__ __forceinline__ bool next() {
+    if (++t < L + 2) return true;
+    if (u >= u1) return false;
+    const int zs = u / H;
+    ya = u - zs * H;
+    seg = zs / D;
+    z = zs - seg * D;
+    L = min(kWgRun, min(H - ya, u1 - u));
+    u += L;
+    t = 0;
+    ++run;
+    return true;
+  }
+};
+
+__global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wgrad_tc(const __grid_constant__ CUtensorMap amap,
+                                                                        const __grid_constant__ CUtensorMap gmap,
+                                                                        float* partial, float* partial_db, int D,
+                                                                        int H, int W) {
   extern __shared__ __align__(1024) unsigned char smem_wg[];
-  unsigned char* obuf = smem_wg;                                // kWgOps operand buffers
-  unsigned char* stage = smem_wg + kWgOps * kWgOp;              // kWgStages staging buffers
-  __shared__ __align__(8) uint64_t full_bar[kWgStages];         // staging buffer loaded
-  __shared__ __align__(8) uint64_t empty_bar[kWgStages];        // staging buffer read (8 warps)
-  __shared__ __align__(8) uint64_t ready_bar[kWgOps];           // operands written (8 warps)
-  __shared__ __align__(8) uint64_t free_bar[kWgOps];            // operands read (MMA commit)
+  __shared__ __align__(8) uint64_t full_bar[kWgStages];  // staging buffer loaded
+  __shared__ __align__(8) uint64_t empty_bar[kWgStages]; // staging buffer read (8 warps)
+  __shared__ __align__(8) uint64_t ready_bar[kWgReady];  // a fill step is written (8 warps)
+  __shared__ __align__(8) uint64_t gfree_bar[kWgGs];     // a G buffer is read (MMA commit)
+  __shared__ __align__(8) uint64_t afree_bar[2];         // a run buffer is read
   __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag, consumed;
-  __shared__ __align__(16) uint4 zero16;  // what the operand writers read outside the grid
+  __shared__ int abort_flag;
   __shared__ float dbs[kWgThreads / kCh][kCh];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nseg = (W + kWgSeg - 1) / kWgSeg;
-  const int nchunks = D * H * nseg;  // (< 2^31: checked by the host)
-  const int mine = (int)blockIdx.x < nchunks ? (nchunks - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  proxy_fence();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < kWgStages; ++k) {
-      mbar_init(&full_bar[k], 1);
-      mbar_init(&empty_bar[k], kWgThreads / 32);
-    }
-    for (int k = 0; k < kWgOps; ++k) {
-      mbar_init(&ready_bar[k], kWgThreads / 32);
-      mbar_init(&free_bar[k], 1);
-    }
+  const int units = nseg * D * H;  // (< 2^31: checked by the host)
+  if (threadIdx.x < kWgReady) {
+    const int k = threadIdx.x;
+    mbar_init(&ready_bar[k], kWgWarps);
+    if (k < kWgStages) mbar_init(&full_bar[k], 1);
+    if (k < kWgStages) mbar_init(&empty_bar[k], kWgWarps);
+    if (k < kWgGs) mbar_init(&gfree_bar[k], 1);
+    if (k < 2) mbar_init(&afree_bar[k], kWgMma);
     mbar_fence_init();
-    abort_flag = 0;
-    consumed = 0;
-    zero16 = make_uint4(0, 0, 0, 0);
+    if (k == 0) abort_flag = 0;
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
@@ -404,178 +483,166 @@ __global__ void __launch_bounds__(kWgThreads + 64) k_conv3d_wgrad_tc(const __nv_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const uint32_t o_base = smem_addr(obuf), s_base = smem_addr(stage);
-  float db = 0.f;  // builders: output channel t % 16 over voxels (t / 16) + 16 k of every segment
-  if (warp == kWgThreads / 32) {
-    // MMA warp, lane 0: per segment, once its operands are written, 4 MMAs and a commit
-    if (lane == 0) {
-      int issued = 0;
-      for (int j = 0; j < mine; ++j) {
-        const int b = j % kWgOps;
-        if (!mbar_wait(&ready_bar[b], (j / kWgOps) & 1) || *(volatile int*)&abort_flag) {
-          abort_flag = 1;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t ob = o_base + b * kWgOp;
+  const uint32_t base = smem_addr(smem_wg);
+  volatile int* const stop = &abort_flag;
+  WgSteps step(units, D, H);
+  if (warp > kWgThreads / 32) {
+    // MMA warps: per output row 4 x 2 MMAs
+    const int me = warp - kWgThreads / 32 - 1;
+    const uint32_t acc = tmem + 128 * me;
+    int last = -1;  // this warp's last row
+    const uint64_t sd = tc_desc(base, 128, 1024);  // (start address in 16-byte units, bits 0-13)
+    int f = 0, j = -1, jg = kWgGs - 1;  // fill steps, output row, j % kWgGs
+    bool ok = true;
+    while (step.next()) {
+      if (step.t >= 2) {
+        ++j;
+        if (++jg == kWgGs) jg = 0;
+      }
+      ok = ok && mbar_wait(&ready_bar[f % kWgReady], (f / kWgReady) & 1);  // (of every step)
+      ++f;
+      if (step.t < 2 || j % kWgMma != me) {
+        if (step.t == step.L + 1 && elect_one()) tc_commit(&afree_bar[step.run & 1]);
+        continue;
+      }
+      ok = !__any_sync(0xffffffffu, !ok || *stop);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t ad = sd + (uint64_t)(((step.run & 1) * kWgA + (step.t - 2) * 3 * kWgRowOp) >> 4);
+      const uint64_t gd = sd + (uint64_t)((2 * kWgA + jg * kWgG) >> 4);
+      const uint32_t more = last >= 0 ? 1u : 0u;
+      if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < kWgKg / 2; ++ks)
-          wg_mma(tmem, tc_desc(ob + 2 * ks * kWgLboA, kWgLboA, 128), tc_desc(ob + kWgA + 2 * ks * kWgLboB, kWgLboB, 128),
-                 (j > 0 || ks > 0) ? 1u : 0u);
-        tc_commit(&free_bar[b]);
-        issued = j + 1;
+        for (int ks = 0; ks < kWgSeg / 16; ++ks) {
+          tc_mma(acc, ad + ks * 16, gd + ks * 16, ks > 0 ? 1u : more);
+          tc_mma<64>(acc + 64, ad + ((8 * kWgRowOp) >> 4) + ks * 16, gd + ks * 16, ks > 0 ? 1u : more);
+        }
+        tc_commit(&gfree_bar[jg]);
+        if (step.t == step.L + 1) tc_commit(&afree_bar[step.run & 1]);
       }
-      // the last commit covers every MMA the block issued
-      if (issued > 0 && !mbar_wait(&free_bar[(issued - 1) % kWgOps], ((issued - 1) / kWgOps) & 1)) abort_flag = 1;
+      __syncwarp();
+      last = j;
     }
-  } else if (warp == kWgThreads / 32 + 1) {
-    // loader warp: the bulk copies of segment j into staging buffer j % kWgStages, once the
-    // writers are done with segment j - kWgStages there (its empty barrier: one phase per use
-    // of the buffer, so the wait cannot mistake a later phase for it); lane r < 11 copies row
-    // r (9 rows of A, then G at (z-1, y-1), (z, y)): the in-grid part [xa, xb) of an in-grid
-    // row, x0 - 1 at staged voxel 0
-    int loaded = 0;
-    for (int j = 0; j < mine; ++j) {
-      if (j >= kWgStages) {
-        const int jr = j - kWgStages;
-        bool ok = true;
-        if (lane == 0) ok = mbar_wait(&empty_bar[j % kWgStages], (jr / kWgStages) & 1) && !*(volatile int*)&abort_flag;
-        if (!__shfl_sync(0xffffffffu, ok, 0)) {
-          if (lane == 0) abort_flag = 1;
+    if (!ok) *stop = 1;
+    // the last commit covers every MMA this warp issued
+    if (last >= 0 && !mbar_wait(&gfree_bar[last % kWgGs], (last / kWgGs) & 1)) *stop = 1;
+  } else if (warp == kWgThreads / 32) {
+    // loader warp: one box of A's three rows (dz) and one of G's row per step
+    if (lane == 0) {
+      int f = 0, sb = 0, use = 0;
+      while (!*stop && step.next()) {
+        if (use > 0 && !mbar_wait(&empty_bar[sb], (use - 1) & 1)) {
+          *stop = 1;
           break;
         }
+        const int x0 = step.seg * kWgSeg - 1, y = step.ya - 1 + step.t;
+        const uint32_t dst = base + 2 * kWgA + kWgGs * kWgG + sb * kWgStage;
+        mbar_expect_tx(&full_bar[sb], step.t < 2 ? 3 * kWgRow : 4 * kWgRow);
+        tc_tma_box(dst, &amap, 0, x0, y, step.z - 1, &full_bar[sb]);
+        if (step.t >= 2) tc_tma_box(dst + kWgStageG, &gmap, 0, x0, y - 1, step.z, &full_bar[sb]);
+        ++f;
+        if (++sb == kWgStages) sb = 0, ++use;
       }
-      const int c = (int)blockIdx.x + j * (int)gridDim.x;
-      const int seg = c % nseg, zy = c / nseg;
-      const int z = zy / H, y = zy % H, x0 = seg * kWgSeg;
-      const int xa = max(0, x0 - 1), xb = min(W, x0 + kWgSeg + 1);
-      const uint32_t bytes = (uint32_t)(xb - xa) * 32;
-      const int sb = j % kWgStages;
-      const int row = lane;
-      const int zz = row < 9 ? z + row / 3 - 1 : z + row - 10, yy = row < 9 ? y + row % 3 - 1 : y + row - 10;
-      const bool in = row < 11 && zz >= 0 && zz < D && yy >= 0 && yy < H;
-      const uint32_t total = bytes * (uint32_t)__popc(__ballot_sync(0xffffffffu, in));
-      if (lane == 0) mbar_expect_tx(&full_bar[sb], total);
-      __syncwarp();
-      if (in)
-        bulk_load(stage + sb * kWgStage + (xa - x0 + 1) * 32 + row * kWgRow,
-                  (row < 9 ? A : G) + (((size_t)zz * H + yy) * W + xa) * kCh, bytes, &full_bar[sb]);
-      loaded = j + 1;
-    }
-    if (lane == 0 && *(volatile int*)&abort_flag) {
-      // bounded waits for the copies the writers did not consume before the memory goes
-      for (int k = *(volatile int*)&consumed; k < loaded; ++k)
-        mbar_wait(&full_bar[k % kWgStages], (k / kWgStages) & 1);
+      // bounded waits for the copies in flight before the block leaves
+      for (int p = max(0, f - kWgStages); p < f; ++p)
+        if (!mbar_wait(&full_bar[p % kWgStages], (p / kWgStages) & 1)) *stop = 1;
     }
   } else {
-    // builders: the operand-writing jobs of this thread, 7 blocks of 8 x 8, their source
-    // offsets in a staging buffer and destinations in an operand buffer, the same for every
-    // segment: 8 shifts s_a x 2 channel halves x 8 K groups of A (128 blocks), then 6 shifts
-    // s_b x 2 x 8 of G (96); lanes 8i .. 8i+7 address the rows of block i of a four-block
-    // instruction
-    constexpr int kGroups = (kWgSa + kWgSb) * 2 * kWgKg / 4;  // 56 instructions per segment
-    constexpr int kWarps = kWgThreads / 32;
-    constexpr int kJobs = kGroups / kWarps;                     // 7 per warp
-    static_assert(kGroups % kWarps == 0, "whole instructions per warp");
-    // where each lane's row comes from: staged row 0 .. 10 and voxel x0 + xoff, read as zeros
-    // outside the grid (coded as row << 8 | (xoff + 1))
-    uint32_t src_off[kJobs], dst_off[kJobs], where[kJobs];
-    {
-      const int r = lane & 7, i = lane >> 3;
-#pragma unroll
-      for (int k = 0; k < kJobs; ++k) {
-        const int grp = warp + kWarps * k;
-        const int q = 4 * grp + i;
-        if (q < kWgSa * 2 * kWgKg) {
-          // A[k + s_a][ci], s_a = combo sa of (dz, dy) without (1, 1): staged row sa
-          const int sa = q >> 4, h = (q >> 3) & 1, kg = q & 7;
-          src_off[k] = (sa * kWgHx + kg * 8 + r + 1) * 32 + h * 16;
-          dst_off[k] = kg * kWgLboA + (sa * 2 + h) * 128 + r * 16;
-          where[k] = ((uint32_t)sa << 8) | (uint32_t)(kg * 8 + r + 1);
-        } else {
-          // G[k - s_b][co]: s_b = (0, 0, dx) reads G row (z, y), (1, 1, dx) row (z-1, y-1)
-          const int qb = q - kWgSa * 2 * kWgKg, sb = qb >> 4, h = (qb >> 3) & 1, kg = qb & 7;
-          const int dx = sb % 3 - 1, grow = sb < 3 ? 10 : 9;
-          src_off[k] = (grow * kWgHx + kg * 8 + r - dx + 1) * 32 + h * 16;
-          dst_off[k] = kWgA + kg * kWgLboB + (sb * 2 + h) * 128 + r * 16;
-          where[k] = ((uint32_t)grow << 8) | (uint32_t)(kg * 8 + r - dx + 1);
-        }
+    // writers: three jobs of four 8 x 8 blocks per fill step and warp, of the 12 of A (dz, channel
+    // half, voxel half) and the 12 of G (dx, channel half, voxel half); warps 0 .. 3: A dz = -1, A
+    // dz = +1, G dx = 0; warps 4 .. 7: A dz = 0, G dx = -1, G dx = +1
+    const int grp = warp / kWgWarps;
+    const bool low = (warp & 7) < 4;
+    const int h = (warp >> 1) & 1, kg = 4 * (warp & 1);
+    // this lane addresses row lane % 8 of block lane / 8: the voxel of the loads, the channel of the
+    // stores
+    const int vox = (kg + (lane >> 3)) * 8 + (lane & 7);
+    const uint32_t dst = h * 1024 + (kg + (lane >> 3)) * 128 + (lane & 7) * 16;
+    const uint32_t src = base + 2 * kWgA + kWgGs * kWgG + h * 16 + (vox + 1) * 32;  // (voxel -1 comes first)
+    constexpr int kWgDb = 2 * kWgWarps;
+    float db = 0.f;  // output channel t % 16 over voxels t / 16 % 16 + 16 k of the group's rows of G
+    const int dc = threadIdx.x & (kCh - 1);
+    int f = 0, j = 0;
+    for (; step.next(); j += step.t >= 2, ++f) {
+      if (f % kWgGroups != grp) continue;
+      const int sb = f % kWgStages;
+      // the step's rows, the run's buffer (a group's first step of the run) and G buffer j
+      bool ok = mbar_wait(&full_bar[sb], (f / kWgStages) & 1);
+      if (step.t < kWgGroups && step.run >= 2) ok = ok && mbar_wait(&afree_bar[step.run & 1], (step.run / 2 - 1) & 1);
+      if (step.t >= 2 && j >= kWgGs) ok = ok && mbar_wait(&gfree_bar[j % kWgGs], (j / kWgGs - 1) & 1);
+      if (__any_sync(0xffffffffu, !ok || *stop)) {
+        *stop = 1;
+        break;
       }
-    }
-    const uint32_t zero_addr = smem_addr(&zero16);
-    const int c = threadIdx.x & (kCh - 1);
-    for (int j = 0; j < mine; ++j) {
-      const int b = j % kWgOps, sb = j % kWgStages;
-      // segment j's data, and operand buffer b free (read by the MMAs of segment j - kWgOps)
-      if (lane == 0) {
-        if (!mbar_wait(&full_bar[sb], (j / kWgStages) & 1) ||
-            (j >= kWgOps && !mbar_wait(&free_bar[b], ((j - kWgOps) / kWgOps) & 1)))
-          abort_flag = 1;
-        else if (warp == 0)
-          consumed = j + 1;
+      const uint32_t st = src + sb * kWgStage, sg = st + kWgStageG;
+      const uint32_t ab = base + (step.run & 1) * kWgA + step.t * 3 * kWgRowOp + dst;
+      const uint32_t gb = base + 2 * kWgA + (j % kWgGs) * kWgG + dst;
+      const bool g = step.t >= 2;
+      uint32_t r[3][4];
+      if (low) {
+        ldsm4t(r[0], st);
+        ldsm4t(r[1], st + 2 * kWgRow);
+        if (g) ldsm4t(r[2], sg);
+        stsm4(ab, r[0]);
+        stsm4(ab + 2 * kWgRowOp, r[1]);
+        if (g) stsm4(gb + kWgRowOp, r[2]);
+      } else {
+        ldsm4t(r[0], st + kWgRow);
+        if (g) ldsm4t(r[1], sg + 32);  // dx = -1: G at k + 1
+        if (g) ldsm4t(r[2], sg - 32);  // dx = +1: G at k - 1
+        stsm4(ab + kWgRowOp, r[0]);
+        if (g) stsm4(gb, r[1]);
+        if (g) stsm4(gb + 2 * kWgRowOp, r[2]);
       }
-      __syncwarp();
-      if (*(volatile int*)&abort_flag) break;
-      const uint32_t st = s_base + sb * kWgStage;
-      const int cc = (int)blockIdx.x + j * (int)gridDim.x;
-      const int zy = cc / nseg, z = zy / H, y = zy % H, x0 = (cc % nseg) * kWgSeg;
-      uint32_t rows_in = 0;  // staged rows inside the grid (bit = row, as the loader numbers them)
+      if (g) {
+        const __nv_bfloat16* g16 = reinterpret_cast<const __nv_bfloat16*>(smem_wg + 2 * kWgA + kWgGs * kWgG +
+                                                                           sb * kWgStage + kWgStageG + 32);
 #pragma unroll
-      for (int row = 0; row < 11; ++row) {
-        const int zz = row < 9 ? z + row / 3 - 1 : z + row - 10, yy = row < 9 ? y + row % 3 - 1 : y + row - 10;
-        if (zz >= 0 && zz < D && yy >= 0 && yy < H) rows_in |= 1u << row;
+        for (int xx = (threadIdx.x / kCh) % kWgDb; xx < kWgSeg; xx += kWgDb)
+          db += __bfloat162float(g16[xx * kCh + dc]);
       }
-      {
-        // G at (z, y), x0 + xx: staged row 10, voxel xx + 1 (inside the grid only)
-        const __nv_bfloat16* g16 = reinterpret_cast<const __nv_bfloat16*>(stage + sb * kWgStage +
-                                                                            (10 * kWgHx + 1) * 32);
-#pragma unroll
-        for (int xx = threadIdx.x / kCh; xx < kWgSeg; xx += kWgThreads / kCh)
-          if (x0 + xx < W) db += __bfloat162float(g16[xx * kCh + c]);
-      }
-      const uint32_t ob = o_base + b * kWgOp;
-      uint32_t f[kJobs][4];  // all loads in flight before the stores
-#pragma unroll
-      for (int k = 0; k < kJobs; ++k) {
-        const bool in = ((rows_in >> (where[k] >> 8)) & 1u) && (unsigned)(x0 + (int)(where[k] & 255) - 1) < (unsigned)W;
-        ldsm4t(f[k], in ? st + src_off[k] : zero_addr);
-      }
-#pragma unroll
-      for (int k = 0; k < kJobs; ++k) stsm4(ob + dst_off[k], f[k]);
       proxy_fence();  // the operands are read by the tensor core (async proxy)
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&ready_bar[b]);
+        mbar_arrive(&ready_bar[f % kWgReady]);
         mbar_arrive(&empty_bar[sb]);
       }
     }
-    dbs[threadIdx.x / kCh][c] = db;
+    dbs[threadIdx.x / kCh][dc] = db;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   float* P = partial + (size_t)blockIdx.x * 27 * kCh * kCh;
   if (!abort_flag && warp < kWgThreads / 32) {
-    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31, column blocks s_b = 3 (w / 4) ..
-    // + 2; row m = (s_a, ci): s_a = m / 16 is (dz, dy) = combo s_a of the 3 x 3 without (1, 1)
-    const int q4 = warp & 3, m = 32 * q4 + lane;
-    const int sa = m >> 4, ci = m & 15, dzdy = sa;  // combos 0 .. 7 are (dz + 1) 3 + (dy + 1)
+    // warps 0 .. 3: lanes 32 w .. + 31 of the first accumulator, row m = (group, ci); warp 4: lanes
+    // 0 .. 15 of the second (group 8); the two MMA warps' sums are added (a block of one row has the
+    // first alone).  Group g is (dy, dz) = (g / 3 - 1, g % 3 - 1); columns (dx, co)
+    const int m = 32 * (warp & 3) + lane, ci = m & 15, g = warp < 4 ? m >> 4 : 8;
+    int u0, u1;
+    unit_share(units, u0, u1);
+    const bool two = u1 - u0 >= kWgMma;
+    if (warp <= 4) {
 #pragma unroll 1
-    for (int sb = 3 * (warp >> 2); sb < 3 * (warp >> 2) + 3; ++sb) {
-      float v[16];
-      tc_ld16(tmem + ((uint32_t)(32 * q4) << 16) + sb * 16, v);
-      const int dx = sb % 3 - 1;
-      int tap = -1;
-      if (sb < 3) tap = 3 * dzdy + (dx + 1);             // (dz, dy, dx)
-      else if (dzdy == 4) tap = 3 * 8 + (dx + 1);        // (0, 0, 0) + (1, 1, dx)
-      if (tap >= 0) {
+      for (int dx = 0; dx < 3; ++dx) {
+        float v[16], v2[16];
+        const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (warp < 4 ? 0 : 64) + dx * 16;
+        tc_ld16(at, v);
+        tc_ld16(at + 128, v2);
+        if (two) {
 #pragma unroll
-        for (int co = 0; co < 16; ++co) P[(tap * kCh + co) * kCh + ci] = mine > 0 ? v[co] : 0.f;
+          for (int co = 0; co < 16; ++co) v[co] += v2[co];
+        }
+        const int tap = 9 * (g % 3) + 3 * (g / 3) + dx;
+        if (warp < 4 || lane < 16) {
+#pragma unroll
+          for (int co = 0; co < 16; ++co) P[(tap * kCh + co) * kCh + ci] = v[co];
+        }
       }
     }
     if (threadIdx.x < kCh) {
       float t = 0.f;
-      for (int g = 0; g < kWgThreads / kCh; ++g) t += dbs[g][threadIdx.x];
+      for (int k = 0; k < kWgThreads / kCh; ++k) t += dbs[k][threadIdx.x];
       partial_db[blockIdx.x * kCh + threadIdx.x] = t;
     }
   } else if (abort_flag && threadIdx.x == 0) {
@@ -649,37 +716,85 @@ __device__ __forceinline__ void grid_sums(int n, double* scratch, F&& f, double 
   }
 }
 
-constexpr int kWsGrid = 152;
+// A voxel's 16 channels: three given, the others zero.  Two 16-byte stores where the voxel is aligned.
+__device__ __forceinline__ void ws_voxel(__nv_bfloat16* o, __nv_bfloat16 c0, __nv_bfloat16 c1, __nv_bfloat16 c2) {
+  if (((uintptr_t)o & 15) == 0) {
+    __nv_bfloat162 q[2];
+    q[0].x = c0;
+    q[0].y = c1;
+    q[1].x = c2;
+    q[1].y = __float2bfloat16_rn(0.f);
+    uint4 lo = make_uint4(*reinterpret_cast<const unsigned int*>(&q[0]), *reinterpret_cast<const unsigned int*>(&q[1]), 0, 0);
+    reinterpret_cast<uint4*>(o)[0] = lo;
+    reinterpret_cast<uint4*>(o)[1] = make_uint4(0, 0, 0, 0);
+  } else {
+    o[0] = c0;
+    o[1] = c1;
+    o[2] = c2;
+    for (int c = 3; c < kCh; ++c) o[c] = __float2bfloat16_rn(0.f);
+  }
+}
+
+constexpr int kWsGrid = 608;  // four blocks per SM: a row's loads are a chain that many warps hide
 
 // Residual of the linear extrapolation e = 2 x_{t-1} - x_{t-2} in row i:
-// r = b_i - sum_j a_ij e_j; d = a_ii (1 where the row has no nonzero diagonal entry).
+// r = b_i - sum_j a_ij e_j (left to right, four entries' loads in flight); d = a_ii (1 where the row
+// has no nonzero diagonal entry).
 __device__ __forceinline__ void ws_row(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                       const double* __restrict__ va, const double* xm1,
-                                       const double* xm2, const double* b, int i, double& r,
-                                       double& d) {
+                                       const double* __restrict__ va, const double* __restrict__ xm1,
+                                       const double* __restrict__ xm2, const double* __restrict__ b, int i,
+                                       double& r, double& d) {
   double s = 0.0;
   d = 0.0;
-  for (int j = rp[i]; j < rp[i + 1]; ++j) {
-    const int c = ci[j];
-    const double e = 2.0 * xm1[c] - xm2[c];
-    s = fma(va[j], e, s);
-    if (c == i) d = va[j];
+  const int j1 = __ldg(rp + i + 1);
+  for (int j = __ldg(rp + i); j < j1; j += 4) {
+    int c[4];
+    double v[4], p[4], q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      c[k] = j + k < j1 ? __ldg(ci + j + k) : -1;
+      v[k] = j + k < j1 ? __ldg(va + j + k) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      p[k] = c[k] >= 0 ? __ldg(xm1 + c[k]) : 0.0;
+      q[k] = c[k] >= 0 ? __ldg(xm2 + c[k]) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (c[k] >= 0) {
+        s = fma(v[k], 2.0 * p[k] - q[k], s);
+        if (c[k] == i) d = v[k];
+      }
   }
   r = b[i] - s;
   if (d == 0.0) d = 1.0;
 }
 
-// scales = rms of (r / d, r, d) (1 where zero).
+// What k_ws_rms leaves for k_ws_pack in the 32 bytes of a voxel of X16: r / d, r, d.
+struct WsStash {
+  double z, r, d, unused;
+};
+static_assert(sizeof(WsStash) == kCh * sizeof(__nv_bfloat16), "a voxel's 16 channels");
+
+// scales = rms of (r / d, r, d) (1 where zero).  stash: X16 where it is 8-byte aligned, else null.
+// Bound by FP64 issue: 26 operations per row of seven entries (11 us at 64^3), which the second pass
+// over the rows that k_ws_pack made before doubled.
 __global__ void __launch_bounds__(kBlock) k_ws_rms(int n, const int32_t* rp, const int32_t* ci,
                                                    const double* va, const double* xm1,
                                                    const double* xm2, const double* b,
-                                                   double* scales, double* scratch) {
+                                                   double* scales, double* scratch, WsStash* stash) {
   double out[3];
   bool last;
   grid_sums<3>(n, scratch, [&](int i, double (&v)[3]) {
     double r, d;
     ws_row(rp, ci, va, xm1, xm2, b, i, r, d);
     const double z = r / d;
+    if (stash) {
+      stash[i].z = z;
+      stash[i].r = r;
+      stash[i].d = d;
+    }
     v[0] = fma(z, z, v[0]);
     v[1] = fma(r, r, v[1]);
     v[2] = fma(d, d, v[2]);
@@ -693,36 +808,47 @@ __global__ void __launch_bounds__(kBlock) k_ws_rms(int n, const int32_t* rp, con
 }
 
 // X16[v] = bf16((r/d)/s0, r/s1, d/s2, 0, ..., 0): the Jacobi-scaled residual of the
-// extrapolation, the residual itself and the diagonal, each channel of order one.
+// extrapolation, the residual itself and the diagonal, each channel of order one.  The quotients by
+// the scales are products with their reciprocals (formed once per block: an FP64 division is nine
+// operations of the narrow FP64 pipe; the product is rounded to 24 and then 8 bits).
 __global__ void k_ws_pack(int n, const int32_t* rp, const int32_t* ci, const double* va,
                           const double* xm1, const double* xm2, const double* b,
-                          const double* scales, __nv_bfloat16* X16) {
+                          const double* scales, __nv_bfloat16* X16, int stashed) {
+  __shared__ double inv[3];
+  if (threadIdx.x < 3) inv[threadIdx.x] = 1.0 / scales[threadIdx.x];
+  __syncthreads();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n) return;
-  double r, d;
-  ws_row(rp, ci, va, xm1, xm2, b, v, r, d);
   __nv_bfloat16* o = X16 + (size_t)v * kCh;
-  o[0] = __float2bfloat16_rn((float)(r / d / scales[0]));
-  o[1] = __float2bfloat16_rn((float)(r / scales[1]));
-  o[2] = __float2bfloat16_rn((float)(d / scales[2]));
-  for (int c = 3; c < kCh; ++c) o[c] = __float2bfloat16_rn(0.f);
+  double z, r, d;
+  if (stashed) {
+    const WsStash s = *reinterpret_cast<const WsStash*>(o);
+    z = s.z;
+    r = s.r;
+    d = s.d;
+  } else {
+    ws_row(rp, ci, va, xm1, xm2, b, v, r, d);
+    z = r / d;
+  }
+  const __nv_bfloat16 c[3] = {__float2bfloat16_rn((float)(z * inv[0])), __float2bfloat16_rn((float)(r * inv[1])),
+                              __float2bfloat16_rn((float)(d * inv[2]))};
+  ws_voxel(o, c[0], c[1], c[2]);
 }
 
 // target y = (x_t - 2 x_{t-1} + x_{t-2}) / s0 (what linear extrapolation misses, in units of
 // the Jacobi-scaled residual); G[v][0] = bf16(2 (out - y) / n); loss = mean((out - y)^2).
-__global__ void __launch_bounds__(kBlock) k_ws_loss(int n, const float* out, const double* xt,
-                                                    const double* xm1, const double* xm2,
+__global__ void __launch_bounds__(kBlock) k_ws_loss(int n, const float* __restrict__ out, const double* __restrict__ xt,
+                                                    const double* __restrict__ xm1, const double* __restrict__ xm2,
                                                     const double* scales, __nv_bfloat16* G,
                                                     double* loss, double* scratch) {
-  const double is = 1.0 / scales[0];
+  const double is = 1.0 / scales[0], gn = 2.0 / n;
+  const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
   double sum[1];
   bool last;
   grid_sums<1>(n, scratch, [&](int i, double (&v)[1]) {
     const double d = (double)out[i] - (xt[i] - 2.0 * xm1[i] + xm2[i]) * is;
     v[0] = fma(d, d, v[0]);
-    __nv_bfloat16* gi = G + (size_t)i * kCh;
-    gi[0] = __float2bfloat16_rn((float)(2.0 * d / n));
-    for (int c = 1; c < kCh; ++c) gi[c] = __float2bfloat16_rn(0.f);
+    ws_voxel(G + (size_t)i * kCh, __float2bfloat16_rn((float)(gn * d)), zero, zero);
   }, sum, last);
   if (last && threadIdx.x == 0) *loss = sum[0] / n;
 }
@@ -859,11 +985,9 @@ __global__ void k_ws_grad_pack(int n, const double* __restrict__ g, __nv_bfloat1
   for (int c = 1; c < kCh; ++c) gi[c] = __float2bfloat16_rn(0.f);
 }
 
-// Adam on FP32 master parameters, optional BF16 copy.
-__global__ void k_adam(int count, float* p, const float* grad, float* m, float* v, float lr,
-                       float b1, float b2, float eps, float c1, float c2, __nv_bfloat16* p16) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= count) return;
+// One parameter of Adam (FP32 master, optional BF16 copy).
+__device__ __forceinline__ __nv_bfloat16 adam_one(int e, float* p, const float* grad, float* m, float* v, float lr, float b1,
+                                                  float b2, float eps, float c1, float c2) {
   const float gr = grad[e];
   const float mm = b1 * m[e] + (1.f - b1) * gr;
   const float vv = b2 * v[e] + (1.f - b2) * gr * gr;
@@ -872,18 +996,56 @@ __global__ void k_adam(int count, float* p, const float* grad, float* m, float* 
   const float mh = mm / c1, vh = vv / c2;
   const float np = p[e] - lr * mh / (sqrtf(vh) + eps);
   p[e] = np;
-  if (p16) p16[e] = __float2bfloat16_rn(np);
+  return __float2bfloat16_rn(np);
 }
 
-// Tensor map of a channels-last BF16 activation [D][H][W][16] for the TMA boxes of
-// k_conv3d_tc: dimensions (channel, x, y, z), box (8, 10, 18, 1), zero fill outside.
+__global__ void k_adam(int count, float* p, const float* grad, float* m, float* v, float lr,
+                       float b1, float b2, float eps, float c1, float c2, __nv_bfloat16* p16) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= count) return;
+  const __nv_bfloat16 np = adam_one(e, p, grad, m, v, lr, b1, b2, eps, c1, c2);
+  if (p16) p16[e] = np;
+}
+
+// The same for all tensors of a network in one launch (a step of the four-layer network was eight
+// launches of k_adam and four of k_conv3d_flip, 3.3 us each whatever their size).
+struct AdamTensor {
+  float* p;
+  const float* grad;
+  float* m;
+  float* v;
+  __nv_bfloat16* p16;
+  __nv_bfloat16* flipped;
+  int count, block0;  // elements; the tensor's first block
+};
+struct AdamTensors {
+  AdamTensor t[PK_ADAM_MAX_TENSORS];
+};
+
+__global__ void k_adam_many(const __grid_constant__ AdamTensors a, int tensors, float lr, float b1, float b2, float eps,
+                            float c1, float c2) {
+  int k = 0;
+  while (k + 1 < tensors && (int)blockIdx.x >= a.t[k + 1].block0) ++k;
+  const AdamTensor& t = a.t[k];
+  const int e = ((int)blockIdx.x - t.block0) * blockDim.x + threadIdx.x;
+  if (e >= t.count) return;
+  const __nv_bfloat16 np = adam_one(e, t.p, t.grad, t.m, t.v, lr, b1, b2, eps, c1, c2);
+  if (t.p16) t.p16[e] = np;
+  if (t.flipped) {
+    const int tap = e / (kCh * kCh), co = (e / kCh) % kCh, ci = e % kCh;
+    t.flipped[((26 - tap) * kCh + ci) * kCh + co] = np;
+  }
+}
+
+// Tensor map of a channels-last BF16 activation [D][H][W][16] for the TMA boxes of the convolution
+// kernels: dimensions (channel, x, y, z), box (bc, bx, by, bz), zero fill outside.
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                  CUtensorMapFloatOOBfill);
 
-static pk_status input_map(CUtensorMap* map, const __nv_bfloat16* X, int D, int H, int W, int bx = kTcBx,
-                           int by = kTcBy, int bz = 1) {
+static pk_status input_map(CUtensorMap* map, const __nv_bfloat16* X, int D, int H, int W, int bc,
+                             int bx, int by, int bz) {
   static EncodeTiled encode = nullptr;
   if (!encode) {
     void* fn = nullptr;
@@ -902,13 +1064,13 @@ static pk_status input_map(CUtensorMap* map, const __nv_bfloat16* X, int D, int 
   }
   const cuuint64_t dims[4] = {(cuuint64_t)kCh, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
   const cuuint64_t strides[3] = {(cuuint64_t)kCh * 2, (cuuint64_t)W * kCh * 2, (cuuint64_t)H * W * kCh * 2};
-  const cuuint32_t box[4] = {8, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
+  const cuuint32_t box[4] = {(cuuint32_t)bc, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(X), dims,
                             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
-    set_error("pk_conv3d_fwd: cuTensorMapEncodeTiled failed");
+    set_error("pk_conv3d: cuTensorMapEncodeTiled failed");
     return PK_ERR_CUDA;
   }
   return PK_OK;
@@ -918,10 +1080,6 @@ static pk_status conv_setup() {
   static bool done = false;
   if (!done) {
     PK_CUDA(cudaFuncSetAttribute(k_conv3d_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem));
-    // several blocks per SM (each with its own chain of accumulating MMAs): the largest
-    // shared-memory carveout
-    PK_CUDA(cudaFuncSetAttribute(k_conv3d_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared));
     PK_CUDA(cudaFuncSetAttribute(k_conv3d_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem));
     done = true;
   }
@@ -956,28 +1114,17 @@ pk_status pk_conv3d_fwd(const void* X, const void* Wt, const float* bias, void* 
   a.W = W;
   a.relu = relu;
   a.out_f32 = out_f32;
-  static int grid_max = 0;
-  if (!grid_max) {
-    // resident blocks per SM from the kernel's own footprint (shared memory incl. the
-    // per-block reservation, registers, threads)
-    int dev = 0, sms = 1, smem_sm = 0, resv = 0, regs_sm = 0;
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
     PK_CUDA(cudaGetDevice(&dev));
     PK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    PK_CUDA(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-    PK_CUDA(cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev));
-    PK_CUDA(cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev));
-    cudaFuncAttributes fa;
-    PK_CUDA(cudaFuncGetAttributes(&fa, k_conv3d_tc));
-    const int per_block = kTcSmem + (int)fa.sharedSizeBytes + resv;
-    const int by_smem = smem_sm / per_block;
-    const int by_regs = regs_sm / (128 * ((fa.numRegs + 7) & ~7));
-    grid_max = sms * std::max(1, std::min(std::min(by_smem, by_regs), 16));
   }
   CUtensorMap map;
-  if ((e = input_map(&map, a.X, D, H, W))) return e;
-  const int64_t ntiles = (int64_t)D * ((H + kTcY - 1) / kTcY) * ((W + kTcX - 1) / kTcX);
-  const int grid = (int)std::min<int64_t>(ntiles, grid_max);
-  k_conv3d_tc<<<grid, 128, kTcSmem, (cudaStream_t)stream>>>(map, a);
+  if ((e = input_map(&map, a.X, D, H, W, 8, kTcBx, kTcBy, 1))) return e;
+  // one block per SM (it takes all of the tensor memory), at most one per (column tile, z) unit
+  const int64_t units = (int64_t)D * ((H + kTcY - 1) / kTcY) * ((W + kTcX - 1) / kTcX);
+  k_conv3d_tc<<<(int)std::min<int64_t>(units, sms), kTcThreads, kTcSmem, (cudaStream_t)stream>>>(map, a);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
 }
@@ -1027,13 +1174,10 @@ pk_status pk_conv3d_wgrad(const void* A, const void* G, float* scratch, float* d
   float* partial = scratch;
   float* partial_db = scratch + (size_t)nmax * 27 * kCh * kCh;
   cudaStream_t s = (cudaStream_t)stream;
-  if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(G)) & 15) {
-    set_error("pk_conv3d_wgrad: activations and gradients must be 16-byte aligned");
-    return PK_ERR_ARG;
-  }
-  k_conv3d_wgrad_tc<<<nblk, kWgThreads + 64, kWgSmem, s>>>(static_cast<const __nv_bfloat16*>(A),
-                                                         static_cast<const __nv_bfloat16*>(G), partial,
-                                                         partial_db, D, H, W);
+  CUtensorMap amap, gmap;
+  if ((e = input_map(&amap, static_cast<const __nv_bfloat16*>(A), D, H, W, kCh, kWgSeg + 2, 1, 3))) return e;
+  if ((e = input_map(&gmap, static_cast<const __nv_bfloat16*>(G), D, H, W, kCh, kWgSeg + 2, 1, 1))) return e;
+  k_conv3d_wgrad_tc<<<nblk, kWgThreads + 32 * (1 + kWgMma), kWgSmem, s>>>(amap, gmap, partial, partial_db, D, H, W);
   k_conv3d_wgrad_reduce<<<(27 * kCh * kCh + kCh + 31) / 32, 256, 0, s>>>(partial, partial_db, nblk, dW, db);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
@@ -1058,9 +1202,10 @@ pk_status pk_warmstart_input(pk_csr* A, const double* xm1, const double* xm2, co
   const int n = A->n;
   cudaStream_t s = (cudaStream_t)stream;
   PK_CUDA(cudaMemsetAsync(scratch + 3 * kWsGrid, 0, sizeof(double), s));
-  k_ws_rms<<<kWsGrid, kBlock, 0, s>>>(n, A->rp, A->ci, A->va, xm1, xm2, b, scales, scratch);
+  WsStash* stash = (reinterpret_cast<uintptr_t>(X16) & 7) == 0 ? static_cast<WsStash*>(X16) : nullptr;
+  k_ws_rms<<<kWsGrid, kBlock, 0, s>>>(n, A->rp, A->ci, A->va, xm1, xm2, b, scales, scratch, stash);
   k_ws_pack<<<(n + 255) / 256, 256, 0, s>>>(n, A->rp, A->ci, A->va, xm1, xm2, b, scales,
-                                             static_cast<__nv_bfloat16*>(X16));
+                                             static_cast<__nv_bfloat16*>(X16), stash != nullptr);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
 }
@@ -1163,6 +1308,39 @@ pk_status pk_adam_step(int64_t count, float* p, const float* grad, float* m, flo
   const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
   k_adam<<<(int)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
       (int)count, p, grad, m, v, lr, beta1, beta2, eps, c1, c2, static_cast<__nv_bfloat16*>(p_bf16));
+  PK_CUDA(cudaGetLastError());
+  return PK_OK;
+}
+
+pk_status pk_adam_step_many(int32_t tensors, const int64_t* counts, float* const* p, const float* const* grad,
+                            float* const* m, float* const* v, void* const* p_bf16, void* const* flipped, float lr,
+                            float beta1, float beta2, float eps, int32_t step, void* stream) {
+  if (tensors < 1 || tensors > PK_ADAM_MAX_TENSORS || !counts || !p || !grad || !m || !v || step < 1) {
+    set_error("pk_adam_step_many: bad arguments");
+    return PK_ERR_ARG;
+  }
+  AdamTensors a;
+  int64_t blocks = 0;
+  for (int k = 0; k < tensors; ++k) {
+    AdamTensor& t = a.t[k];
+    t.p16 = p_bf16 ? static_cast<__nv_bfloat16*>(p_bf16[k]) : nullptr;
+    t.flipped = flipped ? static_cast<__nv_bfloat16*>(flipped[k]) : nullptr;
+    if (counts[k] <= 0 || counts[k] >= (int64_t(1) << 31) || !p[k] || !grad[k] || !m[k] || !v[k] ||
+        (t.flipped && counts[k] != 27 * kCh * kCh)) {
+      set_error("pk_adam_step_many: bad tensor");
+      return PK_ERR_ARG;
+    }
+    t.p = p[k];
+    t.grad = grad[k];
+    t.m = m[k];
+    t.v = v[k];
+    t.count = (int)counts[k];
+    t.block0 = (int)blocks;
+    blocks += (counts[k] + 255) / 256;
+  }
+  if (blocks >= (int64_t(1) << 31)) { set_error("pk_adam_step_many: too many parameters"); return PK_ERR_ARG; }
+  const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
+  k_adam_many<<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(a, tensors, lr, beta1, beta2, eps, c1, c2);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
 }

@@ -111,6 +111,9 @@ EXPORTS = {
                                           C.c_void_p, C.c_void_p, C.c_void_p]),
     "pk_adam_step": (C.c_int, [C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_float,
                                C.c_float, C.c_float, C.c_float, C.c_int32, C.c_void_p, C.c_void_p]),
+    "pk_adam_step_many": (C.c_int, [C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                    C.c_void_p, C.c_void_p, C.c_float, C.c_float, C.c_float, C.c_float,
+                                    C.c_int32, C.c_void_p]),
     "pk_status_string": (C.c_char_p, [C.c_int]),
     "pk_last_error": (C.c_char_p, []),
     "pk_version": (C.c_int32, []),
@@ -444,3 +447,17 @@ def warmstart_loss_swept(A: CSRMatrix, out, xt, xm1, xm2, scales, omega, sweeps,
 def adam_step(p, grad, m, v, lr, step, beta1=0.9, beta2=0.999, eps=1e-8, p_bf16=None, stream=None):
     _check(lib().pk_adam_step(p.numel(), _ptr(p), _ptr(grad), _ptr(m), _ptr(v), lr, beta1, beta2, eps,
                               int(step), _ptr(p_bf16), _stream_ptr(stream)), "pk_adam_step")
+
+
+def adam_step_many(ps, grads, ms, vs, lr, step, beta1=0.9, beta2=0.999, eps=1e-8, p_bf16=None, flipped=None,
+                   stream=None):
+    """pk_adam_step_many: one Adam step of several tensors in one launch; p_bf16 / flipped: lists of
+    BF16 tensors or None (per entry too)."""
+    k = len(ps)
+
+    def arr(ts):
+        return None if ts is None else (C.c_void_p * k)(*[_ptr(t).value for t in ts])
+
+    counts = (C.c_int64 * k)(*[p.numel() for p in ps])
+    _check(lib().pk_adam_step_many(k, counts, arr(ps), arr(grads), arr(ms), arr(vs), arr(p_bf16), arr(flipped), lr,
+                                   beta1, beta2, eps, int(step), _stream_ptr(stream)), "pk_adam_step_many")

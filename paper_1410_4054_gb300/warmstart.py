@@ -157,11 +157,9 @@ class ConvNet:
 
     def adam(self, lr=1e-3):
         self.step += 1
-        for li in range(len(LAYERS)):
-            pk.adam_step(self.W32[li], self.dW[li], self.mW[li], self.vW[li], lr, self.step,
-                         p_bf16=self.W16[li])
-            pk.adam_step(self.b32[li], self.db[li], self.mb[li], self.vb[li], lr, self.step)
-        self.refresh_flipped()
+        none = [None] * len(LAYERS)
+        pk.adam_step_many(self.W32 + self.b32, self.dW + self.db, self.mW + self.mb, self.vW + self.vb, lr, self.step,
+                          p_bf16=self.W16 + none, flipped=self.Wf16 + none)
 
     def train_sample(self, A, xm1, xm2, b, xt, lr=1e-3, swept=None):
         """One Adam step on one sample.  swept = (omega, sweeps): the loss is taken on the guess
