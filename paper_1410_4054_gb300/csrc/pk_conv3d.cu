@@ -209,10 +209,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  griddep_wait();  // nothing in memory is read or written before
   for (int e = (int)threadIdx.x - 32; warp > 0 && e < 27 * kCh * 2; e += kTcThreads - 32) {
     const int half = e & 1, row = e >> 1, t = row / kCh, co = row % kCh;
     *reinterpret_cast<uint4*>(wsm + (t % 9) * kTcWTap + half * (kTcN * 16) + ((t / 9) * kCh + co) * 16) =
-        __ldg(reinterpret_cast<const uint4*>(a.Wt + row * kCh + 8 * half));
+        __ldcg(reinterpret_cast<const uint4*>(a.Wt + row * kCh + 8 * half));
   }
   uint32_t tmem = 0;
   if (warp > 0) {
@@ -277,9 +278,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
     if (mine >= 0 && !mbar_wait(&done_bar[mine % kTcSlots], (mine / kTcSlots) & 1)) *stop = 1;
   } else {
     const int grp = (warp - 1 - kTcMma) >> 2, quarter = warp & 3;  // a warp reads its quarter of the lanes
+    const float bl = a.bias && lane < 16 ? __ldcg(a.bias + lane) : 0.f;
     float bias[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) bias[c] = a.bias ? a.bias[c] : 0.f;
+    for (int c = 0; c < 16; ++c) bias[c] = __shfl_sync(0xffffffffu, bl, c);
     const int m = 32 * quarter + lane;
     int q0 = 0, k = 0;  // first plane of the run, output tiles so far
     while (!__any_sync(0xffffffffu, *stop) && run.next()) {
@@ -322,8 +324,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
               if (a.relu) o[j] = fmaxf(o[j], 0.f);
             }
             if (a.mask) {
-              const uint4 m0 = *reinterpret_cast<const uint4*>(a.mask + v * kCh);
-              const uint4 m1 = *reinterpret_cast<const uint4*>(a.mask + v * kCh + 8);
+              const uint4 m0 = __ldcg(reinterpret_cast<const uint4*>(a.mask + v * kCh));
+              const uint4 m1 = __ldcg(reinterpret_cast<const uint4*>(a.mask + v * kCh + 8));
               const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
               const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
 #pragma unroll
@@ -350,6 +352,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
   }
   tc_fence_before();
   __syncthreads();
+  griddep_trigger();
   if (threadIdx.x == 0 && abort_flag) atomicExch(&g_conv_timeout, 1);
   if (warp == 1) {
     tc_fence_after();
@@ -485,6 +488,7 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
   const uint32_t tmem = tmem_slot;
   const uint32_t base = smem_addr(smem_wg);
   volatile int* const stop = &abort_flag;
+  griddep_wait();  // nothing in memory is read or written before
   WgSteps step(units, D, H);
   if (warp > kWgThreads / 32) {
     // MMA warps: per output row 4 x 2 MMAs
@@ -613,6 +617,7 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_trigger();
   float* P = partial + (size_t)blockIdx.x * 27 * kCh * kCh;
   if (!abort_flag && warp < kWgThreads / 32) {
     // warps 0 .. 3: lanes 32 w .. + 31 of the first accumulator, row m = (group, ci); warp 4: lanes
@@ -666,13 +671,15 @@ __global__ void __launch_bounds__(256) k_conv3d_wgrad_reduce(const float* partia
   const int e = blockIdx.x * 32 + lane;
   constexpr int nw = 27 * kCh * kCh;
   float s = 0.f;
+  griddep_trigger();
+  griddep_wait();
   if (e < nw + kCh) {
     const float* src = e < nw ? partial + e : partial_db + (e - nw);
     const size_t stride = e < nw ? (size_t)nw : (size_t)kCh;
     constexpr int kPer = (kWgMaxBlocks + 7) / 8;  // every load of the thread in flight at once
     float v[kPer];
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) v[q] = warp + 8 * q < nblk ? src[(size_t)(warp + 8 * q) * stride] : 0.f;
+    for (int q = 0; q < kPer; ++q) v[q] = warp + 8 * q < nblk ? __ldcg(src + (size_t)(warp + 8 * q) * stride) : 0.f;
 #pragma unroll
     for (int q = 0; q < kPer; ++q)
       if (warp + 8 * q < nblk) s += v[q];
@@ -1124,7 +1131,7 @@ pk_status pk_conv3d_fwd(const void* X, const void* Wt, const float* bias, void* 
   if ((e = input_map(&map, a.X, D, H, W, 8, kTcBx, kTcBy, 1))) return e;
   // one block per SM (it takes all of the tensor memory), at most one per (column tile, z) unit
   const int64_t units = (int64_t)D * ((H + kTcY - 1) / kTcY) * ((W + kTcX - 1) / kTcX);
-  k_conv3d_tc<<<(int)std::min<int64_t>(units, sms), kTcThreads, kTcSmem, (cudaStream_t)stream>>>(map, a);
+  launch_pdl(k_conv3d_tc, (int)std::min<int64_t>(units, sms), kTcThreads, kTcSmem, (cudaStream_t)stream, map, a);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
 }
@@ -1177,8 +1184,9 @@ pk_status pk_conv3d_wgrad(const void* A, const void* G, float* scratch, float* d
   CUtensorMap amap, gmap;
   if ((e = input_map(&amap, static_cast<const __nv_bfloat16*>(A), D, H, W, kCh, kWgSeg + 2, 1, 3))) return e;
   if ((e = input_map(&gmap, static_cast<const __nv_bfloat16*>(G), D, H, W, kCh, kWgSeg + 2, 1, 1))) return e;
-  k_conv3d_wgrad_tc<<<nblk, kWgThreads + 32 * (1 + kWgMma), kWgSmem, s>>>(amap, gmap, partial, partial_db, D, H, W);
-  k_conv3d_wgrad_reduce<<<(27 * kCh * kCh + kCh + 31) / 32, 256, 0, s>>>(partial, partial_db, nblk, dW, db);
+  launch_pdl(k_conv3d_wgrad_tc, nblk, kWgThreads + 32 * (1 + kWgMma), kWgSmem, s, amap, gmap, partial, partial_db, D, H, W);
+  launch_pdl(k_conv3d_wgrad_reduce, (27 * kCh * kCh + kCh + 31) / 32, 256, 0, s, (const float*)partial,
+             (const float*)partial_db, nblk, dW, db);
   PK_CUDA(cudaGetLastError());
   return PK_OK;
 }
