@@ -8,11 +8,13 @@
 // in flight fit in L2), against 76 bytes per row of vector traffic in the launched form.  An
 // iteration is the launched form's two fused phases:
 //   Ap = A p, gathering p from the owning CTA's shared memory through the cluster's
-//   distributed shared memory, with the block sums of <Ap,Ap>, <p,Ap>;
-//   the x, r, p updates with the block sum of <r,r>;
-// each ending in a cluster barrier after which every CTA adds the C block sums in rank order,
+//   distributed shared memory, with the block sums of <Ap,Ap>, <p,Ap>, and of <r,r> from the
+//   update before;
+//   the x, r, p updates;
+// each ending in a cluster barrier.  After the first every CTA adds the C block sums in rank order,
 // so all CTAs hold bit-identical alpha, beta and <r,r> and take the same decisions: control
-// flow is uniform across the cluster and there is no spin-wait.
+// flow is uniform across the cluster and there is no spin-wait.  The convergence test joins the
+// reduction after the product (the last product of a solve is unused).
 //
 // Three shapes, so that more than one CTA can share an SM and one CTA's reductions and
 // barriers overlap another's row products: 512 threads and up to 4096 rows (1 CTA per SM),
@@ -35,13 +37,13 @@ struct BatchClArgs {
   int maxit;
 };
 
-constexpr int kBcSlots = 4;  // block sums per CTA: <Ap,Ap>, <p,Ap> | <r,r>
+constexpr int kBcSlots = 4;  // block sums per CTA: <r,r>, <Ap,Ap>, <p,Ap>
 
 // Shared memory of a CTA of NT threads and up to MAXR rows: p, x, r, Ap, the slots, the
-// reduction buffer (two values per warp) and MAXR + 1 row pointers (padded).
+// reduction buffer (three values per warp) and MAXR + 1 row pointers (padded).
 template <int NT, int MAXR>
 constexpr size_t bc_smem() {
-  return sizeof(double) * (4 * (size_t)MAXR + kBcSlots + 2 * NT / 32) + sizeof(int) * (MAXR + 4);
+  return sizeof(double) * (4 * (size_t)MAXR + kBcSlots + 3 * NT / 32) + sizeof(int) * (MAXR + 4);
 }
 
 // Row l of this CTA (row pointers staged in srp) times p.
@@ -62,7 +64,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
   __shared__ int scs;
   double* slots = sm + 4 * MAXR;
   double* buf = slots + kBcSlots;
-  int* srp = reinterpret_cast<int*>(buf + 2 * NT / 32);  // this CTA's row pointers
+  int* srp = reinterpret_cast<int*>(buf + 3 * NT / 32);  // this CTA's row pointers
   for (;;) {
     if (rank == 0 && threadIdx.x == 0) s_sys = atomicAdd(a.queue, 1);
     cl.sync();
@@ -124,26 +126,30 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
     } else if (rr <= thr2) status = PK_OK;
     else if (a.maxit <= 0) status = PK_NOT_CONVERGED;
     cl.sync();  // p0 in place before the first remote gather
+    double vr = 0.0;
     for (int i = 0; status == kRunning; ++i) {
-      // A p_i and <Ap_i, Ap_i>, <p_i, Ap_i> -> alpha, beta (Eq. (3))
-      v[0] = v[1] = 0.0;
+      // A p_i and <r_i, r_i>, <Ap_i, Ap_i>, <p_i, Ap_i> -> the test, alpha, beta (Eq. (3))
+      double w[3] = {vr, 0.0, 0.0};
       for (int l = threadIdx.x; l < nown; l += NT) {
         const double y = bc_row(S, cl, sp, srp, lg, l);
         sa[l] = y;
-        v[0] = fma(y, y, v[0]);
-        v[1] = fma(sp[l], y, v[1]);
+        w[1] = fma(y, y, w[1]);
+        w[2] = fma(sp[l], y, w[2]);
       }
-      cluster_block_slots<NT, 2>(v, buf, slots);
+      cluster_block_slots<NT, 3>(w, buf, slots);
       cl.sync();
       if (threadIdx.x < 32) {
-        cluster_total<2>(cl, slots, 0, t);
+        double u[3];
+        cluster_total<3>(cl, slots, 0, u);
         int sts = kRunning;
         double al = 0.0, be = 0.0;
-        if (!isfinite(t[0]) || !isfinite(t[1])) sts = PK_ERR_NAN;
-        else if (t[1] <= 0.0) sts = PK_NOT_SPD;
-        else {
-          cg_coefficients_warp(rr, t[0], t[1], al, be);
-        }
+        if (i >= 1) rr = u[0];  // (warp 0 alone needs it from here on)
+        if (i >= 1 && !isfinite(rr)) sts = PK_ERR_NAN;
+        else if (i >= 1 && rr <= thr2) sts = PK_OK;
+        else if (i >= 1 && i >= a.maxit) sts = PK_NOT_CONVERGED;
+        else if (!isfinite(u[1]) || !isfinite(u[2])) sts = PK_ERR_NAN;
+        else if (u[2] <= 0.0) sts = PK_NOT_SPD;
+        else cg_coefficients_warp(rr, u[1], u[2], al, be);
         if (threadIdx.x == 0) {
           sc[0] = al;
           sc[1] = be;
@@ -151,34 +157,21 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
         }
       }
       __syncthreads();
-      if (scs != kRunning) {
-        status = scs;
-        break;
-      }
+      iters = i;
+      status = scs;
+      if (status != kRunning) break;
       const double alpha = sc[0], beta = sc[1];
-      // x, r, p updates (no CTA gathers p before the next cluster barrier) and <r, r>
-      double w[1] = {0.0};
+      // x, r, p updates (no CTA gathers p before the next cluster barrier) and the part of <r, r>
+      vr = 0.0;
       for (int l = threadIdx.x; l < nown; l += NT) {
         const double pk = sp[l];
         sx[l] = fma(alpha, pk, sx[l]);
         const double rn = fma(-alpha, sa[l], sr[l]);
         sr[l] = rn;
         sp[l] = fma(beta, pk, rn);
-        w[0] = fma(rn, rn, w[0]);
+        vr = fma(rn, rn, vr);
       }
-      cluster_block_slots<NT, 1>(w, buf, slots + 2);
-      cl.sync();
-      iters = i + 1;
-      if (threadIdx.x < 32) {
-        double u[1];
-        cluster_total<1>(cl, slots, 2, u);
-        rr = u[0];  // (warp 0 alone needs it from here on)
-        if (threadIdx.x == 0) {
-          scs = !isfinite(rr) ? PK_ERR_NAN : rr <= thr2 ? PK_OK : i + 1 >= a.maxit ? PK_NOT_CONVERGED : kRunning;
-        }
-      }
-      __syncthreads();
-      status = scs;
+      cl.sync();  // p_{i+1} in place; every CTA has read the slots
     }
     for (int l = threadIdx.x; l < nown; l += NT) S.x[row0 + l] = sx[l];
     if (rank == 0 && threadIdx.x == 0) {

@@ -7,13 +7,16 @@
 // the CTA's shared memory for the whole solve.  An iteration is the two fused phases of the
 // launched form:
 //   K-CG-S  Ap = A p (the gathers of p read the owning CTA's shared memory through the
-//           cluster's distributed shared memory) with the block sums of <Ap,Ap>, <p,Ap>;
-//   K-CG-U  x, r, p updates with the block sum of <r,r>;
-// each ending in a hardware cluster barrier, after which every CTA reads the C block sums in
+//           cluster's distributed shared memory) with the block sums of <Ap,Ap>, <p,Ap>, and of
+//           <r,r> from the update before;
+//   K-CG-U  x, r, p updates;
+// each ending in a hardware cluster barrier.  After the first every CTA reads the C block sums in
 // rank order from distributed shared memory, so all CTAs hold bit-identical alpha, beta and
-// <r,r> and take the same exit decision.  Control flow is uniform across the cluster (no CTA
-// leaves a loop another one continues), there is no spin-wait, and a final cluster barrier
-// keeps every CTA's shared memory alive until the last remote read.
+// <r,r> and take the same exit decision.  The convergence test on <r_i, r_i> joins the reduction
+// after A p_i (the last product of a solve is unused): one reduction per iteration instead of two.
+// Control flow is uniform across the cluster (no CTA leaves a loop another one continues), there
+// is no spin-wait, and a final cluster barrier keeps every CTA's shared memory alive until the
+// last remote read.
 #include <algorithm>
 
 #include "pk_cluster.cuh"
@@ -24,7 +27,7 @@ namespace {
 
 constexpr int kCT = 512;          // threads per CTA
 constexpr int kMaxRows = 4096;    // rows per CTA held in shared memory
-constexpr int kSlots = 4;         // block sums per CTA: <Ap,Ap>, <p,Ap> | <r,r>
+constexpr int kSlots = 4;         // block sums per CTA: <r,r>, <Ap,Ap>, <p,Ap>
 
 struct ClusterArgs {
   int32_t n;
@@ -67,81 +70,69 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
   // round trip on the critical path of every iteration
   double* const trace = st->trace;
   const int trace_cap = st->trace_cap;
-  double alpha_last = 0.0, beta_last = 0.0;
+  double alpha_last = 0.0, beta_last = 0.0, vr = 0.0;
   int iters = 0;
   int status = kRunning;
   __shared__ double sc[2];  // alpha, beta
-  __shared__ int scs;       // exit status decided by thread 0 (kRunning: continue)
+  __shared__ int scs;       // exit status decided by warp 0 (kRunning: continue)
   cl.sync();  // every CTA's p is in place before the first remote gather
   for (int i = 0; !done0; ++i) {
-    // K-CG-S: Ap_i and <Ap_i, Ap_i>, <p_i, Ap_i>
-    double v[2] = {0.0, 0.0};
+    // K-CG-S: Ap_i and <r_i, r_i> (from K-CG-U), <Ap_i, Ap_i>, <p_i, Ap_i>
+    double v[3] = {vr, 0.0, 0.0};
     for (int l = threadIdx.x; l < nown; l += kCT) {
       const int row = row0 + l;
       const double s = cluster_row(cl, a.ci, a.va, sp, a.log_rows, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       sa[l] = s;
-      v[0] = fma(s, s, v[0]);
-      v[1] = fma(sp[l], s, v[1]);
+      v[1] = fma(s, s, v[1]);
+      v[2] = fma(sp[l], s, v[2]);
     }
-    cluster_block_slots<kCT, 2>(v, buf, slots);
+    cluster_block_slots<kCT, 3>(v, buf, slots);
     cl.sync();
-    double t[2];
     // the scalar work (two FP64 divisions) runs in one warp and is broadcast: on GB300 every
     // FP64 instruction issued by all warps of a CTA costs the SM's narrow FP64 pipe
     if (threadIdx.x < 32) {
-      cluster_total<2>(cl, slots, 0, t);
+      double t[3];
+      cluster_total<3>(cl, slots, 0, t);
       int sts = kRunning;
       double al = 0.0, be = 0.0;
-      if (!isfinite(t[0]) || !isfinite(t[1])) sts = PK_ERR_NAN;
-      else if (t[1] <= 0.0) sts = PK_NOT_SPD;
-      else {
-        // Eq. (3): alpha_i = <r_i,r_i>/<p_i,Ap_i>, beta_i = alpha_i^2 <Ap_i,Ap_i>/<r_i,r_i> - 1
-        cg_coefficients_warp(rr, t[0], t[1], al, be);
-        if (lead && trace && i < trace_cap) {
-          trace[(size_t)i * 4 + 0] = al;
-          trace[(size_t)i * 4 + 1] = be;
-        }
-      }
+      if (i >= 1) rr = t[0];  // (warp 0 alone needs it)
+      if (i >= 1 && !isfinite(rr)) sts = PK_ERR_NAN;
+      else if (i >= 1 && rr <= thr2) sts = PK_OK;
+      else if (i >= 1 && i >= maxit) sts = PK_NOT_CONVERGED;
+      else if (!isfinite(t[1]) || !isfinite(t[2])) sts = PK_ERR_NAN;
+      else if (t[2] <= 0.0) sts = PK_NOT_SPD;
+      else cg_coefficients_warp(rr, t[1], t[2], al, be);  // Eq. (3)
       if (threadIdx.x == 0) {
         sc[0] = al;
         sc[1] = be;
         scs = sts;
       }
+      if (lead && trace) {
+        if (i >= 1 && i - 1 < trace_cap) trace[(size_t)(i - 1) * 4 + 3] = rr;
+        if (sts == kRunning && i < trace_cap) {
+          trace[(size_t)i * 4 + 0] = al;
+          trace[(size_t)i * 4 + 1] = be;
+        }
+      }
     }
     __syncthreads();
+    iters = i;
     if (scs != kRunning) { status = scs; break; }
     const double alpha = sc[0], beta = sc[1];
     alpha_last = alpha;
     beta_last = beta;
-    // K-CG-U: x_{i+1}, r_{i+1}, p_{i+1} and <r_{i+1}, r_{i+1}>.  No CTA gathers p again
-    // before the next barrier, so p is updated in place.
-    double w[1] = {0.0};
+    // K-CG-U: x_{i+1}, r_{i+1}, p_{i+1} and the part of <r_{i+1}, r_{i+1}>.  No CTA gathers p
+    // again before the next barrier, so p is updated in place.
+    vr = 0.0;
     for (int l = threadIdx.x; l < nown; l += kCT) {
       const double pk = sp[l];
       sx[l] = fma(alpha, pk, sx[l]);
       const double rn = fma(-alpha, sa[l], sr[l]);
       sr[l] = rn;
       sp[l] = fma(beta, pk, rn);
-      w[0] = fma(rn, rn, w[0]);
+      vr = fma(rn, rn, vr);
     }
-    cluster_block_slots<kCT, 1>(w, buf, slots + 2);
-    cl.sync();
-    double u[1];
-    if (threadIdx.x < 32) {
-      cluster_total<1>(cl, slots, 2, u);
-      rr = u[0];  // (warp 0 alone needs it)
-    }
-    iters = i + 1;
-    if (threadIdx.x == 0) {
-      int sts = kRunning;
-      if (!isfinite(rr)) sts = PK_ERR_NAN;
-      else if (rr <= thr2) sts = PK_OK;
-      else if (i + 1 >= maxit) sts = PK_NOT_CONVERGED;
-      if (lead && trace && i < trace_cap) trace[(size_t)i * 4 + 3] = rr;
-      scs = sts;
-    }
-    __syncthreads();
-    if (scs != kRunning) { status = scs; break; }
+    cl.sync();  // p_{i+1} in place; every CTA has read the slots
   }
   for (int l = threadIdx.x; l < nown; l += kCT) {
     a.x[row0 + l] = sx[l];
@@ -161,7 +152,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
   cl.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-size_t cluster_smem(int rows) { return sizeof(double) * ((size_t)4 * rows + kSlots + 2 * kCT / 32); }
+size_t cluster_smem(int rows) { return sizeof(double) * ((size_t)4 * rows + kSlots + 3 * kCT / 32); }
 
 // Cluster size the device runs with the largest shared-memory footprint (16, else 8); 0 if
 // neither.
