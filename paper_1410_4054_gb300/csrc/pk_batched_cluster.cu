@@ -3,7 +3,7 @@
 // the system's p, x, r and Ap in shared memory.
 //
 // A system of n rows goes to a cluster of C CTAs (C = 1, 2, 4, 8 or 16) of R rows each
-// (R = 2^k, R C >= n); CTA k owns rows [k R, (k+1) R).  Per iteration only the matrix is read
+// (equal shares, R C >= n); CTA k owns rows [k R, (k+1) R).  Per iteration only the matrix is read
 // from global memory (12 bytes per nonzero, 4 per row pointer, and the matrices of the systems
 // in flight fit in L2), against 76 bytes per row of vector traffic in the launched form.  An
 // iteration is the launched form's two fused phases:
@@ -48,8 +48,8 @@ constexpr size_t bc_smem() {
 
 // Row l of this CTA (row pointers staged in srp) times p.
 __device__ __forceinline__ double bc_row(const BatchClSys& S, cg::cluster_group& cl, double* sp, const int* srp,
-                                         int lg, int l) {
-  return cluster_row(cl, S.ci, S.va, sp, lg, srp[l], srp[l + 1]);
+                                         const ClusterRows& rows, int l) {
+  return cluster_row(cl, rows, S.ci, S.va, sp, srp[l], srp[l + 1]);
 }
 
 }  // namespace
@@ -73,9 +73,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
     if (k >= a.end) break;  // the same k in every CTA: the cluster leaves together
     const BatchClSys S = a.sys[k];
     const int n = S.n;
-    int lg = 5;
-    while ((1 << lg) * C < n) ++lg;
-    const int R = 1 << lg;
+    const int R = cluster_share(n, C);
+    const ClusterRows rows(R);
     if (R > MAXR) {  // the host plans classes so that this does not happen
       if (rank == 0 && threadIdx.x == 0) a.sys[k].status = PK_ERR_ARG;
       cl.sync();
@@ -99,7 +98,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
     double v[2] = {0.0, 0.0};
     for (int l = threadIdx.x; l < nown; l += NT) {
       const double bi = __ldg(S.b + row0 + l);
-      const double ri = bi - bc_row(S, cl, sp, srp, lg, l);
+      const double ri = bi - bc_row(S, cl, sp, srp, rows, l);
       sr[l] = ri;
       v[0] = fma(ri, ri, v[0]);
       v[1] = fma(bi, bi, v[1]);
@@ -131,7 +130,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       // A p_i and <r_i, r_i>, <Ap_i, Ap_i>, <p_i, Ap_i> -> the test, alpha, beta (Eq. (3))
       double w[3] = {vr, 0.0, 0.0};
       for (int l = threadIdx.x; l < nown; l += NT) {
-        const double y = bc_row(S, cl, sp, srp, lg, l);
+        const double y = bc_row(S, cl, sp, srp, rows, l);
         sa[l] = y;
         w[1] = fma(y, y, w[1]);
         w[2] = fma(sp[l], y, w[2]);

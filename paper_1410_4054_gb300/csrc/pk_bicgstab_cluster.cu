@@ -31,7 +31,7 @@ constexpr int kBiSlots = 8;       // two groups of four block sums
 
 struct BiClusterArgs {
   int32_t n;
-  int32_t log_rows;  // rows per CTA = 1 << log_rows
+  int32_t rows;  // per CTA
   const int32_t* rp;
   const int32_t* ci;
   const double* va;
@@ -49,7 +49,8 @@ size_t bi_cluster_smem(int rows) { return sizeof(double) * ((size_t)6 * rows + k
 __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
   extern __shared__ __align__(16) double sm[];
   cg::cluster_group cl = cg::this_cluster();
-  const int R = 1 << a.log_rows, lg = a.log_rows;
+  const int R = a.rows;
+  const ClusterRows rows(R);
   const int rank = (int)cl.block_rank();
   double* sp = sm;           // p (gathered remotely in phase 1)
   double* ss = sm + R;       // s (gathered remotely in phase 3)
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
     double w[1] = {0.0};
     for (int l = threadIdx.x; l < nown; l += kBiCT) {
       const int row = row0 + l;
-      const double y = cluster_row(cl, a.ci, a.va, sp, lg, __ldg(a.rp + row), __ldg(a.rp + row + 1));
+      const double y = cluster_row(cl, rows, a.ci, a.va, sp, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       sap[l] = y;
       w[0] = fma(y, sz[l], w[0]);
     }
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(kBiCT, 1) k_bi_cluster(BiClusterArgs a) {
     double v[3] = {0.0, 0.0, 0.0};
     for (int l = threadIdx.x; l < nown; l += kBiCT) {
       const int row = row0 + l;
-      const double y = cluster_row(cl, a.ci, a.va, ss, lg, __ldg(a.rp + row), __ldg(a.rp + row + 1));
+      const double y = cluster_row(cl, rows, a.ci, a.va, ss, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       sas[l] = y;
       v[0] = fma(y, ss[l], v[0]);
       v[1] = fma(y, y, v[1]);
@@ -259,11 +260,10 @@ int bi_cluster_size() {
   return cs;
 }
 
-// Rows per CTA (a power of two, at least 32) for n rows on C CTAs; 0 if n does not fit.
+// Rows per CTA for n rows on C CTAs; 0 if n does not fit.
 int bi_rows_per_cta(int64_t n, int C) {
   if (C <= 0) return 0;
-  int R = 32;
-  while ((int64_t)R * C < n) R *= 2;
+  const int R = cluster_share(n, C);
   return R <= kBiMaxRows ? R : 0;
 }
 
@@ -280,9 +280,7 @@ pk_status launch_bicgstab_persistent(pk_csr* A, double* x, const double* r, cons
     set_error("persistent BiCGStab: n too large for one cluster, or no cluster launch");
     return PK_ERR_ARG;
   }
-  int lg = 0;
-  while ((1 << lg) < R) ++lg;
-  BiClusterArgs a{A->n, lg, A->rp, A->ci, A->va, x, r, r0s, A->st};
+  BiClusterArgs a{A->n, R, A->rp, A->ci, A->va, x, r, r0s, A->st};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(kBiCT);

@@ -49,17 +49,32 @@ __device__ __forceinline__ void cluster_total(cg::cluster_group& cl, double* slo
   warp_sums<NV>(out);
 }
 
-// Element `c` of a vector distributed over the cluster, R = 2^lg rows per CTA, each CTA's part
-// at `local` in its shared memory.
-__device__ __forceinline__ double cluster_elem(cg::cluster_group& cl, double* local, int lg, int c) {
-  return *cl.map_shared_rank(local + (c & ((1 << lg) - 1)), c >> lg);
+// Rows over a cluster: CTA k owns rows [k R, (k + 1) R).
+struct ClusterRows {
+  int R;
+  uint32_t inv;  // ceil(2^32 / R): c / R = mulhi(c, inv) for c R < 2^32
+  __device__ __forceinline__ explicit ClusterRows(int rows) : R(rows), inv(0xffffffffu / (uint32_t)rows + 1) {}
+};
+
+// Rows per CTA for n rows on C CTAs: equal shares in whole warps, at least one warp's.  (Shares of a
+// power of two left up to half of the CTAs without rows.)
+__host__ __device__ inline int cluster_share(int64_t n, int C) {
+  const int64_t r = (n + C - 1) / C;
+  return r <= 32 ? 32 : (int)((r + 31) & ~(int64_t)31);
 }
 
-// Row `row` of A times a distributed vector: four entries per step with their loads
+// Element `c` of a vector distributed over the cluster, each CTA's part at `local` in its shared
+// memory.
+__device__ __forceinline__ double cluster_elem(cg::cluster_group& cl, const ClusterRows& rows, double* local, int c) {
+  const int k = (int)__umulhi((uint32_t)c, rows.inv);
+  return *cl.map_shared_rank(local + (c - k * rows.R), k);
+}
+
+// Row of A times a distributed vector: four entries per step with their loads
 // independent, products added left to right.  j, j1: the row's entries.
-__device__ __forceinline__ double cluster_row(cg::cluster_group& cl, const int32_t* __restrict__ ci,
-                                              const double* __restrict__ va, double* local, int lg, int j,
-                                              const int j1) {
+__device__ __forceinline__ double cluster_row(cg::cluster_group& cl, const ClusterRows& rows,
+                                              const int32_t* __restrict__ ci, const double* __restrict__ va,
+                                              double* local, int j, const int j1) {
   double s = 0.0;
   for (; j + 4 <= j1; j += 4) {
     int c[4];
@@ -70,11 +85,11 @@ __device__ __forceinline__ double cluster_row(cg::cluster_group& cl, const int32
       w[k] = __ldg(va + j + k);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) pv[k] = cluster_elem(cl, local, lg, c[k]);
+    for (int k = 0; k < 4; ++k) pv[k] = cluster_elem(cl, rows, local, c[k]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) s = fma(w[k], pv[k], s);
   }
-  for (; j < j1; ++j) s = fma(__ldg(va + j), cluster_elem(cl, local, lg, __ldg(ci + j)), s);
+  for (; j < j1; ++j) s = fma(__ldg(va + j), cluster_elem(cl, rows, local, __ldg(ci + j)), s);
   return s;
 }
 

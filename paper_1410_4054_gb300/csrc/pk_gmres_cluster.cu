@@ -37,7 +37,7 @@ constexpr int kGcSlots = 72;      // partial sums per slot group (up to m - 1 do
 constexpr double kGcEstFloor = 1e-12;
 
 struct GmClusterArgs {
-  int32_t n, log_rows, m;
+  int32_t n, rows, m;  // rows: per CTA
   const int32_t* rp;
   const int32_t* ci;
   const double* va;
@@ -81,7 +81,8 @@ __device__ __forceinline__ double gc_warp_total(cg::cluster_group& cl, double* s
 __global__ void __launch_bounds__(kGcCT, 1) k_gm_cluster(GmClusterArgs a) {
   extern __shared__ __align__(16) double sm[];
   cg::cluster_group cl = cg::this_cluster();
-  const int R = 1 << a.log_rows, lg = a.log_rows;
+  const int R = a.rows;
+  const ClusterRows rows(R);
   const int rank = (int)cl.block_rank();
   double* cur = sm;              // the gathered vector: x at a cycle start, then v_{i-1}
   double* sw = sm + R;           // own rows of r, then of w and v_i
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(kGcCT, 1) k_gm_cluster(GmClusterArgs a) {
     for (int l = threadIdx.x; l < nown; l += kGcCT) {
       const int row = row0 + l;
       const double bi = __ldg(a.b + row);
-      const double ri = bi - cluster_row(cl, a.ci, a.va, cur, lg, __ldg(a.rp + row), __ldg(a.rp + row + 1));
+      const double ri = bi - cluster_row(cl, rows, a.ci, a.va, cur, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       sw[l] = ri;
       p0 = fma(ri, ri, p0);
       p1 = fma(bi, bi, p1);
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(kGcCT, 1) k_gm_cluster(GmClusterArgs a) {
       // A: w = A v_{i-1}
       for (int l = threadIdx.x; l < nown; l += kGcCT) {
         const int row = row0 + l;
-        sw[l] = cluster_row(cl, a.ci, a.va, cur, lg, __ldg(a.rp + row), __ldg(a.rp + row + 1));
+        sw[l] = cluster_row(cl, rows, a.ci, a.va, cur, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       }
       __syncthreads();
       // B: partial <v_j, w>, j = 1 .. i-1, one warp per j (four interleaved row chains)
@@ -389,8 +390,7 @@ int gc_cluster_size() {
 
 int gc_rows_per_cta(int64_t n, int C) {
   if (C <= 0) return 0;
-  int R = 32;
-  while ((int64_t)R * C < n) R *= 2;
+  const int R = cluster_share(n, C);
   return R <= kGcMaxRows ? R : 0;
 }
 
@@ -411,9 +411,7 @@ pk_status launch_gmres_persistent(pk_csr* A, const double* b, double* x, int m, 
     set_error("persistent GMRES: n too large for one cluster, restart outside 1..64, or no cluster launch");
     return PK_ERR_ARG;
   }
-  int lg = 0;
-  while ((1 << lg) < R) ++lg;
-  GmClusterArgs a{A->n, lg, m, A->rp, A->ci, A->va, b, x, V, ld, Rout, xiout, A->st};
+  GmClusterArgs a{A->n, R, m, A->rp, A->ci, A->va, b, x, V, ld, Rout, xiout, A->st};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(kGcCT);

@@ -3,7 +3,7 @@
 // iteration would dominate the solve.
 //
 // One cluster of C CTAs (16 where the device allows it, else 8) runs every iteration of the
-// solve.  CTA k owns rows [k*R, (k+1)*R) with R a power of two; their p, x, r and Ap live in
+// solve.  CTA k owns rows [k*R, (k+1)*R); their p, x, r and Ap live in
 // the CTA's shared memory for the whole solve.  An iteration is the two fused phases of the
 // launched form:
 //   K-CG-S  Ap = A p (the gathers of p read the owning CTA's shared memory through the
@@ -31,7 +31,7 @@ constexpr int kSlots = 4;         // block sums per CTA: <r,r>, <Ap,Ap>, <p,Ap>
 
 struct ClusterArgs {
   int32_t n;
-  int32_t log_rows;  // rows per CTA = 1 << log_rows
+  int32_t rows;  // per CTA
   const int32_t* rp;
   const int32_t* ci;
   const double* va;
@@ -44,7 +44,8 @@ struct ClusterArgs {
 __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
   extern __shared__ __align__(16) double sm[];
   cg::cluster_group cl = cg::this_cluster();
-  const int R = 1 << a.log_rows;
+  const int R = a.rows;
+  const ClusterRows rows(R);
   const int rank = (int)cl.block_rank();
   double* sp = sm;            // p of the owned rows (read remotely by the SpMV)
   double* sx = sm + R;
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cg_cluster(ClusterArgs a) {
     double v[3] = {vr, 0.0, 0.0};
     for (int l = threadIdx.x; l < nown; l += kCT) {
       const int row = row0 + l;
-      const double s = cluster_row(cl, a.ci, a.va, sp, a.log_rows, __ldg(a.rp + row), __ldg(a.rp + row + 1));
+      const double s = cluster_row(cl, rows, a.ci, a.va, sp, __ldg(a.rp + row), __ldg(a.rp + row + 1));
       sa[l] = s;
       v[1] = fma(s, s, v[1]);
       v[2] = fma(sp[l], s, v[2]);
@@ -189,11 +190,10 @@ int cluster_size(int device) {
   return cs;
 }
 
-// Rows per CTA (a power of two, at least 32) for n rows on C CTAs; 0 if n does not fit.
+// Rows per CTA for n rows on C CTAs; 0 if n does not fit.
 int rows_per_cta(int64_t n, int C) {
   if (C <= 0) return 0;
-  int R = 32;
-  while ((int64_t)R * C < n) R *= 2;
+  const int R = cluster_share(n, C);
   return R <= kMaxRows ? R : 0;
 }
 
@@ -213,9 +213,7 @@ pk_status launch_cg_persistent(pk_csr* A, double* x, double* r, double* p, doubl
     set_error("persistent loop: n too large for one cluster, or no cluster launch");
     return PK_ERR_ARG;
   }
-  int lg = 0;
-  while ((1 << lg) < R) ++lg;
-  ClusterArgs a{A->n, lg, A->rp, A->ci, A->va, x, r, p, A->st};
+  ClusterArgs a{A->n, R, A->rp, A->ci, A->va, x, r, p, A->st};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(kCT);
