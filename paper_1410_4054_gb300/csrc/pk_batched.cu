@@ -524,7 +524,7 @@ struct TuneKey {
 };
 struct TuneVal {
   int block, per_sm, lanes;  // lanes -1: the tile engine (block 288, 2 per SM); -2: clusters
-  int rows_cta;              // cluster engine: rows per CTA it aims for (a power of 2)
+  int rows_cta;              // cluster engine: rows per CTA it aims for (a power of 2), 0: automatic
 };
 static std::mutex g_tune_mutex;
 static std::map<TuneKey, TuneVal> g_tune;
@@ -534,6 +534,15 @@ static TuneVal g_last{512, 2, 1, 0};
 constexpr int kClSizes = 5;  // clusters of 1, 2, 4, 8, 16 CTAs
 constexpr int kClClasses = kBcShapeCount * kClSizes;
 constexpr int kClRowsDefault = 2048;
+
+// What the automatic choice plans: CTAs of shape 0 (512 threads, two per SM) with up to t rows each,
+// half as many for a system of at most 2 t rows; shape 0's log2 of the cluster size.
+static int auto_cluster(int n, int t) {
+  const int rows = n <= 2 * t ? t / 2 : t;
+  int c = 0;
+  while (c + 1 < kClSizes && ((long long)rows << c) < n) ++c;
+  return c;
+}
 
 // Class of a system of n rows when the batch aims at rows_cta rows per CTA: the CTA shape
 // whose row limit is rows_cta, else the next larger one that holds n on 16 CTAs, with the
@@ -561,8 +570,22 @@ struct ClusterPlan {
   int first[kClClasses + 1];    // slot j's systems: [first[j], first[j + 1])
 };
 
+// rows_cta 0: the automatic choice.  An SM takes two CTAs of shape 0, so that one system's reductions
+// and barriers overlap another's FP64 work; t, the rows per CTA, is the largest the CTAs hold as long
+// as the batch fills the device (fewer barriers per row), else smaller (an iteration's latency).
+// The short systems at the end of the queues run on shares half as large: their iterations are the
+// batch's tail.  Measured (512 shifted 2D Laplacians, ms): 256 threads x 2048 rows, two per SM 13.5;
+// this with t everywhere 11.4, halved up to t rows 11.2, up to 2 t rows 10.9, up to 4 t rows 11.4.
 static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterPlan& P) {
   const int nsys = (int)h.size();
+  int t = batched_cluster_max_rows(0);
+  const int device_ctas = rows_cta == 0 ? batched_cluster_capacity(0, 1) : 0;
+  while (rows_cta == 0 && t > 512) {
+    long long ctas = 0;
+    for (const BatchSys& S : h) ctas += 1ll << auto_cluster(S.n, t);
+    if (ctas >= device_ctas) break;
+    t /= 2;
+  }
   // launch slots: classes by rows per cluster (descending), then by shape
   std::vector<int> slots(kClClasses);
   for (int c = 0; c < kClClasses; ++c) slots[c] = c;
@@ -575,7 +598,7 @@ static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterP
   }
   std::vector<int> sl(nsys);
   for (int k = 0; k < nsys; ++k) {
-    const int c = cluster_class(std::max(h[k].n, 1), rows_cta);
+    const int c = rows_cta == 0 ? auto_cluster(h[k].n, t) : cluster_class(std::max(h[k].n, 1), rows_cta);
     if (c < 0 || batched_cluster_capacity(c / kClSizes, 1 << (c % kClSizes)) <= 0) return false;
     sl[k] = slot_of[c];
   }
@@ -768,13 +791,15 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
   const int lanes_auto = mean_len <= 12 ? 1 : mean_len <= 24 ? 2 : mean_len <= 48 ? 4 : 8;
   // lanes -1: the tile engine; -2: the cluster engine; otherwise the row kernel with the given
   // lanes.  Automatic: the cluster engine for FP64 batches of rows short enough for one thread each
-  // (512 shifted 2D Laplacians of 1,024 to 65,536 rows to 1e-10 on GB300: 16.9 ms a call, the row kernel at
-  // 512 threads x 2 37.5 ms, tuned 17.5 ms: a large system runs on up to 16 SMs instead of one
-  // block, and its vectors stay in shared memory); longer rows keep the row kernel's lanes.
+  // (512 shifted 2D Laplacians of 1,024 to 65,536 rows to 1e-10 on GB300: 10.9 ms a call, the row kernel at
+  // 512 threads x 2 36.9 ms; 200 of them 5.6 / 25.5 ms, 24 1.6 / 11.6 ms, 2 1.1 / 3.3 ms: a large system
+  // runs on up to 16 SMs instead of one block, and its vectors stay in shared memory); longer rows keep
+  // the row kernel's lanes.
   const TuneVal cluster_cfg{kClRowsDefault / 8, 4096 / kClRowsDefault, -2, kClRowsDefault};
+  const TuneVal cluster_auto{512, 2, -2, 0};
   TuneVal cfg = o->lanes == -1                                          ? TuneVal{kTileThreads, 2, -1, 0}
                 : o->lanes == -2                                        ? cluster_cfg
-                : o->lanes == 0 && clusters_ok && lanes_auto == 1 ? cluster_cfg
+                : o->lanes == 0 && clusters_ok && lanes_auto == 1 ? cluster_auto
                                                                     : TuneVal{512, 2, o->lanes ? o->lanes : lanes_auto, 0};
   const TuneKey key{nsys, rows, nnz, mixed};
   bool have = false;
@@ -827,8 +852,8 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
         if (rep == 1 && ms < best) { best = ms; cfg = TuneVal{kTileThreads, 2, -1, 0}; }
       }
     }
-    if (clusters_ok && o->lanes == 0) {  // the cluster engine at 1024, 2048, 4096 rows per CTA
-      for (int rc = 1024; rc <= 4096; rc *= 2) {
+    if (clusters_ok && o->lanes == 0) {  // the cluster engine as planned, and at 1024, 2048, 4096 rows per CTA
+      for (int rc : {0, 1024, 2048, 4096}) {
         ClusterPlan P;
         if (!plan_clusters(h, rc, P)) continue;
         PK_CUDA(cudaMemcpyAsync(dcl, P.sys.data(), sizeof(BatchClSys) * nsys, cudaMemcpyHostToDevice, s));
@@ -840,7 +865,7 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
           PK_CUDA(cudaEventSynchronize(a1));
           float ms = 0;
           PK_CUDA(cudaEventElapsedTime(&ms, a0, a1));
-          if (rep == 1 && ms < best) { best = ms; cfg = TuneVal{rc / 8, 4096 / rc, -2, rc}; }
+          if (rep == 1 && ms < best) { best = ms; cfg = rc ? TuneVal{rc / 8, 4096 / rc, -2, rc} : cluster_auto; }
         }
       }
     }

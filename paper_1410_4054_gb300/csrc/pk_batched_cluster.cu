@@ -1,6 +1,6 @@
 // The cluster engine of the batched solver: pipelined CG (Alg. 2, Sec. 3.1) on many
 // independent systems, each solved to completion by one thread-block cluster whose CTAs hold
-// the system's p, x, r and Ap in shared memory.
+// the system's p, r and Ap in shared memory.
 //
 // A system of n rows goes to a cluster of C CTAs (C = 1, 2, 4, 8 or 16) of R rows each
 // (equal shares, R C >= n); CTA k owns rows [k R, (k+1) R).  Per iteration only the matrix is read
@@ -16,11 +16,15 @@
 // flow is uniform across the cluster and there is no spin-wait.  The convergence test joins the
 // reduction after the product (the last product of a solve is unused).
 //
-// Three shapes, so that more than one CTA can share an SM and one CTA's reductions and
-// barriers overlap another's row products: 512 threads and up to 4096 rows (1 CTA per SM),
-// 256 threads and 2048 rows (2 per SM), 128 threads and 1024 rows (4 per SM).  Each (shape,
-// C) class of the batch is one persistent launch that takes systems from the class's queue;
-// the host puts the classes on streams of their own so that they share the GPU.
+// x stays in global memory (its owner reads and writes it once per iteration), which leaves shared
+// memory for 1,024 threads per SM: one CTA's reductions and barriers overlap another's row products.
+// Bound by FP64 issue (11 operations per row of five entries and iteration, 512 systems 6.8 ms of the
+// 10.9) and by the last systems of the queues, whose iteration counts nobody knows beforehand.  With x
+// in shared memory and 512 threads per SM the same batch took 13.3 ms.
+//
+// Three shapes: 512 threads and up to 4096 rows (2 CTAs per SM), 256 threads and 2048 rows, 128 threads
+// and 1024 rows.  Each (shape, C) class of the batch is one persistent launch that takes systems from
+// the class's queue; the host puts the classes on streams of their own so that they share the GPU.
 #include <algorithm>
 
 #include "pk_cluster.cuh"
@@ -39,11 +43,11 @@ struct BatchClArgs {
 
 constexpr int kBcSlots = 4;  // block sums per CTA: <r,r>, <Ap,Ap>, <p,Ap>
 
-// Shared memory of a CTA of NT threads and up to MAXR rows: p, x, r, Ap, the slots, the
+// Shared memory of a CTA of NT threads and up to MAXR rows: p, r, Ap, the slots, the
 // reduction buffer (three values per warp) and MAXR + 1 row pointers (padded).
 template <int NT, int MAXR>
 constexpr size_t bc_smem() {
-  return sizeof(double) * (4 * (size_t)MAXR + kBcSlots + 3 * NT / 32) + sizeof(int) * (MAXR + 4);
+  return sizeof(double) * (3 * (size_t)MAXR + kBcSlots + 3 * NT / 32) + sizeof(int) * (MAXR + 4);
 }
 
 // Row l of this CTA (row pointers staged in srp) times p.
@@ -55,14 +59,14 @@ __device__ __forceinline__ double bc_row(const BatchClSys& S, cg::cluster_group&
 }  // namespace
 
 template <int NT, int MAXR>
-__global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a) {
+__global__ void __launch_bounds__(NT, 1024 / NT) k_batched_cluster(BatchClArgs a) {
   extern __shared__ __align__(16) double sm[];
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   __shared__ int s_sys;
   __shared__ double sc[2];
   __shared__ int scs;
-  double* slots = sm + 4 * MAXR;
+  double* slots = sm + 3 * MAXR;
   double* buf = slots + kBcSlots;
   int* srp = reinterpret_cast<int*>(buf + 3 * NT / 32);  // this CTA's row pointers
   for (;;) {
@@ -81,16 +85,12 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       continue;
     }
     double* sp = sm;  // p (read remotely by the SpMV); x during the setup product
-    double* sx = sm + R;
-    double* sr = sm + 2 * R;
-    double* sa = sm + 3 * R;
+    double* sr = sm + R;
+    double* sa = sm + 2 * R;
     const int row0 = rank * R;
     const int nown = max(0, min(n - row0, R));
-    for (int l = threadIdx.x; l < nown; l += NT) {
-      const double xv = S.x[row0 + l];
-      sx[l] = xv;
-      sp[l] = xv;
-    }
+    double* const gx = S.x + row0;  // x stays in global memory: only its owner reads it, once per iteration
+    for (int l = threadIdx.x; l < nown; l += NT) sp[l] = gx[l];
     if (nown > 0)  // (a CTA past the last row reads no row pointer: rp has n + 1 entries)
       for (int l = threadIdx.x; l <= nown; l += NT) srp[l] = __ldg(S.rp + row0 + l);
     cl.sync();
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
     int status = kRunning, iters = 0;
     if (!isfinite(rr) || !isfinite(bb)) status = PK_ERR_NAN;
     else if (bb == 0.0) {
-      for (int l = threadIdx.x; l < nown; l += NT) sx[l] = 0.0;
+      for (int l = threadIdx.x; l < nown; l += NT) gx[l] = 0.0;
       status = PK_OK;
     } else if (rr <= thr2) status = PK_OK;
     else if (a.maxit <= 0) status = PK_NOT_CONVERGED;
@@ -162,9 +162,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       const double alpha = sc[0], beta = sc[1];
       // x, r, p updates (no CTA gathers p before the next cluster barrier) and the part of <r, r>
       vr = 0.0;
+#pragma unroll 4
       for (int l = threadIdx.x; l < nown; l += NT) {
         const double pk = sp[l];
-        sx[l] = fma(alpha, pk, sx[l]);
+        gx[l] = fma(alpha, pk, gx[l]);
         const double rn = fma(-alpha, sa[l], sr[l]);
         sr[l] = rn;
         sp[l] = fma(beta, pk, rn);
@@ -172,7 +173,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batched_cluster(BatchClArgs a)
       }
       cl.sync();  // p_{i+1} in place; every CTA has read the slots
     }
-    for (int l = threadIdx.x; l < nown; l += NT) S.x[row0 + l] = sx[l];
     if (rank == 0 && threadIdx.x == 0) {
       a.sys[k].iters = iters;
       a.sys[k].status = status;
