@@ -701,9 +701,6 @@ pk_status pk_csr_destroy(pk_csr* A) {
   if (A->res_flag) cudaFree(A->res_flag);
   if (A->blk_row) cudaFree(A->blk_row);
   if (A->sm_own) cudaFree(A->sm_own);
-  if (A->sm_halo_ptr) cudaFree(A->sm_halo_ptr);
-  if (A->sm_halo) cudaFree(A->sm_halo);
-  if (A->sm_ci16) cudaFree(A->sm_ci16);
   if (A->sm_exchange) cudaFree(A->sm_exchange);
   if (A->small) cudaFree(A->small);
   if (A->partials) cudaFree(A->partials);

@@ -398,10 +398,10 @@ struct pk_csr {
   bool sm_irregular = false;
   void* sm_own = nullptr;
   int sm_halo_max = 0;              // most halo columns of one block
-  int32_t* sm_halo_ptr = nullptr;   // grid_tma + 1
+  void* sm_exchange = nullptr;      // exchange buffers, then the three arrays below
+  int32_t* sm_halo_ptr = nullptr;   // sm_grid + 1
   int32_t* sm_halo = nullptr;
   uint16_t* sm_ci16 = nullptr;
-  void* sm_exchange = nullptr;
   uint64_t sm_epoch = 0, sm_epoch_next = 0;
   pk_graph_entry graphs[4];
   cudaEvent_t ev_pool[64] = {nullptr};

@@ -90,11 +90,13 @@ pk_status build(pk_csr* A, cudaStream_t s) {
   for (auto k : {k_sm_plan<false>, k_sm_plan<true>})
     PK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   std::vector<int32_t> ptr(G + 1, 0);
-  // counts, then the list's offsets (G + 1 each would do; one allocation)
-  PK_CUDA(cudaMalloc(&A->sm_halo_ptr, sizeof(int32_t) * (G + 1)));
-  k_sm_plan<false><<<G, kPlanThreads, smem, s>>>(A->rp, A->ci, A->sm_blk_row, words, A->sm_halo_ptr, nullptr, nullptr, nullptr);
+  if (pk_status e = ensure_state(A)) return e;
+  // the counts in the reductions' scratch (three sums per block); one allocation, one wait: a handle's
+  // first solve pays for them
+  int32_t* cnt = reinterpret_cast<int32_t*>(A->partials);
+  k_sm_plan<false><<<G, kPlanThreads, smem, s>>>(A->rp, A->ci, A->sm_blk_row, words, cnt, nullptr, nullptr, nullptr);
   PK_CUDA(cudaGetLastError());
-  PK_CUDA(cudaMemcpyAsync(ptr.data(), A->sm_halo_ptr, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, s));
+  PK_CUDA(cudaMemcpyAsync(ptr.data(), cnt, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, s));
   PK_CUDA(cudaStreamSynchronize(s));
   int sum = 0, most = 0;
   for (int b = 0; b < G; ++b) {
@@ -109,14 +111,18 @@ pk_status build(pk_csr* A, cudaStream_t s) {
   if (sm_even(A->sm_rows_max) + most > 65535) return PK_OK;
   need = sm_bytes(A->sm_rows_max, A->sm_nnz_max, most, 3, 1);
   if (need > kSmBytesMax) return PK_OK;  // no loop fits
+  const auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+  const size_t b0 = up(exchange_bytes(A)), b1 = up(sizeof(int32_t) * (G + 1)), b2 = up(sizeof(int32_t) * std::max(1, sum));
+  PK_CUDA(cudaMalloc(&A->sm_exchange, b0 + b1 + b2 + sizeof(uint16_t) * ((size_t)A->nnz + 64)));
+  char* d = reinterpret_cast<char*>(A->sm_exchange);
+  A->sm_halo_ptr = reinterpret_cast<int32_t*>(d + b0);
+  A->sm_halo = reinterpret_cast<int32_t*>(d + b0 + b1);
+  A->sm_ci16 = reinterpret_cast<uint16_t*>(d + b0 + b1 + b2);
+  // (from pageable memory: staged before the call returns)
   PK_CUDA(cudaMemcpyAsync(A->sm_halo_ptr, ptr.data(), sizeof(int32_t) * (G + 1), cudaMemcpyHostToDevice, s));
-  PK_CUDA(cudaMalloc(&A->sm_halo, sizeof(int32_t) * std::max(1, sum)));
-  PK_CUDA(cudaMalloc(&A->sm_ci16, sizeof(uint16_t) * ((size_t)A->nnz + 64)));
-  PK_CUDA(cudaMalloc(&A->sm_exchange, exchange_bytes(A)));
   k_sm_plan<true><<<G, kPlanThreads, smem, s>>>(A->rp, A->ci, A->sm_blk_row, words, nullptr, A->sm_halo_ptr, A->sm_halo,
                                                  A->sm_ci16);
   PK_CUDA(cudaGetLastError());
-  PK_CUDA(cudaStreamSynchronize(s));  // (ptr is a host vector)
   A->sm_state = 1;
   return PK_OK;
 }
