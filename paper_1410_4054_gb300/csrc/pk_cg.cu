@@ -17,6 +17,30 @@
 
 namespace pk {
 
+// The solver state from <r0, r0> and <b, b>; s0: BiCGStab's <r0, r0*> with r0* = r0.
+__device__ __forceinline__ void residual_state(DevState* st, double rr, double bb, bool s0) {
+  const double tol = st->thr2;
+  st->rr = rr;
+  st->bb = bb;
+  st->thr2 = tol * tol * bb;
+  st->iter = 0;
+  if (s0) st->s[0] = rr;
+  if (__ldcg(&st->timeout)) {
+    finish(st, PK_TIMEOUT);
+  } else if (!isfinite(rr) || !isfinite(bb)) {
+    finish(st, PK_ERR_NAN);
+  } else if (bb == 0.0) {
+    st->zero_x = 1;
+    st->rr = 0.0;
+    finish(st, PK_OK);
+  } else if (rr <= st->thr2) {
+    finish(st, PK_OK);
+  } else if (st->maxit <= 0) {
+    finish(st, PK_NOT_CONVERGED);
+  }
+  st->counter = 0;
+}
+
 // r = b - A x, p = r; first stage of <r, r> and <b, b>.  Last block: rr, bb, thr2, and the
 // zero-iteration exits (b = 0 -> x = 0; ||r0|| <= tol ||b||).
 __global__ void __launch_bounds__(kBlock) k_residual_init(RowArgs a, const double* __restrict__ b,
@@ -39,27 +63,34 @@ __global__ void __launch_bounds__(kBlock) k_residual_init(RowArgs a, const doubl
   if (arrive_last(&a.st->counter)) {
     double t[2];
     final_sums<2>(a.partials, t);
-    if (threadIdx.x == 0) {
-      DevState* st = a.st;
-      const double tol = st->thr2;
-      st->rr = t[0];
-      st->bb = t[1];
-      st->thr2 = tol * tol * t[1];
-      st->iter = 0;
-      if (r0s) st->s[0] = t[0];  // BiCGStab: <r0, r0*> with r0* = r0
-      if (!isfinite(t[0]) || !isfinite(t[1])) {
-        finish(st, PK_ERR_NAN);
-      } else if (t[1] == 0.0) {
-        st->zero_x = 1;
-        st->rr = 0.0;
-        finish(st, PK_OK);
-      } else if (t[0] <= st->thr2) {
-        finish(st, PK_OK);
-      } else if (st->maxit <= 0) {
-        finish(st, PK_NOT_CONVERGED);
-      }
-      st->counter = 0;
-    }
+    if (threadIdx.x == 0) residual_state(a.st, t[0], t[1], r0s != nullptr);
+  }
+}
+
+// The same on the CSR tile engine.
+template <bool IRR>
+__global__ void __launch_bounds__(kTileThreads, 2) k_residual_init_tma(CsrTiles T, const double* __restrict__ b,
+                                                                       const double* __restrict__ x,
+                                                                       double* __restrict__ r, double* __restrict__ p,
+                                                                       double* __restrict__ r0s, double* partials,
+                                                                       DevState* st) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  double v[2] = {0.0, 0.0};
+  csr_tiles<IRR>(T, smem, st, [&]() { return true; }, x, [&](int row, double y) {
+    const double bi = b[row];
+    const double ri = bi - y;
+    r[row] = ri;
+    if (p) p[row] = ri;
+    if (r0s) r0s[row] = ri;
+    v[0] = fma(ri, ri, v[0]);
+    v[1] = fma(bi, bi, v[1]);
+  });
+  __syncthreads();
+  tile_block_partials<2>(v, partials);
+  if (arrive_last(&st->counter)) {
+    double t[2];
+    final_sums<2>(partials, t);
+    if (threadIdx.x == 0) residual_state(st, t[0], t[1], r0s != nullptr);
   }
 }
 
@@ -351,6 +382,8 @@ static pk_status tma_setup() {
                                  stream_smem_bytes<4, double, 2>()));
     for (auto k : {k_cg_spmv_dots_tma<false>, k_cg_spmv_dots_tma<true>})
       PK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, csr_smem_bytes()));
+    for (auto k : {k_residual_init_tma<false>, k_residual_init_tma<true>})
+      PK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, csr_smem_bytes()));
     for (auto k : {k_spmv_tma<false>, k_spmv_tma<true>})
       PK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, csr_smem_bytes()));
     done = true;
@@ -538,7 +571,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if (resident) {
     // r0, p0, <r0,r0>, <b,b>; then the whole iteration loop in one cooperative launch
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    k_residual_init<<<A->grid, kBlock, 0, s>>>(row_args(A), bd, xd, r, p, nullptr);
+    if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, true, s))) return e;
     if ((e = T.end())) return e;
     k_zero_x<<<A->grid, kBlock, 0, s>>>(row_args(A), xd);
     PK_CUDA(cudaGetLastError());
@@ -571,7 +604,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
 
   // setup: r0 = b - A x0, p0 = r0, <r0,r0>, <b,b>
   if ((e = T.begin(PK_SLOT_OTHER))) return e;
-  k_residual_init<<<G, kBlock, 0, s>>>(ra, bd, xd, r, p, nullptr);
+  if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, !(o->flags & PK_FLAG_NO_TMA), s))) return e;
   if ((e = T.end())) return e;
   k_zero_x<<<G, kBlock, 0, s>>>(ra, xd);
   launches += 2;
@@ -694,9 +727,24 @@ pk_status launch_spmv_tma(pk_csr* A, const double* x, double* y, int first, int 
   return PK_OK;
 }
 
-void launch_residual_init(const pk_csr* A, const double* b, const double* x, double* r,
-                          double* p, double* r0s, cudaStream_t s) {
-  k_residual_init<<<A->grid, kBlock, 0, s>>>(row_args(A), b, x, r, p, r0s);
+// Whether a solve's setup product runs on the CSR tiles: where they fill most SMs, or where some rows
+// take several lanes.  Measured (us, tiles / a thread per row): 64^2 11.8 / 12.0, 24^3 14.0 / 12.1, 300^2
+// 14.3 / 15.6, 48^3 16.4 / 19.0, 64^3 19.3 / 30.5, 100^3 36.9 / 47.8; power law 10^4 rows 26.9 / 74.3,
+// 10^5 33.3 / 108.
+static bool setup_on_tiles(const pk_csr* A) { return A->tma_ok && (A->grid_tma >= 128 || csr_irregular(A)); }
+
+pk_status launch_residual_init(const pk_csr* A, const double* b, const double* x, double* r, double* p, double* r0s,
+                               bool tma, cudaStream_t s) {
+  if (tma && setup_on_tiles(A)) {
+    if (pk_status e = tma_setup()) return e;
+    (csr_irregular(A) ? k_residual_init_tma<true> : k_residual_init_tma<false>)<<<A->grid_tma, kTileThreads,
+                                                                                 csr_smem_bytes(), s>>>(
+        csr_tiles_of(A), b, x, r, p, r0s, A->partials, A->st);
+  } else {
+    k_residual_init<<<A->grid, kBlock, 0, s>>>(row_args(A), b, x, r, p, r0s);
+  }
+  PK_CUDA(cudaGetLastError());
+  return PK_OK;
 }
 
 void launch_zero_x(const pk_csr* A, double* x, cudaStream_t s) {

@@ -461,8 +461,10 @@ void launch_true_residual(pk_csr* A, const double* b, const double* x, double* t
                           double* out2, cudaStream_t s);
 RowArgs row_args(const pk_csr* A);
 
-void launch_residual_init(const pk_csr* A, const double* b, const double* x, double* r,
-                          double* p, double* r0s, cudaStream_t s);
+// r0 = b - A x0 (to r, and p, r0s where given), <r0, r0>, <b, b> and the state that follows from them;
+// tma: the tile engine may be used.
+pk_status launch_residual_init(const pk_csr* A, const double* b, const double* x, double* r, double* p, double* r0s,
+                               bool tma, cudaStream_t s);
 void launch_zero_x(const pk_csr* A, double* x, cudaStream_t s);
 pk_status check_opts(const pk_csr* A, const double* b, double* x, const pk_opts* o,
                      pk_info* info);
