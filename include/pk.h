@@ -188,10 +188,10 @@ typedef struct {
  * preconditioner fusion as the method's extension).
  * CG: pipelined FP64 CG (Alg. 2 with the preconditioned
  * inner products <r, M^-1 r> and <Ap, M^-1 Ap>; beta = alpha^2 <Ap, M^-1 Ap>/<r, M^-1 r> - 1)
- * on the graph or host loop; the fused SpMV kernel forms Ap, <p, Ap>, <Ap, M^-1 Ap>, the
+ * on the graph or host loop, or (PK_LOOP_AUTO) with the matrix in shared memory; the fused SpMV kernel forms Ap, <p, Ap>, <Ap, M^-1 Ap>, the
  * update kernel x, r, p = M^-1 r + beta p, <r, M^-1 r> and <r, r>.  The stopping test stays
  * ||r|| <= tol ||b||.  A diagonal entry <= 0 returns PK_NOT_SPD.  Other variants, precisions
- * and the persistent loop return PK_ERR_ARG (PK_LOOP_AUTO uses the graph loop).
+ * and the persistent loop return PK_ERR_ARG (PK_LOOP_AUTO: see there).
  * BiCGStab and GMRES (both variants): right preconditioning.  The solver runs unchanged on
  * A M^-1 y = b, whose residual is b - A x for x = M^-1 y, so the stopping test and the trace
  * are those of the plain solver on A M^-1; the values of A M^-1 (columns scaled by the
@@ -240,7 +240,7 @@ typedef struct {
   int32_t kernel;            /* SpMV engine: 0 thread-per-row loads, 2 warp-specialised bulk-copy tiles */
   int32_t values_fp32_exact; /* 1 if every value is exactly representable in float32 */
   /* bulk-copy tiles by row schedule: every row one thread (tiles_thread: rows short enough
-   * for one thread to walk); short rows one thread and long rows a whole warp each
+   * for one thread to walk); every row the lanes its length asks for, longest first
    * (tiles_long: rows of very different lengths); rows of similar length G = 2..16 lanes each
    * (tiles_group).  The chunk tiles of a row longer than a tile (4096 nonzeros), summed by
    * the whole block, count in tiles_long too: ceil(length / 4096) per such row */
@@ -345,24 +345,26 @@ pk_status pk_gmres_cycle_factors(const pk_csr* A, int32_t m, double* R, double* 
  * must be DEVICE pointers.  opts: tol, maxit (per system; MIXED: total inner iterations),
  * precision PK_PREC_FP64 or PK_PREC_MIXED (FP32 SpMV/vectors inside FP64 iterative
  * refinement, inner tolerance 1e-4, at most 20 refinement steps), lanes, wait_ns, flags
- * PK_FLAG_AUTOTUNE.  Two engines:
- *   - the row engine (default): plain row loops, lanes = 1, 2, 4 or 8 lanes per row (0 = from
- *     the batch's mean row length), FP64 or MIXED;
+ * PK_FLAG_AUTOTUNE.  lanes = 0 (default): the cluster engine for FP64 batches whose systems have at
+ * most 65536 rows and whose rows have at most 12 nonzeros on average, with CTAs of 512 threads (2 per
+ * SM) and as many rows per CTA as still fill the device; else the row engine with lanes from the mean
+ * row length.  The engines:
+ *   - the row engine: plain row loops, lanes = 1, 2, 4 or 8 lanes per row, FP64 or MIXED;
  *   - lanes = -1, FP64, every system with CSR tiles: the tile engine -- each block (288
  *     threads, 2 per SM) streams its system's CSR tiles and vectors through shared memory with
  *     bulk copies, as the single-system kernels do (bounded waits: PK_TIMEOUT).  Measured
  *     slower than the row engine on small systems (18 resident warps per SM against 64 hide
  *     less of the gather latency), so it is an option and a candidate of the tuner;
  *   - lanes = -2, FP64, every system of at most 65536 rows: the cluster engine -- a system of
- *     n rows is solved by a thread-block cluster of C = 1, 2, 4, 8 or 16 CTAs holding p, x, r
+ *     n rows is solved by a thread-block cluster of C = 1, 2, 4, 8 or 16 CTAs holding p, r
  *     and Ap in the CTAs' shared memory, the SpMV gathering p across the cluster (distributed
  *     shared memory), so that per iteration only the matrix is read from global memory.  CTA
- *     shapes: 256 threads and up to 2048 rows (2 per SM), the smallest C with C * 2048 >= n;
- *     systems of more than 32768 rows on CTAs of 512 threads and up to 4096 rows (1 per SM).
+ *     shapes: 256 threads and up to 2048 rows, the smallest C with C * 2048 >= n; systems of more
+ *     than 32768 rows on CTAs of 512 threads and up to 4096 rows.
  *     One persistent cluster launch per (shape, C) class, the launches on streams of their
  *     own that join the caller's stream.
  * PK_FLAG_AUTOTUNE (lanes 0) times the tile engine and the cluster engine (FP64, the cluster
- * engine aiming at 1024, 2048 and 4096 rows per CTA: CTAs of 128, 256, 512 threads) and every
+ * engine as lanes = 0 plans it, and at 1024, 2048 and 4096 rows per CTA: CTAs of 128, 256, 512 threads) and every
  * (block size, blocks per SM, lanes per row) of the row engine on the batch, each solving the
  * whole batch to tol / maxit from x as given (x is restored after each), and keeps the
  * fastest (cached per batch shape and precision for the process).  PK_FLAG_SELL, PK_FLAG_CGS2 and a
@@ -375,8 +377,8 @@ pk_status pk_batched_solve(int32_t nsys, pk_csr* const* A, const double* const* 
                            double* const* x, const pk_opts* opts, pk_info* infos, void* stream);
 
 /* Block size and blocks per SM used by the last pk_batched_solve call in this process
- * (the cluster engine: the CTA shape of its default or tuned rows per CTA, e.g. 256 threads and
- * 2 blocks per SM for 2048 rows). */
+ * (the cluster engine: 512 and 2 as lanes = 0 plans it, else the CTA shape of its rows per CTA, e.g.
+ * 256 threads and 2 blocks per SM for 2048 rows). */
 pk_status pk_batched_last_config(int32_t* block, int32_t* blocks_per_sm);
 
 /* Lanes per row (1, 2, 4 or 8) that the last pk_batched_solve call ran with; -1 = the tile

@@ -511,7 +511,7 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
   int launches = 0;
   const RowArgs ra = row_args(A);
   const CsrTiles ct = csr_tiles_of(A);
-  const bool irr = csr_irregular(A);  // some tile needs the grouped or whole-warp rows
+  const bool irr = csr_irregular(A);  // some tile needs several lanes per row
   const int G = A->grid, Gt = A->grid_tma, Gs = A->grid_stream, n = A->n;
   double* part = A->partials;
   DevState* dst = A->st;

@@ -392,13 +392,13 @@ static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, i
     if (!tile_z0.empty()) tile_z0.resize(P.ntiles, -1);
   }
   // per tile, the lanes that compute one row (see csr_tiles): 1 = one thread per row (two rows
-  // per thread, in one pass), 2..16 = a group of lanes per row, 32 = short rows one thread and
-  // rows longer than 32 nonzeros a whole warp each, in a length-sorted row order.  A tile
+  // per thread, in one pass), 2..16 = a group of lanes per row, 32 = rows in a length-sorted order,
+  // longest first, each with the lanes its length asks for (sorted_rows).  A tile
   // holds at most kTileNnz nonzeros, so long rows mean few rows per tile: with one thread per
   // row most consumer threads would idle.  The group size minimises the rounds of (at most 8)
   // dependent gathers a lane waits for: ceil(rows G / consumers) rows one after the other,
   // each ceil(lmax / 8 G) batches.  Tiles whose longest row is far above their mean (power-law
-  // rows) take the sorted whole-warp schedule instead.
+  // rows) take the sorted schedule instead.
   auto tile_lanes = [&](int64_t rows, int64_t lmax, int64_t z) -> int {
     if (lmax <= 8) return 1;
     const double mean = (double)z / (double)rows;
@@ -425,9 +425,8 @@ static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, i
     (tile_grp[t] == 1 ? P.tiles_thread : tile_grp[t] == 32 ? P.tiles_long : P.tiles_group) += 1;
   }
   // row order of every irregular tile: rows sorted by length (longest first), dealt
-  // round-robin over the 8 consumer warps -- slot (warp w, lane l) takes sorted rows
-  // 8 l + w and 256 + 8 l + w -- so that each warp holds rows of similar length and the
-  // long rows spread over all warps; -1 marks an empty slot
+  // round-robin over the 8 consumer warps -- slot (warp w, lane l) holds sorted rows
+  // 8 l + w and 256 + 8 l + w (sorted_rows reads them back in order); -1 marks an empty slot
   auto& tile_perm = P.tile_perm;
   if (P.tiles_long > 0) {
     tile_perm.assign((size_t)P.ntiles * kTileRows, (int16_t)-1);

@@ -524,8 +524,8 @@ __device__ __forceinline__ double sell_row(const SellArgs& s, int64_t base, int 
   return acc;
 }
 
-// Kernels on the CSR tile engine take the instantiation with the grouped and whole-warp row
-// paths when some tile needs one of them.
+// Kernels on the CSR tile engine take the instantiation with the paths of several lanes per row
+// when some tile needs one of them.
 // Systems whose update kernel takes the tile blocks' rows (blk_row) instead of equal chunks: the
 // ones that a shared-memory-resident loop may run, so that both sum in the same order.
 constexpr int kSmMaxRows = 655360;  // (the plan's column bitmap fits shared memory)

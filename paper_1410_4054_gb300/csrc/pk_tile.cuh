@@ -330,7 +330,7 @@ struct CsrTilesT {
   const VT* va;             // values: FP64, or the FP32 copy for the mixed-precision inner loop
   const int32_t* tile_row;  // row start of every tile (global tile list), plus n at the end
   const int32_t* blk_tile;  // tiles of block b: [blk_tile[b], blk_tile[b+1])
-  const int8_t* tile_grp;   // 1: every row of the tile has at most kLongRow nonzeros
+  const int8_t* tile_grp;   // 1: a thread per row; 2..16: lanes per row; 32: sorted_rows; 64: a chunk
   const int16_t* tile_perm; // [tile][512]: row (offset in the tile) of every consumer slot, or -1
   const int32_t* tile_z0;   // chunk tiles (tile_grp 64): first nonzero of the chunk, else -1
 };
@@ -421,12 +421,11 @@ __device__ __forceinline__ void row_pair(const float* sva, const CI* sci, int ja
 // Runs the CSR pipeline and the row products y_row = sum_j A[row][j] x[col j]; every finished
 // row goes to `row_done(row, y_row)`, called by the one consumer thread that owns the row.
 // Consumer thread t computes rows R0 + t and R0 + t + 256 of every tile itself (summed left
-// to right, the order of a plain CSR loop).  In tiles that hold rows longer than kLongRow
-// nonzeros (T.tile_grp != 1, set at pk_csr_create) a thread skips its long rows, and each
-// warp then takes its lanes' long rows one at a time with all 32 lanes (lane l sums entries
-// l, l + 32, ... left to right, then a butterfly), so that no thread walks a long row alone;
-// no synchronisation beyond the warp is involved.  Tiles of rows of similar length that are
-// too long for one thread (T.tile_grp = G in 2..16) give each row a group of G lanes instead.
+// to right, the order of a plain CSR loop).  Tiles of rows of similar length that are too long for
+// one thread (T.tile_grp = G in 2..16, set at pk_csr_create) give each row a group of G lanes
+// instead; tiles of very different row lengths, some beyond kLongRow nonzeros (T.tile_grp = 32), take
+// their rows longest first with as many lanes as their length asks for (sorted_rows).  No
+// synchronisation beyond the warp is involved.
 // A row longer than a tile is cut into chunk tiles of kTileNnz nonzeros (T.tile_grp = 64,
 // consecutive tiles of one block) and summed by the whole block: see block_row_chunk.
 constexpr int kLongRow = 32;
@@ -476,14 +475,66 @@ __device__ __forceinline__ void block_row_chunk(int row, int zc0, int zr1, VT* s
   }
 }
 
+// The rows of a tile that holds rows of very different lengths, longest first (sperm: see
+// pk_csr_create), by the whole block: a round takes the next 256 / G rows with G lanes each, G such
+// that the longest of them, the first, is at most kLaneEntries entries per lane (32 lanes at most), so
+// that rounds are short and every warp has as much to do.  A lane adds its entries left to right, the
+// lanes by a butterfly.  Before, a thread walked a row of up to 32 entries and a warp took the longer
+// ones in turn: on a power-law matrix of 10^5 rows (3 to 256 entries, 341 rows per block) a product
+// took 32,000 clocks in the slowest block (24,500 in the median) with the gathered vector in shared
+// memory, now 23,000 (17,000); its FP64 work is 4,100.  BiCGStab there 65 -> 53 us per iteration, with
+// launched kernels 70 -> 60; CG 28 -> 22 and 33 -> 29; GMRES 36 -> 31 and 71 -> 67.
+constexpr int kLaneEntries = 8;
+
+template <class VT, class CI, class XP, class RowDone>
+__device__ __forceinline__ void sorted_rows(const int16_t* sperm, const int32_t* srp, const VT* sva, const CI* sci,
+                                            int R0, int R1, XP x, RowDone& row_done) {
+  constexpr int B = GatherShared<XP>::value ? 4 : 8;  // entries in flight per lane
+  const int nr = R1 - R0;
+  // sorted position -> slot of sperm (dealt over the warps)
+  auto row_at = [&](int k) { return R0 + sperm[(k & 256) | ((k & 7) << 5) | ((k & 255) >> 3)]; };
+#pragma unroll 1
+  for (int pos = 0; pos < nr;) {
+    const int first = row_at(pos), len = srp[first + 1] - srp[first];
+    int lg = 0;
+    while (lg < 5 && (kLaneEntries << lg) < len) ++lg;
+    const int k = pos + ((int)threadIdx.x >> lg), q = (int)threadIdx.x & ((1 << lg) - 1);
+    const bool live = k < nr;
+    const int r = live ? row_at(k) : R0;
+    int j = live ? srp[r] + q : 0;
+    const int j1 = live ? srp[r + 1] : 0;
+    VT s = (VT)0;
+    for (;;) {
+      const int m = j < j1 ? min(B, (j1 - j + (1 << lg) - 1) >> lg) : 0;
+      const int mx = __reduce_max_sync(0xffffffffu, m);
+      if (mx == 0) break;
+      VT v[B], xv[B];
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        v[u] = u < m ? sva[j + (u << lg)] : (VT)0;
+        xv[u] = u < m ? gather(x, sci[j + (u << lg)]) : (VT)0;
+      }
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (u < mx) {  // (uniform: a predicated-off FP64 instruction still takes a slot of the pipe)
+          if (u < m) s = fma_t(v[u], xv[u], s);
+        }
+      j += B << lg;
+    }
+#pragma unroll 1
+    for (int o = (1 << lg) >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (live && q == 0) row_done(r, s);
+    pos += kConsumers >> lg;
+  }
+}
+
 // The row products of one tile, rows [R0, R1), from shared memory: srp[row] is the index of the
 // row's first entry in sva / sci; G is the tile's schedule (1: a thread per row; 2 .. 16: G lanes
-// per row; 32: whole warps for the long rows, with the row order sperm if there is one).  Called
-// by the kConsumers consumer threads together; row_done(row, y) runs in one thread per row.
+// per row; 32: sorted_rows in the row order sperm).  Called by the kConsumers consumer threads
+// together; row_done(row, y) runs in one thread per row.
 template <bool IRR, class VT, class CI, class XP, class RowDone>
 __device__ __forceinline__ void tile_rows(int R0, int R1, int G, const int16_t* sperm, const int32_t* srp,
                                           const VT* sva, const CI* sci, XP x, RowDone& row_done) {
-  const int lane = threadIdx.x & 31;
   if (!IRR || G == 1) {
     const int ra = R0 + (int)threadIdx.x;
     if (ra < R1) {
@@ -506,37 +557,7 @@ __device__ __forceinline__ void tile_rows(int R0, int R1, int G, const int16_t* 
       }
     }
   } else {
-    // every lane takes part (the ballots below need the whole warp).  With a row order
-    // (sorted by length, dealt round-robin over the warps) each warp holds rows of similar
-    // length, so its FMA batches carry few idle lanes.
-    const int ka = sperm ? sperm[threadIdx.x] : (int)threadIdx.x;
-    const int kb = sperm ? sperm[threadIdx.x + kConsumers] : (int)threadIdx.x + kConsumers;
-    const int ra = ka >= 0 && R0 + ka < R1 ? R0 + ka : -1;
-    const int rb = kb >= 0 && R0 + kb < R1 ? R0 + kb : -1;
-    int ja0 = ra >= 0 ? srp[ra] : 0, ja1 = ra >= 0 ? srp[ra + 1] : 0;
-    int jb0 = rb >= 0 ? srp[rb] : 0, jb1 = rb >= 0 ? srp[rb + 1] : 0;
-    const bool la = ja1 - ja0 > kLongRow, lb = jb1 - jb0 > kLongRow;
-    if (ra >= 0 || rb >= 0) {
-      VT sa, sb;
-      row_pair(sva, sci, ja0, la ? ja0 : ja1, jb0, lb ? jb0 : jb1, x, sa, sb);
-      if (ra >= 0 && !la) row_done(ra, sa);
-      if (rb >= 0 && !lb) row_done(rb, sb);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      unsigned pending = __ballot_sync(0xffffffffu, h == 0 ? la : lb);
-      while (pending) {
-        const int src = __ffs(pending) - 1;
-        pending &= pending - 1;
-        const int r = __shfl_sync(0xffffffffu, h == 0 ? ra : rb, src);
-        const int j0 = srp[r], j1 = srp[r + 1];
-        VT acc = (VT)0;
-        for (int j = j0 + lane; j < j1; j += 32) acc = fma_t(sva[j], gather(x, sci[j]), acc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == src) row_done(r, acc);
-      }
-    }
+    sorted_rows(sperm, srp, sva, sci, R0, R1, x, row_done);
   }
 }
 
