@@ -430,15 +430,18 @@ static void build_plan(int64_t n, int64_t nnz, const std::vector<int32_t>& rp, i
   auto& tile_perm = P.tile_perm;
   if (P.tiles_long > 0) {
     tile_perm.assign((size_t)P.ntiles * kTileRows, (int16_t)-1);
-    std::vector<int32_t> order;
+    std::vector<int32_t> order, at;
     for (int t = 0; t < P.ntiles; ++t) {
       if (tile_grp[t] != 32) continue;
       const int32_t R0 = tile_row[t], m = tile_row[t + 1] - R0;
+      // by counting: lengths are at most kTileNnz (a comparison sort was most of the plan's time)
+      int32_t lmax = 0;
+      for (int k = 0; k < m; ++k) lmax = std::max(lmax, rp[R0 + k + 1] - rp[R0 + k]);
+      at.assign(lmax + 2, 0);
+      for (int k = 0; k < m; ++k) ++at[lmax - (rp[R0 + k + 1] - rp[R0 + k]) + 1];
+      for (int l = 0; l <= lmax; ++l) at[l + 1] += at[l];
       order.resize(m);
-      for (int k = 0; k < m; ++k) order[k] = k;
-      std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-        return rp[R0 + a + 1] - rp[R0 + a] > rp[R0 + b + 1] - rp[R0 + b];
-      });
+      for (int k = 0; k < m; ++k) order[at[lmax - (rp[R0 + k + 1] - rp[R0 + k])]++] = k;
       int16_t* P = tile_perm.data() + (size_t)t * kTileRows;
       for (int tid = 0; tid < kTileRows / 2; ++tid) {
         const int w = tid / 32, l = tid % 32;
