@@ -380,14 +380,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
 // per thread, took 560 clocks of issue per step.)  Two warps issue the MMAs of every other output row,
 // each into accumulators of its own (one warp's waits and issue took 1,000 clocks per row).  Runs have
 // at most kWgRun rows: two run buffers alternate, and four buffers of G (its three dx shifts) rotate.
+// One more warp sums the block's part of db from global memory, over segments b, b + G, b + 2 G, ... of
+// the whole grid instead of the rows that the block multiplies.  G of a loss sums to nearly nothing over
+// the grid and is smooth along it: the sum over a run of neighbouring rows is large and of one sign, over
+// rows from everywhere it has cancelled already, and what the block sums are rounded to is what db is off
+// by.  (Runs of rows moved db of the last layer by up to 6e-5 of itself against these sums, in the worst of
+// 400 random boxes of 12 to 72 voxels a side.)
 // Every wait is bounded (a wait that runs out sets the device flag that pk_conv3d_check reports, and
 // the block waits, bounded, for what it issued before it frees its tensor memory).  At the end each
 // thread reads its accumulator lane into the block's partial; a fixed-order reduction over blocks
 // follows.
-// Measured with that reduction (64^3, launches back to back): 33.0 us before (an im2col operand per
-// 64-voxel segment), 22.9 us now; 72^3 (two segments per row, the second mostly empty): 69.0 -> 41.9;
-// 32^3: 14.7 -> 14.5.  The rest is issue and wait latency: tensor pipe and memory are idle for most
-// of it.
+// Measured with that reduction (64^3, launches back to back with programmatic launches): 32.9 us before
+// (an im2col operand per 64-voxel segment, plain launches), 17.5 us now; 72^3 (two segments per row, the
+// second mostly empty): 68.7 -> 34.6; 32^3: 14.4 -> 11.4.  The rest is issue and wait latency: tensor pipe
+// and memory are idle for most of it.
 constexpr int kWgSeg = 64;                       // voxels (K) per segment
 constexpr int kWgRun = 10;                       // output rows per run
 constexpr int kWgSlots = kWgRun + 2;             // y rows of A per run
@@ -407,6 +413,9 @@ constexpr uint32_t kWgCols = 128 * kWgMma;       // tensor memory: 48 columns at
 constexpr int kWgWarps = 8;                      // warps that write a step's operands
 constexpr int kWgGroups = 2;                     // groups of them, fill steps in turn
 constexpr int kWgThreads = 32 * kWgWarps * kWgGroups;
+constexpr int kWgBlock = kWgThreads + 32 * (2 + kWgMma);  // ... the loader warp, the MMA warps, the warp of db
+constexpr int kWgDbRows = 16;                    // chains of db per channel
+static_assert(kWgDbRows * kCh == 32 * 8 && kWgSeg % kWgDbRows == 0, "a lane of the db warp: 8 channels of a chain");
 // A group's steps with an output row are every other row, the rows of one MMA warp, and an even number
 // of G buffers keeps a buffer with that pair: its phases complete in order, and no wait can take the
 // phase before the last for the one it needs.
@@ -450,10 +459,41 @@ struct WgSteps {
   }
 };
 
-__global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wgrad_tc(const __grid_constant__ CUtensorMap amap,
-                                                                        const __grid_constant__ CUtensorMap gmap,
-                                                                        float* partial, float* partial_db, int D,
-                                                                        int H, int W) {
+// The block's part of db, in one warp: chain i = 0 .. 15 of a channel adds voxels i, i + 16, i + 32, i + 48
+// of segments b, b + G, ... (unit numbers (z, y, segment), the segment fastest) one after the other.  A
+// lane holds 8 channels of a chain, so a load of the warp is 16 voxels, 512 bytes.  One segment in flight:
+// the warp keeps pace with the MMAs (1,100 clocks a row), and two or four in flight raise the kernel's
+// registers from 54 to 80 and 96 (64^3: 17.5, 17.6 and 18.3 us; the sums in the writer warps 18.5).
+__device__ __forceinline__ void wg_db(const __nv_bfloat16* G, int D, int H, int W, float (*dbs)[kCh]) {
+  const int lane = threadIdx.x & 31, i = lane >> 1, c8 = 8 * (lane & 1);
+  const int nseg = (W + kWgSeg - 1) / kWgSeg;
+  const int64_t units = (int64_t)nseg * D * H;
+  float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+  for (int64_t c = blockIdx.x; c < units; c += gridDim.x) {
+    const int64_t zy = c / nseg;
+    const int x0 = (int)(c - zy * nseg) * kWgSeg + i;
+    uint4 g[kWgSeg / kWgDbRows];
+#pragma unroll
+    for (int k = 0; k < kWgSeg / kWgDbRows; ++k)
+      g[k] = x0 + kWgDbRows * k < W
+                 ? __ldcg(reinterpret_cast<const uint4*>(G + (zy * W + x0 + kWgDbRows * k) * kCh + c8))
+                 : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int k = 0; k < kWgSeg / kWgDbRows; ++k) {
+      const __nv_bfloat16* v = reinterpret_cast<const __nv_bfloat16*>(&g[k]);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) db[q] += __bfloat162float(v[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) dbs[i][c8 + q] = db[q];
+}
+
+__global__ void __launch_bounds__(kWgBlock, 1) k_conv3d_wgrad_tc(const __grid_constant__ CUtensorMap amap,
+                                                                 const __grid_constant__ CUtensorMap gmap,
+                                                                 const __nv_bfloat16* G, float* partial,
+                                                                 float* partial_db, int D, int H, int W) {
   extern __shared__ __align__(1024) unsigned char smem_wg[];
   __shared__ __align__(8) uint64_t full_bar[kWgStages];  // staging buffer loaded
   __shared__ __align__(8) uint64_t empty_bar[kWgStages]; // staging buffer read (8 warps)
@@ -462,7 +502,7 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
   __shared__ __align__(8) uint64_t afree_bar[2];         // a run buffer is read
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ float dbs[kWgThreads / kCh][kCh];
+  __shared__ float dbs[kWgDbRows][kCh];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nseg = (W + kWgSeg - 1) / kWgSeg;
   const int units = nseg * D * H;  // (< 2^31: checked by the host)
@@ -490,7 +530,9 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
   volatile int* const stop = &abort_flag;
   griddep_wait();  // nothing in memory is read or written before
   WgSteps step(units, D, H);
-  if (warp > kWgThreads / 32) {
+  if (warp == kWgBlock / 32 - 1) {
+    wg_db(G, D, H, W, dbs);
+  } else if (warp > kWgThreads / 32) {
     // MMA warps: per output row 4 x 2 MMAs
     const int me = warp - kWgThreads / 32 - 1;
     const uint32_t acc = tmem + 128 * me;
@@ -563,9 +605,6 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
     const int vox = (kg + (lane >> 3)) * 8 + (lane & 7);
     const uint32_t dst = h * 1024 + (kg + (lane >> 3)) * 128 + (lane & 7) * 16;
     const uint32_t src = base + 2 * kWgA + kWgGs * kWgG + h * 16 + (vox + 1) * 32;  // (voxel -1 comes first)
-    constexpr int kWgDb = 2 * kWgWarps;
-    float db = 0.f;  // output channel t % 16 over voxels t / 16 % 16 + 16 k of the group's rows of G
-    const int dc = threadIdx.x & (kCh - 1);
     int f = 0, j = 0;
     for (; step.next(); j += step.t >= 2, ++f) {
       if (f % kWgGroups != grp) continue;
@@ -598,13 +637,6 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
         if (g) stsm4(gb, r[1]);
         if (g) stsm4(gb + 2 * kWgRowOp, r[2]);
       }
-      if (g) {
-        const __nv_bfloat16* g16 = reinterpret_cast<const __nv_bfloat16*>(smem_wg + 2 * kWgA + kWgGs * kWgG +
-                                                                           sb * kWgStage + kWgStageG + 32);
-#pragma unroll
-        for (int xx = (threadIdx.x / kCh) % kWgDb; xx < kWgSeg; xx += kWgDb)
-          db += __bfloat162float(g16[xx * kCh + dc]);
-      }
       proxy_fence();  // the operands are read by the tensor core (async proxy)
       __syncwarp();
       if (lane == 0) {
@@ -612,7 +644,6 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
         mbar_arrive(&empty_bar[sb]);
       }
     }
-    dbs[threadIdx.x / kCh][dc] = db;
   }
   tc_fence_before();
   __syncthreads();
@@ -647,7 +678,7 @@ __global__ void __launch_bounds__(kWgThreads + 32 * (1 + kWgMma), 1) k_conv3d_wg
     }
     if (threadIdx.x < kCh) {
       float t = 0.f;
-      for (int k = 0; k < kWgThreads / kCh; ++k) t += dbs[k][threadIdx.x];
+      for (int k = 0; k < kWgDbRows; ++k) t += dbs[k][threadIdx.x];
       partial_db[blockIdx.x * kCh + threadIdx.x] = t;
     }
   } else if (abort_flag && threadIdx.x == 0) {
@@ -1184,7 +1215,8 @@ pk_status pk_conv3d_wgrad(const void* A, const void* G, float* scratch, float* d
   CUtensorMap amap, gmap;
   if ((e = input_map(&amap, static_cast<const __nv_bfloat16*>(A), D, H, W, kCh, kWgSeg + 2, 1, 3))) return e;
   if ((e = input_map(&gmap, static_cast<const __nv_bfloat16*>(G), D, H, W, kCh, kWgSeg + 2, 1, 1))) return e;
-  launch_pdl(k_conv3d_wgrad_tc, nblk, kWgThreads + 32 * (1 + kWgMma), kWgSmem, s, amap, gmap, partial, partial_db, D, H, W);
+  launch_pdl(k_conv3d_wgrad_tc, nblk, kWgBlock, kWgSmem, s, amap, gmap, static_cast<const __nv_bfloat16*>(G), partial,
+             partial_db, D, H, W);
   launch_pdl(k_conv3d_wgrad_reduce, (27 * kCh * kCh + kCh + 31) / 32, 256, 0, s, (const float*)partial,
              (const float*)partial_db, nblk, dW, db);
   PK_CUDA(cudaGetLastError());
