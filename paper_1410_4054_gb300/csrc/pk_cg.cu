@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "pk_guard.cuh"
 #include "pk_sm.cuh"
 
 namespace pk {
@@ -755,5 +756,5 @@ void launch_zero_x(const pk_csr* A, double* x, cudaStream_t s) {
 
 extern "C" pk_status pk_cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* opts,
                                  pk_info* info, void* stream) {
-  return pk::cg_solve(A, b, x, opts, info, (cudaStream_t)stream);
+  return pk::guarded([&] { return pk::cg_solve(A, b, x, opts, info, (cudaStream_t)stream); });
 }

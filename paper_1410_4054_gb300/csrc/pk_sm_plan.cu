@@ -5,6 +5,7 @@
 #include <atomic>
 #include <vector>
 
+#include "pk_guard.cuh"
 #include "pk_sm.cuh"
 
 namespace pk {
@@ -140,10 +141,15 @@ pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable) {
   PK_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, A->device));
   PK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device));
   if (!coop || A->grid_tma > 2 * sms) return PK_OK;
-  pk_status e = sm_tiles(A, sms, s);
-  if (!e) e = build(A, s);
+  // (guarded here and not only at the entry: a failed host allocation is no reason to fail the solve)
+  const pk_status e = guarded([&]() -> pk_status {
+    const pk_status t = sm_tiles(A, sms, s);
+    return t ? t : build(A, s);
+  });
   if (e == PK_ERR_OOM) {  // no memory for the plan: the launched loop needs none
     cudaGetLastError();
+    if (A->sm_own) cudaFree(A->sm_own);
+    A->sm_own = nullptr;
     A->sm_state = -1;
     return PK_OK;
   }
