@@ -19,6 +19,7 @@
 #include <mutex>
 #include <vector>
 
+#include "pk_batched_plan.h"
 #include "pk_guard.cuh"
 #include "pk_tile.cuh"
 
@@ -531,33 +532,14 @@ static std::map<TuneKey, TuneVal> g_tune;
 static TuneVal g_last{512, 2, 1, 0};
 
 // The cluster engine (pk_batched_cluster.cu): classes are (CTA shape, cluster size) pairs.
-constexpr int kClSizes = 5;  // clusters of 1, 2, 4, 8, 16 CTAs
 constexpr int kClClasses = kBcShapeCount * kClSizes;
 constexpr int kClRowsDefault = 2048;
 
-// What the automatic choice plans: CTAs of shape 0 (512 threads, two per SM) with up to t rows each,
-// half as many for a system of at most 2 t rows; shape 0's log2 of the cluster size.
-static int auto_cluster(int n, int t) {
-  const int rows = n <= 2 * t ? t / 2 : t;
-  int c = 0;
-  while (c + 1 < kClSizes && ((long long)rows << c) < n) ++c;
-  return c;
-}
-
-// Class of a system of n rows when the batch aims at rows_cta rows per CTA: the CTA shape
-// whose row limit is rows_cta, else the next larger one that holds n on 16 CTAs, with the
-// smallest power-of-2 cluster that holds n.  shape * kClSizes + log2(C), or -1.
-static int cluster_class(int n, int rows_cta) {
-  int s0 = -1;
-  for (int sh = 0; sh < kBcShapeCount; ++sh)
-    if (batched_cluster_max_rows(sh) == rows_cta) s0 = sh;
-  for (int sh = s0; sh >= 0; --sh) {  // shape 0 has the largest row limit
-    const long long mx = batched_cluster_max_rows(sh);
-    for (int c = 0; c < kClSizes; ++c)
-      if (mx << c >= n) return sh * kClSizes + c;
-  }
-  return -1;
-}
+struct DeviceLimits {
+  int shapes() const { return kBcShapeCount; }
+  int max_rows(int shape) const { return batched_cluster_max_rows(shape); }
+  int capacity(int shape, int C) const { return batched_cluster_capacity(shape, C); }
+};
 
 // The batch as the cluster engine runs it: systems grouped by class, the classes that hold the
 // most rows per cluster first (within a class, largest systems first); one persistent launch
@@ -570,22 +552,9 @@ struct ClusterPlan {
   int first[kClClasses + 1];    // slot j's systems: [first[j], first[j + 1])
 };
 
-// rows_cta 0: the automatic choice.  An SM takes two CTAs of shape 0, so that one system's reductions
-// and barriers overlap another's FP64 work; t, the rows per CTA, is the largest the CTAs hold as long
-// as the batch fills the device (fewer barriers per row), else smaller (an iteration's latency).
-// The short systems at the end of the queues run on shares half as large: their iterations are the
-// batch's tail.  Measured (512 shifted 2D Laplacians, ms): 256 threads x 2048 rows, two per SM 13.5;
-// this with t everywhere 11.4, halved up to t rows 11.2, up to 2 t rows 10.9, up to 4 t rows 11.4.
-static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterPlan& P) {
+// The plan of the classes cls (pk_batched_plan.h).
+static void plan_clusters(const std::vector<BatchSys>& h, const std::vector<int>& cls, ClusterPlan& P) {
   const int nsys = (int)h.size();
-  int t = batched_cluster_max_rows(0);
-  const int device_ctas = rows_cta == 0 ? batched_cluster_capacity(0, 1) : 0;
-  while (rows_cta == 0 && t > 512) {
-    long long ctas = 0;
-    for (const BatchSys& S : h) ctas += 1ll << auto_cluster(S.n, t);
-    if (ctas >= device_ctas) break;
-    t /= 2;
-  }
   // launch slots: classes by rows per cluster (descending), then by shape
   std::vector<int> slots(kClClasses);
   for (int c = 0; c < kClClasses; ++c) slots[c] = c;
@@ -597,11 +566,7 @@ static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterP
     slot_of[slots[j]] = j;
   }
   std::vector<int> sl(nsys);
-  for (int k = 0; k < nsys; ++k) {
-    const int c = rows_cta == 0 ? auto_cluster(h[k].n, t) : cluster_class(std::max(h[k].n, 1), rows_cta);
-    if (c < 0 || batched_cluster_capacity(c / kClSizes, 1 << (c % kClSizes)) <= 0) return false;
-    sl[k] = slot_of[c];
-  }
+  for (int k = 0; k < nsys; ++k) sl[k] = slot_of[cls[k]];
   P.order.resize(nsys);
   for (int k = 0; k < nsys; ++k) P.order[k] = k;
   std::stable_sort(P.order.begin(), P.order.end(), [&](int a, int c) {
@@ -616,7 +581,6 @@ static bool plan_clusters(const std::vector<BatchSys>& h, int rows_cta, ClusterP
   }
   P.first[0] = 0;
   for (int j = 0; j < kClClasses; ++j) P.first[j + 1] = P.first[j] + count[j];
-  return true;
 }
 
 // The class streams and events are shared by every caller: a batch is enqueued under the mutex
@@ -779,10 +743,15 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
     return PK_ERR_ARG;
   }
   ClusterPlan plan;
+  const DeviceLimits dev_limits;
   const int max_cl_rows = 16 * batched_cluster_max_rows(0);
-  bool clusters_ok = !mixed;
-  for (int k = 0; k < nsys && clusters_ok; ++k) clusters_ok = h[k].n <= max_cl_rows;
-  if (clusters_ok) clusters_ok = plan_clusters(h, kClRowsDefault, plan);
+  std::vector<int> sizes(nsys), cls(nsys);
+  bool cluster_sizes = !mixed;  // FP64 systems that some cluster could hold
+  for (int k = 0; k < nsys; ++k) {
+    sizes[k] = h[k].n;
+    cluster_sizes = cluster_sizes && h[k].n <= max_cl_rows;
+  }
+  const bool clusters_ok = cluster_sizes && cluster_classes(dev_limits, sizes.data(), nsys, kClRowsDefault, cls.data());
   if (o->lanes == -2 && !clusters_ok) {
     set_error("lanes = -2: the cluster engine runs FP64 batches of systems of at most 65536 rows");
     return PK_ERR_ARG;
@@ -797,10 +766,11 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
   // the row kernel's lanes.
   const TuneVal cluster_cfg{kClRowsDefault / 8, 4096 / kClRowsDefault, -2, kClRowsDefault};
   const TuneVal cluster_auto{512, 2, -2, 0};
-  TuneVal cfg = o->lanes == -1                                          ? TuneVal{kTileThreads, 2, -1, 0}
-                : o->lanes == -2                                        ? cluster_cfg
-                : o->lanes == 0 && clusters_ok && lanes_auto == 1 ? cluster_auto
-                                                                    : TuneVal{512, 2, o->lanes ? o->lanes : lanes_auto, 0};
+  const TuneVal row_cfg{512, 2, o->lanes > 0 ? o->lanes : lanes_auto, 0};
+  TuneVal cfg = o->lanes == -1                                      ? TuneVal{kTileThreads, 2, -1, 0}
+                : o->lanes == -2                                    ? cluster_cfg
+                : o->lanes == 0 && cluster_sizes && lanes_auto == 1 ? cluster_auto
+                                                                    : row_cfg;
   const TuneKey key{nsys, rows, nnz, mixed};
   bool have = false;
   if (o->lanes == 0) {
@@ -808,7 +778,7 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
     auto it = g_tune.find(key);
     if (it != g_tune.end()) { cfg = it->second; have = true; }
   }
-  if (have && ((cfg.lanes == -1 && !tiles_ok) || (cfg.lanes == -2 && !clusters_ok))) {
+  if (have && ((cfg.lanes == -1 && !tiles_ok) || (cfg.lanes == -2 && !cluster_sizes))) {
     cfg = TuneVal{512, 2, lanes_auto, 0};  // tuned on handles that allowed that engine
     have = false;
   }
@@ -852,10 +822,11 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
         if (rep == 1 && ms < best) { best = ms; cfg = TuneVal{kTileThreads, 2, -1, 0}; }
       }
     }
-    if (clusters_ok && o->lanes == 0) {  // the cluster engine as planned, and at 1024, 2048, 4096 rows per CTA
+    if (cluster_sizes && o->lanes == 0) {  // the cluster engine as planned, and at 1024, 2048, 4096 rows per CTA
       for (int rc : {0, 1024, 2048, 4096}) {
         ClusterPlan P;
-        if (!plan_clusters(h, rc, P)) continue;
+        if (!cluster_classes(dev_limits, sizes.data(), nsys, rc, cls.data())) continue;
+        plan_clusters(h, cls, P);
         PK_CUDA(cudaMemcpyAsync(dcl, P.sys.data(), sizeof(BatchClSys) * nsys, cudaMemcpyHostToDevice, s));
         for (int rep = 0; rep < 2; ++rep) {
           if ((e = restore())) return e;
@@ -895,17 +866,18 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
       g_tune[key] = cfg;
     }
   }
+  if (cfg.lanes == -2) {
+    // the plan that runs; a device without the clusters that it asks for takes the fixed shape's, or rows
+    const int rc = choose_clusters(dev_limits, sizes.data(), nsys, cfg.rows_cta, kClRowsDefault, cls.data());
+    if (rc != cfg.rows_cta) cfg = rc > 0 ? cluster_cfg : row_cfg;
+    if (cfg.lanes == -2) plan_clusters(h, cls, plan);
+  }
   g_last = cfg;
   cudaEvent_t e0, e1;
   PK_CUDA(cudaEventCreate(&e0));
   PK_CUDA(cudaEventCreate(&e1));
-  if (cfg.lanes == -2) {
-    if (cfg.rows_cta != kClRowsDefault && !plan_clusters(h, cfg.rows_cta, plan)) {
-      set_error("cluster engine: no plan for the tuned rows per CTA");
-      return PK_ERR_ARG;
-    }
+  if (cfg.lanes == -2)
     PK_CUDA(cudaMemcpyAsync(dcl, plan.sys.data(), sizeof(BatchClSys) * nsys, cudaMemcpyHostToDevice, s));
-  }
   PK_CUDA(cudaEventRecord(e0, s));
   if (cfg.lanes == -2) {
     if ((e = run_clusters(dcl, plan, dqueue + 1, o->tol, o->maxit, s))) return e;
