@@ -82,9 +82,10 @@ enum {
                         120,000) and what fits nothing below run on one cluster; then, as long as
                         the matrix and the solver vectors fit the GPU's shared memory (7-point
                         stencils to about 270,000 rows), the whole loop runs in one cooperative
-                        launch that keeps them there (one solve at a time per process; a solve
-                        of another host thread meanwhile takes the graph).  Where CG's graph loop
-                        runs on more than 65,536 rows, both give the same bits.  In detail:
+                        launch that keeps them there.  The system alone decides, not what else
+                        runs: the launch queues until the GPU has room for all of its blocks at
+                        once, and pk_opts.wait_ns bounds the waits after that.  Where CG's graph
+                        loop runs on more than 65,536 rows, both give the same bits.  In detail:
                         PK_LOOP_PERSISTENT for pipelined FP64 CG with n <= PK_PERSISTENT_AUTO_N
                         and nnz <= PK_PERSISTENT_AUTO_NNZ, pipelined BiCGStab with n <=
                         PK_PERSISTENT_BICGSTAB_AUTO_N and nnz <= PK_PERSISTENT_BICGSTAB_AUTO_NNZ,

@@ -467,14 +467,11 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
                  A->nnz <= PK_PERSISTENT_BICGSTAB_AUTO_NNZ && A->stats.tiles_long == 0 &&
                  !(o->flags & PK_FLAG_TIMING) && bicgstab_persistent_usable(A);
   }
-  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
-  // other host thread's is running
+  // the shared-memory-resident loop, where the system fits it and is past the cluster's sizes
   bool sm = false;
-  SmTurn turn;
   if (o->loop == PK_LOOP_AUTO && !(persistent && cluster_size_work(A)) && o->variant == PK_VARIANT_PIPELINED &&
       !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
     if ((e = sm_bicgstab_usable(A, s, &sm))) return e;
-    sm = sm && turn.take();
     if (sm) persistent = false;
   }
   cudaEvent_t e0, e1;

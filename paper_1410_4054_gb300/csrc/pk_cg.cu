@@ -518,14 +518,11 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
                  A->nnz <= PK_PERSISTENT_AUTO_NNZ &&
                  !(o->flags & PK_FLAG_TIMING) && persistent_usable(A, o);
   }
-  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
-  // other host thread's is running
+  // the shared-memory-resident loop, where the system fits it and is past the cluster's sizes
   bool sm = false;
-  SmTurn turn;
   if (o->loop == PK_LOOP_AUTO && !(persistent && cluster_size_work(A)) && !sell &&
       o->variant == PK_VARIANT_PIPELINED && !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
     if ((e = sm_cg_usable(A, false, s, &sm))) return e;
-    sm = sm && turn.take();
     if (sm) persistent = false;
   }
   bool resident = false;

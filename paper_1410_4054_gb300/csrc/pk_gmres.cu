@@ -829,14 +829,11 @@ pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, p
     persistent = plain && A->n <= PK_PERSISTENT_GMRES_AUTO_N && A->nnz <= PK_PERSISTENT_GMRES_AUTO_NNZ &&
                  A->stats.tiles_long == 0 && !(o->flags & PK_FLAG_TIMING) && gmres_persistent_usable(A, m);
   }
-  // the shared-memory-resident loop, where the system fits it, is past the cluster's sizes, and no
-  // other host thread's is running
+  // the shared-memory-resident loop, where the system fits it and is past the cluster's sizes
   bool sm = false;
-  SmTurn turn;
   if (o->loop == PK_LOOP_AUTO && plain && !(persistent && cluster_size_work(A)) &&
       !(o->flags & (PK_FLAG_TIMING | PK_FLAG_NO_TMA))) {
     if ((e = sm_gmres_usable(A, s, &sm))) return e;
-    sm = sm && turn.take();
     if (sm) persistent = false;
   }
   if (!A->tma_ok && !persistent) { set_error("GMRES needs the tile engine"); return PK_ERR_ARG; }

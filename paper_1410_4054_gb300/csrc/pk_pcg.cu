@@ -219,13 +219,9 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
   }
   pk_status e;
   if ((e = pcg_setup())) return e;
-  // the shared-memory-resident loop, where the system fits it and no other host thread's is running
+  // the shared-memory-resident loop, where the system fits it
   bool sm = false;
-  SmTurn turn;
-  if (o->loop == PK_LOOP_AUTO && !(o->flags & PK_FLAG_TIMING)) {
-    if ((e = sm_cg_usable(A, true, s, &sm))) return e;
-    sm = sm && turn.take();
-  }
+  if (o->loop == PK_LOOP_AUTO && !(o->flags & PK_FLAG_TIMING) && (e = sm_cg_usable(A, true, s, &sm))) return e;
   cudaEvent_t e0, e1;
   PK_CUDA(cudaEventCreate(&e0));
   PK_CUDA(cudaEventCreate(&e1));

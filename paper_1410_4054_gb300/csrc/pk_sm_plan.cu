@@ -2,7 +2,6 @@
 // from other blocks, and every entry's column as a 16-bit index into the block's own rows or its
 // halo.  Built on the device from the tile schedule, once per handle.
 #include <algorithm>
-#include <atomic>
 #include <vector>
 
 #include "pk_guard.cuh"
@@ -78,8 +77,6 @@ __global__ void __launch_bounds__(kBlock) k_sm_publish(SmArgs a, const double* v
   const int row = blockIdx.x * kBlock + threadIdx.x;
   if (row < a.n) sm_publish(a, row, v[row], a.ep0);
 }
-
-std::atomic_flag g_turn = ATOMIC_FLAG_INIT;
 
 size_t exchange_bytes(const pk_csr* A) {
   return sizeof(ulonglong2) * (2 * (size_t)A->n + kSmSlotWords + kSmBcWords + kSmColWords);
@@ -208,14 +205,5 @@ void launch_sm_publish(const SmArgs& a, const double* v, cudaStream_t s) {
 }
 
 void sm_done(pk_csr* A, uint64_t epochs) { A->sm_epoch = epochs ? A->sm_epoch_next + epochs : 0; }
-
-bool SmTurn::take() {
-  if (!mine) mine = !g_turn.test_and_set(std::memory_order_acquire);
-  return mine;
-}
-
-SmTurn::~SmTurn() {
-  if (mine) g_turn.clear(std::memory_order_release);
-}
 
 }  // namespace pk
