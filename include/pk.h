@@ -143,7 +143,10 @@ enum {
 #define PK_FLAG_TEST_STALL 64u  /* testing the failure path: the CSR tile engine's producer
                                    issues no copies, so the first wait of every consumer runs
                                    out after pk_opts.wait_ns and the solve returns PK_TIMEOUT
-                                   (nothing is in flight; the context stays usable) */
+                                   (nothing is in flight; the context stays usable).  The
+                                   shared-memory loops' blocks send no sums, with the same
+                                   result.  The setup product runs without the tile engine, so
+                                   that the loop is what stalls */
 #define PK_FLAG_GM_SHIFT 128u   /* pipelined GMRES: the shift-invariant three-kernel form that
                                    Sec. 3.3 names (after l1-GMRES).  A v_{i-1} and
                                    w = (A - sigma_i I) v_{i-1} have the same part orthogonal

@@ -515,7 +515,7 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
 
   // setup: r0 = b - A x0, p0 = r0, r0* = r0, <r0, r0*>
   if ((e = T.begin(PK_SLOT_OTHER))) return e;
-  if ((e = launch_residual_init(A, v.b_dev, xd, r, p, r0s, !(o->flags & PK_FLAG_NO_TMA), s))) return e;
+  if ((e = launch_residual_init(A, v.b_dev, xd, r, p, r0s, setup_tma(o), s))) return e;
   if ((e = T.end())) return e;
   launch_zero_x(A, xd, s);
   launches += 2;

@@ -569,7 +569,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if (resident) {
     // r0, p0, <r0,r0>, <b,b>; then the whole iteration loop in one cooperative launch
     if ((e = T.begin(PK_SLOT_OTHER))) return e;
-    if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, true, s))) return e;
+    if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, setup_tma(o), s))) return e;
     if ((e = T.end())) return e;
     k_zero_x<<<A->grid, kBlock, 0, s>>>(row_args(A), xd);
     PK_CUDA(cudaGetLastError());
@@ -602,7 +602,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
 
   // setup: r0 = b - A x0, p0 = r0, <r0,r0>, <b,b>
   if ((e = T.begin(PK_SLOT_OTHER))) return e;
-  if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, !(o->flags & PK_FLAG_NO_TMA), s))) return e;
+  if ((e = launch_residual_init(A, bd, xd, r, p, nullptr, setup_tma(o), s))) return e;
   if ((e = T.end())) return e;
   k_zero_x<<<G, kBlock, 0, s>>>(ra, xd);
   launches += 2;

@@ -869,7 +869,7 @@ pk_status gmres_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, p
     if (sm) {
       double* r;
       if ((e = work_vec(A, 0, &r))) return e;
-      if ((e = launch_residual_init(A, v.b_dev, v.x_dev, r, nullptr, nullptr, true, s))) return e;
+      if ((e = launch_residual_init(A, v.b_dev, v.x_dev, r, nullptr, nullptr, setup_tma(o), s))) return e;
       e = launch_sm_gmres(A, v.b_dev, r, v.x_dev, m, A->basis, ld, A->small, A->small + kXiOff, o->maxit, s);
       launches += 2;  // the setup kernel, r_0 to the exchange
     } else {

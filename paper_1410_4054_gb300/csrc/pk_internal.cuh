@@ -44,7 +44,8 @@ struct DevState {
   cudaGraphConditionalHandle cond2;
   unsigned int gbar;      // grid-barrier arrivals of the persistent (cooperative) solve
   unsigned long long wait_ns;  // bound on a pipeline wait that should make progress
-  int32_t stall_test;          // PK_FLAG_TEST_STALL: the CSR tile producer issues no copies
+  int32_t stall_test;          // PK_FLAG_TEST_STALL: the CSR tile producer issues no copies, the
+                               // shared-memory loops' blocks send no sums
   int32_t stall_pad;
   // grid-resident CG loop: the last block of iteration i's reduction publishes epoch = i + 1
   // once alpha_i, beta_i and the exit decision are in place
@@ -462,9 +463,12 @@ void launch_true_residual(pk_csr* A, const double* b, const double* x, double* t
 RowArgs row_args(const pk_csr* A);
 
 // r0 = b - A x0 (to r, and p, r0s where given), <r0, r0>, <b, b> and the state that follows from them;
-// tma: the tile engine may be used.
+// tma: the tile engine may be used (setup_tma).
 pk_status launch_residual_init(const pk_csr* A, const double* b, const double* x, double* r, double* p, double* r0s,
                                bool tma, cudaStream_t s);
+// PK_FLAG_TEST_STALL is for the loop: a setup product on the tile engine would stall first, and the loop's
+// waits would never be entered.
+inline bool setup_tma(const pk_opts* o) { return !(o->flags & (PK_FLAG_NO_TMA | PK_FLAG_TEST_STALL)); }
 void launch_zero_x(const pk_csr* A, double* x, cudaStream_t s);
 pk_status check_opts(const pk_csr* A, const double* b, double* x, const pk_opts* o,
                      pk_info* info);

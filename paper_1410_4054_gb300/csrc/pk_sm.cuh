@@ -246,7 +246,7 @@ __device__ __forceinline__ void group_rows_shared(int G, const int32_t* srp, con
 struct SmBlock {
   int b, G, r0, rows, t0, t1, nh;
   int hoff;   // index of the first halo element: rows rounded up
-  int stall;  // PK_FLAG_TEST_STALL: no block sum is sent, so block 0's wait runs out
+  int stall;  // PK_FLAG_TEST_STALL: no block sum is sent, so block 0's wait runs out (GMRES: no column sum)
   const int32_t* halo;
 };
 

@@ -45,7 +45,9 @@ __global__ void __launch_bounds__(kSmThreads, 2) k_sm_gm(SmArgs a, SmGm g) {
   if (state_done(st)) return;  // decided by the setup kernel, the same for every block
   SmLayout L = sm_layout<2, 1>(smem, a);
   sm_shorten(L, a, 2 - g.nvec);
-  const SmBlock B = sm_begin(a, L);
+  SmBlock B = sm_begin(a, L);
+  const int stall = B.stall;  // (the columns' waits; the other loops run out sm_reduce's)
+  B.stall = 0;
   double* const cur = L.vec[0];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int maxit = st->maxit, trace_cap = st->trace_cap, m = g.m;
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(kSmThreads, 2) k_sm_gm(SmArgs a, SmGm g) {
       ulonglong2* const bc = mbc + (size_t)par * kSgCopies * kSgLd;
       double p[1] = {xip};
       block_sums<1, kSmThreads / 32>(p, [&](int, double t) {
-        if (!B.stall) ll_put(slots + B.b, t, me);
+        if (!stall) ll_put(slots + B.b, t, me);
       });  // (a barrier inside: w is complete)
       // a warp per column, or per part of one while there are fewer columns than warps
       const int lc = nc == 1 ? 3 : nc == 2 ? 2 : nc <= 4 ? 1 : 0, step = 32 << lc;
