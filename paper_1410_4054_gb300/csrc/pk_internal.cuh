@@ -530,10 +530,10 @@ __device__ __forceinline__ double sell_row(const SellArgs& s, int64_t base, int 
 
 // Kernels on the CSR tile engine take the instantiation with the paths of several lanes per row
 // when some tile needs one of them.
-// Systems whose update kernel takes the tile blocks' rows (blk_row) instead of equal chunks: the
-// ones that a shared-memory-resident loop may run, so that both sum in the same order.
 constexpr int kSmMaxRows = 655360;  // (the plan's column bitmap fits shared memory)
-inline bool rows_by_tile_block(const pk_csr* A) { return A->tma_ok && !A->tile_z0 && A->n <= kSmMaxRows; }
+// Systems whose CG update kernel takes the tile blocks' rows (blk_row) instead of equal chunks: the ones
+// that the shared-memory loop may run, so that both sum in the same order (pk_sm_plan.cu).
+bool rows_by_tile_block(const pk_csr* A);
 
 inline bool csr_irregular(const pk_csr* A) { return A->stats.tiles_long > 0 || A->stats.tiles_group > 0; }
 

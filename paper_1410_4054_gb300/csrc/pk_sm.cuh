@@ -26,6 +26,7 @@ namespace pk {
 constexpr int kSmThreads = kConsumers;  // 256: the consumer threads of the launched kernels
 constexpr int kSmMaxBlocks = 320;
 constexpr size_t kSmBytesMax = 225 * 1024;  // dynamic shared memory of a block (227 KB less the static part)
+constexpr size_t kSmBytesPair = 113 * 1024;  // ... of each of two blocks on an SM (228 KB, 1 KB of each reserved)
 constexpr int kSmFineRows = 65536;      // up to here blocks of kSmFineWork FMAs (see sm_tiles)
 constexpr int kSmFineWork = 1600;
 constexpr int kSmSums = 4;              // block sums per reduction
