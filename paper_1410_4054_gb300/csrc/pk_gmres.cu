@@ -65,7 +65,9 @@ struct GmArgs {
 // The reductions of this file stay FP64 trees (TREE, warp_sum_tree): classical Gram-Schmidt
 // divides their rounding by R_{i,i}, so any other rounding of equal quality moves xi_i of a badly
 // scaled matrix by as much as its parity bar (1.7e-12 against 1e-12 on rows of 9,000 nonzeros
-// among rows of 3), and the integer sums gain only 2 % of a step here.
+// among rows of 3), and the integer sums gain only 2 % of a step here.  (The loops that run in one launch
+// take the integer sums: there they gain 10 %, and the automatic choice gives them no such rows; see
+// pk_sm_gmres.cu.)
 template <int NV>
 __device__ __forceinline__ void gm_final_sums(const double* partials, double (&out)[NV]) {
   __shared__ double sm[NV];

@@ -10,6 +10,13 @@
 //   owner's, so the same bits), which lets the exchange travel during the reduction.
 // The basis stays in global memory (L2); every block touches its own rows only.  R and xi go to the
 // handle's scratch; block 0 solves R eta = xi at the end of a cycle and broadcasts eta.
+// Sums are the integer ones (warp_sums), where the launched form keeps FP64 trees (pk_gmres.cu): trees here
+// cost 10 % of a step (64^3, m = 30: 8.87 against 9.73 ms a solve) and are no closer to the oracle.  Largest
+// deviation of xi_i over the first cycle, integer / trees / launched form, on a 2D Laplacian with three rows
+// of 4,000 couplings among rows of 5 (four such matrices, one right-hand side): 2.2e-10 / 4.3e-10 / 2.2e-10,
+// 2.2e-10 / 1.8e-10 / 2.2e-10, 4.4e-10 / 4.5e-10 / 4.3e-10, 4.6e-10 / 4.4e-10 / 4.6e-10; the first with rows
+// and columns scaled by up to 100: 4.8e-12 / 4.8e-12 / 2.5e-12.  Classical Gram-Schmidt makes that of any
+// rounding; the one matrix where it passed a bar has rows longer than a tile, which this loop does not take.
 #include "pk_sm.cuh"
 
 namespace pk {
