@@ -481,9 +481,9 @@ pk_status bicgstab_solve(pk_csr* A, const double* b, double* x, const pk_opts* o
   if ((e = state_init(A, o, s))) return e;
   VecStage v;
   if ((e = stage_in(A, b, x, 14, 15, s, &v))) return e;
-  double *r, *p, *ap, *sv, *as, *r0s;
-  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (e = work_vec(A, 2, &ap)) ||
-      (e = work_vec(A, 3, &sv)) || (e = work_vec(A, 4, &as)) || (e = work_vec(A, 5, &r0s)))
+  double *r, *p = nullptr, *ap = nullptr, *sv = nullptr, *as, *r0s;  // (the shared-memory loop keeps p, Ap, s there)
+  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 4, &as)) || (e = work_vec(A, 5, &r0s)) ||
+      (!sm && ((e = work_vec(A, 1, &p)) || (e = work_vec(A, 2, &ap)) || (e = work_vec(A, 3, &sv)))))
     return e;
   const bool tma = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && o->variant == PK_VARIANT_PIPELINED && !persistent && !sm;
   // the classical form's SpMV runs on the same tile engine (only the fusion differs)

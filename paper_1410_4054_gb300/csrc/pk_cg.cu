@@ -545,8 +545,8 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if ((e = state_init(A, o, s))) return e;
   VecStage v;
   if ((e = stage_in(A, b, x, 14, 15, s, &v))) return e;
-  double *r, *p, *ap;
-  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (e = work_vec(A, 2, &ap))) return e;
+  double *r, *p, *ap = nullptr;  // (the shared-memory loop keeps Ap there)
+  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (!sm && (e = work_vec(A, 2, &ap)))) return e;
   const RowArgs ra = row_args(A);
   double* xd = v.x_dev;
   // The bulk-copy kernels read x in 16-byte units: a caller's x that is not 16-byte aligned or

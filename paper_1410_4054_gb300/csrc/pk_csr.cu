@@ -468,7 +468,9 @@ namespace pk {
 // Blocks and tiles of the shared-memory-resident loops.  Up to kSmFineRows rows the launched
 // kernels' tiles of 512 rows would leave most SMs without work (8 blocks at 4,096 rows, each with
 // 3,000 clocks of FP64 work per product); these blocks hold about kSmFineWork FMAs of an iteration.
-// Larger systems keep the launched kernels' blocks and with them their summation order.
+// Larger systems keep the launched kernels' blocks and with them their summation order.  Rows of at most
+// eight entries (every tile one thread per row) are shared out on the device, without the row pointers' way
+// to the host and back (sm_tiles_short).
 pk_status sm_tiles(pk_csr* A, int sms, cudaStream_t s) {
   A->sm_grid = A->grid_tma;
   A->sm_rows_max = A->blk_rows_max;
@@ -480,13 +482,14 @@ pk_status sm_tiles(pk_csr* A, int sms, cudaStream_t s) {
   A->sm_tile_perm = A->tile_perm;
   A->sm_irregular = csr_irregular(A);
   if (A->n > kSmFineRows || A->grid_tma >= sms) return PK_OK;
+  const int64_t work = (int64_t)A->nnz + 6 * (int64_t)A->n;
+  const int blocks = (int)std::max<int64_t>(A->grid_tma, std::min<int64_t>(sms, (work + kSmFineWork - 1) / kSmFineWork));
+  if (A->stats.row_max <= 8 && blocks <= kSmFineBlocks) return sm_tiles_short(A, blocks);
   std::vector<int32_t> rp(A->n + 1);
   PK_CUDA(cudaMemcpyAsync(rp.data(), A->rp, sizeof(int32_t) * (A->n + 1), cudaMemcpyDeviceToHost, s));
   PK_CUDA(cudaStreamSynchronize(s));
   CsrPlan P;
-  const int64_t work = (int64_t)A->nnz + 6 * (int64_t)A->n;
-  build_plan(A->n, A->nnz, rp, sms, P,
-             (int)std::max<int64_t>(A->grid_tma, std::min<int64_t>(sms, (work + kSmFineWork - 1) / kSmFineWork)));
+  build_plan(A->n, A->nnz, rp, sms, P, blocks);
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t b0 = up(4 * P.blk_row.size()), b1 = up(4 * P.tile_row.size()), b2 = up(4 * P.blk_tile.size()),
                b3 = up(P.tile_grp.size()), b4 = up(2 * P.tile_perm.size());
@@ -704,6 +707,7 @@ pk_status pk_csr_destroy(pk_csr* A) {
   if (A->blk_row) cudaFree(A->blk_row);
   if (A->sm_own) cudaFree(A->sm_own);
   if (A->sm_exchange) cudaFree(A->sm_exchange);
+  if (A->sm_col_own) cudaFree(A->sm_col_own);
   if (A->small) cudaFree(A->small);
   if (A->partials) cudaFree(A->partials);
   if (A->st) cudaFree(A->st);

@@ -400,6 +400,8 @@ struct pk_csr {
   void* sm_own = nullptr;
   int sm_halo_max = 0;              // most halo columns of one block
   void* sm_exchange = nullptr;      // exchange buffers, then the three arrays below
+  void* sm_col = nullptr;           // GMRES: its column exchange, with the plan that GMRES builds,
+  void* sm_col_own = nullptr;       // else an allocation of its own on first use
   int32_t* sm_halo_ptr = nullptr;   // sm_grid + 1
   int32_t* sm_halo = nullptr;
   uint16_t* sm_ci16 = nullptr;

@@ -229,8 +229,8 @@ pk_status pcg_jacobi_solve(pk_csr* A, const double* b, double* x, const pk_opts*
   if ((e = state_init(A, o, s))) return e;
   VecStage v;
   if ((e = stage_in(A, b, x, 14, 15, s, &v))) return e;
-  double *r, *p, *ap, *dinv;
-  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (e = work_vec(A, 2, &ap)) ||
+  double *r, *p, *ap = nullptr, *dinv;  // (the shared-memory loop keeps Ap there)
+  if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (!sm && (e = work_vec(A, 2, &ap))) ||
       (e = work_vec(A, 6, &dinv)))
     return e;
   double* xd = v.x_dev;

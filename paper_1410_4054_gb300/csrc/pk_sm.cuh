@@ -393,8 +393,8 @@ __device__ __forceinline__ int sm_reduce(const SmArgs& a, const SmBlock& B, doub
 // ------------------------------------------------------------------ host side (pk_sm_plan.cu)
 
 // The plan of A for this device (built on first use, kept with the handle): false if A does not
-// fit.  nvec vectors per row, ngather of them gathered.
-pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable);
+// fit.  columns: GMRES's column exchange too.
+pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable, bool columns = false);
 // Whether the system is small enough for one thread-block cluster to beat the SM loops.  Measured
 // on GB300 (us per iteration, cluster / SM loop; work = nnz + 6 n): CG 64x64 (45k) 4.3 / 5.4, 16^3
 // (52k) 4.6 / 6.3, 24^3 (176k) 7.2 / 6.6, 32^3 (420k) 11.0 / 6.4, 256x256 (720k) 16.0 / 6.7, P1
@@ -402,8 +402,13 @@ pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable);
 // 23.7 / 13.6: the cluster's 16 SMs slow down with the FP64 work, the SM loop hardly does.
 inline bool cluster_size_work(const pk_csr* A) { return (int64_t)A->nnz + 6 * (int64_t)A->n <= 120000; }
 
-// Blocks and tiles of A's SM loops (pk_csr.cu).
+// Blocks and tiles of A's SM loops (pk_csr.cu); those of a system of rows of at most eight entries on `blocks`
+// blocks, formed on the device when the plan is built (pk_sm_plan.cu).
 pk_status sm_tiles(pk_csr* A, int sms, cudaStream_t s);
+constexpr int kSmFineBlocks = 256;  // blocks that sm_tiles_short takes: one per thread of its kernel
+pk_status sm_tiles_short(pk_csr* A, int blocks);
+// GMRES's column exchange, on first use; usable = false: no memory for it.
+pk_status sm_columns(pk_csr* A, cudaStream_t s, bool* usable);
 // Whether a block of `kernel` with nvec vectors (ngather gathered) fits, with every block resident.
 bool sm_fits(const pk_csr* A, const void* kernel, int nvec, int ngather, size_t* smem);
 // Arguments of one launch whose epochs stay below ep0 + epochs.

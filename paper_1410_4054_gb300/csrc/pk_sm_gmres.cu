@@ -355,11 +355,11 @@ int sm_gm_vectors(const pk_csr* A, size_t* smem) {
 }  // namespace
 
 pk_status sm_gmres_usable(pk_csr* A, cudaStream_t s, bool* usable) {
-  pk_status e = sm_prepare(A, s, usable);
+  pk_status e = sm_prepare(A, s, usable, true);
   if (e || !*usable) return e;
   size_t smem;
   *usable = sm_gm_vectors(A, &smem) > 0;
-  return PK_OK;
+  return *usable ? sm_columns(A, s, usable) : PK_OK;
 }
 
 // Epochs that a solve of `iters` steps in `cycles` cycles uses at most, of each kind.

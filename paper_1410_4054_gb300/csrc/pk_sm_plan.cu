@@ -12,6 +12,7 @@ namespace pk {
 namespace {
 
 constexpr int kPlanThreads = 1024;
+constexpr size_t kColBytes = sizeof(ulonglong2) * kSmColWords;
 
 // The columns of block b's rows outside [r0, r1) as a bitmap, then their ranks.  EMIT = false:
 // cnt[b] = their number; true: the ascending list at halo + ptr[b], and ci16 of the block's entries.
@@ -78,8 +79,62 @@ __global__ void __launch_bounds__(kBlock) k_sm_publish(SmArgs a, const double* v
   if (row < a.n) sm_publish(a, row, v[row], a.ep0);
 }
 
+// What build_plan (pk_csr.cu) gives G blocks of a system whose rows have at most eight entries: block b's rows
+// start at the first row with rp[row] + 2 row >= wtot b / G, rounded down to a warp, and its tiles are
+// kTileRows rows each.  A thread per block.  most: the rows and entries of the largest block.
+__global__ void __launch_bounds__(kSmFineBlocks) k_sm_short_tiles(const int32_t* rp, int n, int G, double wtot,
+                                                                  int32_t* blk_row, int32_t* blk_tile,
+                                                                  int32_t* tile_row, int32_t* most) {
+  __shared__ int row[kSmFineBlocks + 1], wsum[kSmFineBlocks / 32], wmax[2][kSmFineBlocks / 32];
+  const int b = threadIdx.x, lane = b & 31, warp = b >> 5;
+  if (b < G) {
+    const double target = wtot * b / G;
+    int lo = 0, hi = n;
+    while (b && lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if ((double)rp[mid] + 2.0 * (double)mid < target) lo = mid + 1;
+      else hi = mid;
+    }
+    row[b] = lo / 32 * 32;
+  }
+  if (b == 0) row[G] = n;
+  __syncthreads();
+  const int r0 = b < G ? row[b] : 0, rows = b < G ? row[b + 1] - r0 : 0;
+  const int tiles = (rows + kTileRows - 1) / kTileRows;
+  int inc = tiles, mr = rows, mz = rows ? rp[r0 + rows] - rp[r0] : 0;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += up;
+    mr = max(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+    mz = max(mz, __shfl_xor_sync(0xffffffffu, mz, o));
+  }
+  if (lane == 31) wsum[warp] = inc;
+  if (lane == 0) {
+    wmax[0][warp] = mr;
+    wmax[1][warp] = mz;
+  }
+  __syncthreads();
+  int first = inc - tiles;
+  for (int w = 0; w < warp; ++w) first += wsum[w];
+  if (b < G) {
+    blk_row[b] = r0;
+    blk_tile[b] = first;
+    for (int t = 0; t < tiles; ++t) tile_row[first + t] = r0 + t * kTileRows;
+    if (b == G - 1) {
+      blk_row[G] = n;
+      blk_tile[G] = first + tiles;
+      tile_row[first + tiles] = n;
+    }
+  }
+  if (b < 2) {
+    int m = 0;
+    for (int w = 0; w < kSmFineBlocks / 32; ++w) m = max(m, wmax[b][w]);
+    most[b] = m;
+  }
+}
+
 size_t exchange_bytes(const pk_csr* A) {
-  return sizeof(ulonglong2) * (2 * (size_t)A->n + kSmSlotWords + kSmBcWords + kSmColWords);
+  return sizeof(ulonglong2) * (2 * (size_t)A->n + kSmSlotWords + kSmBcWords);
 }
 
 // Whether the loops may fit, by what the handle knows without a plan: the matrix and three vectors, without
@@ -90,20 +145,32 @@ bool may_fit(const pk_csr* A, int sms) {
   return sm_bytes(A->blk_rows_max, A->blk_nnz_max, 0, 3, 1) <= most;
 }
 
-pk_status build(pk_csr* A, cudaStream_t s) {
+pk_status build(pk_csr* A, bool columns, cudaStream_t s) {
   const int G = A->sm_grid, words = (A->n + 31) / 32;
   const size_t smem = sizeof(uint32_t) * 2 * (size_t)words;
   for (auto k : {k_sm_plan<false>, k_sm_plan<true>})
     PK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  std::vector<int32_t> ptr(G + 1, 0);
+  std::vector<int32_t> ptr(G + 2, 0);
   if (pk_status e = ensure_state(A)) return e;
-  // the counts in the reductions' scratch (three sums per block); one allocation, one wait: a handle's
-  // first solve pays for them
+  // the counts in the reductions' scratch (three sums per block), the largest block's rows and entries after
+  // them; one allocation, one wait: a handle's first solve pays for them
   int32_t* cnt = reinterpret_cast<int32_t*>(A->partials);
+  const bool tiles_due = A->sm_rows_max == 0;  // (see sm_tiles_short)
+  if (tiles_due) {
+    k_sm_short_tiles<<<1, kSmFineBlocks, 0, s>>>(A->rp, A->n, G, (double)A->nnz + 2.0 * (double)A->n,
+                                                 const_cast<int32_t*>(A->sm_blk_row),
+                                                 const_cast<int32_t*>(A->sm_blk_tile),
+                                                 const_cast<int32_t*>(A->sm_tile_row), cnt + G);
+    PK_CUDA(cudaGetLastError());
+  }
   k_sm_plan<false><<<G, kPlanThreads, smem, s>>>(A->rp, A->ci, A->sm_blk_row, words, cnt, nullptr, nullptr, nullptr);
   PK_CUDA(cudaGetLastError());
-  PK_CUDA(cudaMemcpyAsync(ptr.data(), cnt, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, s));
+  PK_CUDA(cudaMemcpyAsync(ptr.data(), cnt, sizeof(int32_t) * (G + 2), cudaMemcpyDeviceToHost, s));
   PK_CUDA(cudaStreamSynchronize(s));
+  if (tiles_due) {
+    A->sm_rows_max = ptr[G];
+    A->sm_nnz_max = ptr[G + 1];
+  }
   int sum = 0, most = 0;
   for (int b = 0; b < G; ++b) {
     const int c = ptr[b];
@@ -118,9 +185,10 @@ pk_status build(pk_csr* A, cudaStream_t s) {
   need = sm_bytes(A->sm_rows_max, A->sm_nnz_max, most, 3, 1);
   if (need > kSmBytesMax) return PK_OK;  // no loop fits
   const auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
-  const size_t b0 = up(exchange_bytes(A)), b1 = up(sizeof(int32_t) * (G + 1)), b2 = up(sizeof(int32_t) * std::max(1, sum));
+  const size_t bx = up(exchange_bytes(A)), b0 = bx + (columns ? up(kColBytes) : 0), b1 = up(sizeof(int32_t) * (G + 1)), b2 = up(sizeof(int32_t) * std::max(1, sum));
   PK_CUDA(cudaMalloc(&A->sm_exchange, b0 + b1 + b2 + sizeof(uint16_t) * ((size_t)A->nnz + 64)));
   char* d = reinterpret_cast<char*>(A->sm_exchange);
+  if (columns) A->sm_col = d + bx;
   A->sm_halo_ptr = reinterpret_cast<int32_t*>(d + b0);
   A->sm_halo = reinterpret_cast<int32_t*>(d + b0 + b1);
   A->sm_ci16 = reinterpret_cast<uint16_t*>(d + b0 + b1 + b2);
@@ -135,7 +203,7 @@ pk_status build(pk_csr* A, cudaStream_t s) {
 
 }  // namespace
 
-pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable) {
+pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable, bool columns) {
   *usable = A->sm_state == 1;
   if (A->sm_state) return PK_OK;
   A->sm_state = -1;
@@ -146,7 +214,7 @@ pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable) {
   // (guarded here and not only at the entry: a failed host allocation is no reason to fail the solve)
   const pk_status e = guarded([&]() -> pk_status {
     const pk_status t = sm_tiles(A, sms, s);
-    return t ? t : build(A, s);
+    return t ? t : build(A, columns, s);
   });
   if (e == PK_ERR_OOM) {  // no memory for the plan: the launched loop needs none
     cudaGetLastError();
@@ -157,6 +225,44 @@ pk_status sm_prepare(pk_csr* A, cudaStream_t s, bool* usable) {
   }
   *usable = A->sm_state == 1;
   return e;
+}
+
+// A handle's first solve pays for its plan, so a small system's is short: with the row pointers copied back,
+// shared out by the host and the blocks copied down again, and with GMRES's column exchange (680 KB) in every
+// solver's allocation, the first solve of few iterations on a new handle took up to 120 us longer than on the
+// launched loop.  Measured (us of the first solve, 6 to 10 iterations; launched loop / plan by the host /
+// this): CG 150^2 241 / 347 / 233, 250^2 304 / 406 / 324, 32^3 296 / 427 / 315, 40^3 397 / 475 / 316,
+// BiCGStab 32^3 352 / 462 / 402; the second solve there 201 / 143 / 142, 264 / 147 / 149, 181 / 136 / 136,
+// 238 / 145 / 141 and 229 / 153 / 164.
+pk_status sm_tiles_short(pk_csr* A, int blocks) {
+  auto up = [](size_t b) { return (b + 63) & ~size_t(63); };
+  const size_t w0 = up(blocks + 1), w1 = up(blocks + 1), w2 = (size_t)A->n / kTileRows + blocks + 2;
+  PK_CUDA(cudaMalloc(&A->sm_own, sizeof(int32_t) * (w0 + w1 + w2)));
+  int32_t* d = static_cast<int32_t*>(A->sm_own);
+  A->sm_grid = blocks;
+  A->sm_blk_row = d;
+  A->sm_blk_tile = d + w0;
+  A->sm_tile_row = d + w0 + w1;
+  A->sm_tile_grp = nullptr;
+  A->sm_tile_perm = nullptr;
+  A->sm_irregular = false;
+  A->sm_rows_max = A->sm_nnz_max = 0;  // with the blocks, when the plan is built
+  return PK_OK;
+}
+
+pk_status sm_columns(pk_csr* A, cudaStream_t s, bool* usable) {
+  if (A->sm_col) return PK_OK;
+  const cudaError_t e = cudaMalloc(&A->sm_col_own, kColBytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    A->sm_col_own = nullptr;
+    *usable = false;
+    return PK_OK;
+  }
+  PK_CUDA(e);
+  PK_CUDA(cudaMemsetAsync(A->sm_col_own, 0, kColBytes, s));
+  A->sm_col = A->sm_col_own;
+  return PK_OK;
 }
 
 // By the handle alone, not by a plan that an earlier solve may have made: a graph solve gives the same bits
@@ -190,6 +296,7 @@ pk_status sm_args(pk_csr* A, uint64_t epochs, cudaStream_t s, SmArgs* out) {
   // solve that did not say how many it used
   if (A->sm_epoch == 0 || A->sm_epoch + epochs >= (1ull << 32)) {
     PK_CUDA(cudaMemsetAsync(A->sm_exchange, 0, exchange_bytes(A), s));
+    if (A->sm_col) PK_CUDA(cudaMemsetAsync(A->sm_col, 0, kColBytes, s));
     A->sm_epoch = 1;
   }
   SmArgs a;
@@ -205,7 +312,7 @@ pk_status sm_args(pk_csr* A, uint64_t epochs, cudaStream_t s, SmArgs* out) {
   a.vex = reinterpret_cast<ulonglong2*>(A->sm_exchange);
   a.slots = a.vex + 2 * (size_t)A->n;
   a.bc = a.slots + kSmSlotWords;
-  a.col = a.bc + kSmBcWords;
+  a.col = static_cast<ulonglong2*>(A->sm_col);
   a.n = A->n;
   a.max_rows = A->sm_rows_max;
   a.max_nnz = A->sm_nnz_max;
