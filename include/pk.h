@@ -78,22 +78,23 @@ enum {
                         the block partials itself in a fixed order; for n <=
                         PK_PERSISTENT_MAX_N.  Larger n, other variants, precisions, GMRES
                         with PK_FLAG_CGS2 or PK_FLAG_GM_SHIFT return PK_ERR_ARG */
-  PK_LOOP_AUTO = 3,  /* by size.  The smallest pipelined FP64 CG and BiCGStab solves (nnz + 6 n up to
-                        120,000) and what fits nothing below run on one cluster; then, as long as
-                        the matrix and the solver vectors fit the GPU's shared memory (7-point
-                        stencils to about 270,000 rows), the whole loop runs in one cooperative
-                        launch that keeps them there.  The system alone decides, not what else
-                        runs: the launch queues until the GPU has room for all of its blocks at
-                        once, and pk_opts.wait_ns bounds the waits after that.  Where CG's graph
-                        loop runs on more than 65,536 rows, both give the same bits.  In detail:
-                        PK_LOOP_PERSISTENT for pipelined FP64 CG with n <= PK_PERSISTENT_AUTO_N
-                        and nnz <= PK_PERSISTENT_AUTO_NNZ, pipelined BiCGStab with n <=
-                        PK_PERSISTENT_BICGSTAB_AUTO_N and nnz <= PK_PERSISTENT_BICGSTAB_AUTO_NNZ,
-                        and pipelined GMRES (one Gram-Schmidt pass) with n <=
-                        PK_PERSISTENT_GMRES_AUTO_N and nnz <= PK_PERSISTENT_GMRES_AUTO_NNZ (and
-                        no PK_FLAG_TIMING; for BiCGStab and GMRES also no rows of very
-                        different lengths, stats.tiles_long == 0) when the device can run it,
-                        PK_LOOP_GRAPH otherwise */
+  PK_LOOP_AUTO = 3,  /* for pipelined FP64 CG (not PK_FLAG_SELL), BiCGStab and GMRES (one
+                        Gram-Schmidt pass, not PK_FLAG_GM_SHIFT) without PK_FLAG_TIMING, the
+                        first of these that applies:
+                        1. PK_LOOP_PERSISTENT up to nnz + 6 n = 120,000, within the limits of 3;
+                        2. with the matrix and the solver vectors in the GPU's shared memory, as
+                           long as they fit (7-point stencils to about 270,000 rows; no row
+                           longer than 4096 nonzeros; not PK_FLAG_NO_TMA): the whole loop in one
+                           cooperative launch;
+                        3. PK_LOOP_PERSISTENT up to PK_PERSISTENT_AUTO_N rows and
+                           PK_PERSISTENT_AUTO_NNZ nonzeros (BiCGStab, GMRES: their own limits
+                           below, and no rows of very different lengths, stats.tiles_long == 0),
+                           when the device can run it.  Not CG with PK_PRECOND_JACOBI;
+                        4. PK_LOOP_GRAPH, as for everything else.
+                        The system alone decides, not what else runs: the launch of 2 queues
+                        until the GPU has room for all of its blocks at once, and
+                        pk_opts.wait_ns bounds the waits after that.  On more than 65,536 rows
+                        CG without preconditioner gives the same bits on 2 and 4 */
   PK_LOOP_RESIDENT = 4 /* pipelined FP64 CG only: the whole iteration loop in one cooperative
                         launch of one block per SM.  Each iteration's update (x, r, p) and fused
                         SpMV run back to back in the launch; the SpMV of a block waits only for

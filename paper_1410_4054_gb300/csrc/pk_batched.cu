@@ -760,8 +760,8 @@ pk_status batched_solve(int32_t nsys, pk_csr* const* A, const double* const* b, 
   const int lanes_auto = mean_len <= 12 ? 1 : mean_len <= 24 ? 2 : mean_len <= 48 ? 4 : 8;
   // lanes -1: the tile engine; -2: the cluster engine; otherwise the row kernel with the given
   // lanes.  Automatic: the cluster engine for FP64 batches of rows short enough for one thread each
-  // (512 shifted 2D Laplacians of 1,024 to 65,536 rows to 1e-10 on GB300: 10.9 ms a call, the row kernel at
-  // 512 threads x 2 36.9 ms; 200 of them 5.6 / 25.5 ms, 24 1.6 / 11.6 ms, 2 1.1 / 3.3 ms: a large system
+  // (512 shifted 2D Laplacians of 1,024 to 65,536 rows to 1e-10 on GB300: 10.6-10.9 ms a call, the row kernel at
+  // 512 threads x 2 30.0-36.9 ms; 200 of them 5.6 / 25.5 ms, 24 1.6 / 11.6 ms, 2 1.1 / 3.3 ms: a large system
   // runs on up to 16 SMs instead of one block, and its vectors stay in shared memory); longer rows keep
   // the row kernel's lanes.
   const TuneVal cluster_cfg{kClRowsDefault / 8, 4096 / kClRowsDefault, -2, kClRowsDefault};

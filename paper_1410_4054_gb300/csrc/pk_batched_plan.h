@@ -53,8 +53,11 @@ int fixed_cluster(const Limits& d, int n, int rows_cta) {
 // and barriers overlap another's FP64 work; t, the rows per CTA, is the largest the CTAs hold as long
 // as the batch fills the device (fewer barriers per row), else smaller (an iteration's latency).
 // The short systems at the end of the queues run on shares half as large: their iterations are the
-// batch's tail.  Measured (512 shifted 2D Laplacians, ms): 256 threads x 2048 rows, two per SM 13.5;
-// this with t everywhere 11.4, halved up to t rows 11.2, up to 2 t rows 10.9, up to 4 t rows 11.4.
+// batch's tail.  Measured (512 shifted 2D Laplacians, ms): 256 threads x 2048 rows, two per SM 13.5, this
+// 10.9.  With t everywhere / halved up to t / 2 t / 4 t rows (rectangles, sides log-uniform): 512 of 32-256
+// 9.6 / 9.6 / 9.0 / 9.5, another 512 8.9 / 8.2 / 8.2 / 8.7, 200 of them 4.3 / 4.3 / 3.6 / 3.8, 60 of them 2.4 in
+// all, 300 of 100-250 12.0 / 12.1 / 12.1 / 11.8, 400 of 128 x 128 10.1 / 10.1 / 10.1 / 10.4; only short systems
+// lose by it: 1,000 of 20-90 3.2 / 3.5 / 3.7 / 3.6, 2,000 of 16-64 3.7 / 3.8 / 3.8 / 3.8.
 template <class Limits>
 bool cluster_classes(const Limits& d, const int* n, int nsys, int rows_cta, int* cls) {
   int t = d.max_rows(0);

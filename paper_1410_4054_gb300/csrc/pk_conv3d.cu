@@ -61,10 +61,10 @@ struct ConvArgs {
 // the output tiles in turn (tcgen05.ld, bias, ReLU or mask, BF16 store).  Planes pass through
 // kTcStages staging buffers and kTcSlots accumulator slots in tensor memory; a slot is free once the
 // (up to three) output tiles that read it have.  One block per SM.
-// Measured (64^3, launches back to back): 18.6 us before (one MMA per tap, two blocks per SM), 12.2
-// us now (one MMA warp: 14.7); 72^3: 23.8 -> 14.5; 32^3: 10.7 -> 10.4, which is the launch, the
-// prologue (barriers, tensor memory, weights: 1.2 us) and one run's latency.  The 16.8 MB in and out
-// take 2.4 us of memory time.
+// Measured (launches back to back): 64^3 17.9 us before (one MMA per tap, two blocks per SM, plain
+// launches), 10.6 now (with plain launches 12.2, and 14.7 with one MMA warp); 72^3: 22.9 -> 12.0; 32^3:
+// 10.3 -> 10.6, which is the launch, the prologue (barriers, tensor memory, weights: 1.2 us) and one run's
+// latency.  The 16.8 MB in and out take 2.4 us of memory time.
 // A box lands in the no-swizzle K-major layout of the MMA's A operand: a core matrix is 8
 // voxels consecutive in x (8 x 16 bytes), the two K halves are kTcHalf bytes apart (leading
 // byte offset) and consecutive y rows kTcRow bytes apart (stride byte offset); a tap (dy, dx) is the

@@ -6,7 +6,9 @@
 // kernels and computes them with the same schedule (tile_rows), so per iteration no matrix byte
 // leaves the SM; what remains is the FP64 work and two kinds of exchange between blocks through
 // L2, both of 16-byte words that carry their own epoch, so that neither needs a fence or a flag
-// (a reader polls the data itself and each 8-byte half is valid once its epoch matches):
+// (a reader polls the data itself and each 8-byte half is valid once its epoch matches; the steps are
+// those of the publicly documented low-latency protocol of collective libraries, NCCL's LL: data and flag
+// in one 8-byte store):
 //   - the gathered vector: every block publishes its rows, and fetches the rows it gathers from
 //     other blocks (its halo, a sorted list built with the plan) into shared memory, where the
 //     product's gathers find own and halo rows by one 16-bit index;
@@ -27,7 +29,13 @@ constexpr int kSmThreads = kConsumers;  // 256: the consumer threads of the laun
 constexpr int kSmMaxBlocks = 320;
 constexpr size_t kSmBytesMax = 225 * 1024;  // dynamic shared memory of a block (227 KB less the static part)
 constexpr size_t kSmBytesPair = 113 * 1024;  // ... of each of two blocks on an SM (228 KB, 1 KB of each reserved)
-constexpr int kSmFineRows = 65536;      // up to here blocks of kSmFineWork FMAs (see sm_tiles)
+// Up to kSmFineRows rows blocks of kSmFineWork FMAs (see sm_tiles).  Measured (us per iteration, 800 / 1200 /
+// 1600 / 2400 / 3200 FMAs, and the launched kernels' blocks): CG 150^2 7.2 7.2 7.2 7.5 7.1, 8.4; 40^3 7.5 in
+// all five, 9.2; P1 elasticity 4,752 rows 8.6 8.6 9.6 8.2 10.6, 11.9; SPD power law 20,000 rows 11.7 11.7 11.6
+// 11.7 13.1, 15.7; BiCGStab 32^3 14.8 14.9 14.8 14.8 15.5, 17.9; GMRES 32^3 12.5 12.5 12.5 12.5 13.9, 17.9: flat
+// up to 2,400.  The row limit: 250^2 8.0 against 7.5 with the launched blocks, 40^3 (64,000 rows) 7.5 against
+// 9.2; beyond it the launched kernels have a block for nearly every SM (41^3 9.4 against 9.5).
+constexpr int kSmFineRows = 65536;
 constexpr int kSmFineWork = 1600;
 constexpr int kSmSums = 4;              // block sums per reduction
 constexpr int kSmWords = 4;             // scalars broadcast per reduction
