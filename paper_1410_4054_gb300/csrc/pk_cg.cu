@@ -629,7 +629,7 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if (tma && (e = tma_setup())) return e;
   const CsrTiles ct = csr_tiles_of(A);
   const bool irr = csr_irregular(A);  // some tile needs several lanes per row
-  const int32_t* urows = rows_by_tile_block(A) ? A->blk_row : nullptr;
+  const int32_t* urows = !sell && rows_by_tile_block(A) ? A->blk_row : nullptr;
   const int Gt = A->grid_tma, Gs = urows ? Gt : A->grid_stream;
   double* part = A->partials;
   DevState* dst = A->st;

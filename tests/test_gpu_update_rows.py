@@ -41,3 +41,19 @@ def test_update_time_does_not_follow_the_row_lengths():
     even, uneven = update_us(two_bands(n, 1, 1)), update_us(two_bands(n, 1, 30))
     print(f"update kernel: {even:.2f} us on even rows, {uneven:.2f} us on uneven ones")
     assert uneven <= 1.5 * even
+
+
+def test_sell_loop_keeps_its_own_rows():
+    """SELL sums in an order of its own, so its update kernel has no reason to take the tile blocks' rows: on 39,744
+    unknowns of 45 entries these are 304 blocks of 130 rows, where equal chunks are 78 (5 us per iteration more)."""
+    a = W.fe_elasticity_3d(23)
+    A = pk.CSRMatrix.from_workload(a)
+    b = torch.from_numpy(W.manufactured(a, seed=1)[1]).cuda()
+
+    def us(flags):
+        return min(pk.cg_solve(A, b, torch.zeros_like(b), tol=0.0, maxit=60, loop="graph", flags=flags)["solve_ms"]
+                   for _ in range(10)) * 1e3 / 60
+
+    tiles, sell = us(0), us(pk.FLAG_SELL)
+    print(f"CG on the CSR tiles {tiles:.1f} us per iteration, on SELL {sell:.1f}")
+    assert sell <= 1.05 * tiles
