@@ -88,8 +88,8 @@ enum {
                            cooperative launch;
                         3. PK_LOOP_PERSISTENT up to PK_PERSISTENT_AUTO_N rows and
                            PK_PERSISTENT_AUTO_NNZ nonzeros (BiCGStab, GMRES: their own limits
-                           below, and no rows of very different lengths, stats.tiles_long == 0),
-                           when the device can run it.  Not CG with PK_PRECOND_JACOBI;
+                           below) without rows of very different lengths (stats.tiles_long ==
+                           0), when the device can run it.  Not CG with PK_PRECOND_JACOBI;
                         4. PK_LOOP_GRAPH, as for everything else.
                         The system alone decides, not what else runs: the launch of 2 queues
                         until the GPU has room for all of its blocks at once, and

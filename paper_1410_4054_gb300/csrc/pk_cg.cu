@@ -514,8 +514,11 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
     }
     persistent = true;
   } else if (o->loop == PK_LOOP_AUTO && !sell) {
+    // (one thread of the cluster walks a row.  Rows of very different lengths, us per iteration, cluster / in
+    // shared memory: 900 rows, the longest of 105 15.9 / 7.1, 303 38.8 / 7.4; 7,225 rows, 205 25.4 / 7.4, 1,006
+    // 119 / 11.6; power law of 2,000 rows 29.6 / 8.9; 10,000 rows, the longest of 9,002 1,034 / 25.4 launched)
     persistent = o->variant == PK_VARIANT_PIPELINED && A->n <= PK_PERSISTENT_AUTO_N &&
-                 A->nnz <= PK_PERSISTENT_AUTO_NNZ &&
+                 A->nnz <= PK_PERSISTENT_AUTO_NNZ && A->stats.tiles_long == 0 &&
                  !(o->flags & PK_FLAG_TIMING) && persistent_usable(A, o);
   }
   // the shared-memory-resident loop, where the system fits it and is past the cluster's sizes
