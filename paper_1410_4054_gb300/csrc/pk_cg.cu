@@ -552,11 +552,13 @@ pk_status cg_solve(pk_csr* A, const double* b, double* x, const pk_opts* o, pk_i
   if ((e = work_vec(A, 0, &r)) || (e = work_vec(A, 1, &p)) || (!sm && (e = work_vec(A, 2, &ap)))) return e;
   const RowArgs ra = row_args(A);
   double* xd = v.x_dev;
-  // The bulk-copy kernels read x in 16-byte units: a caller's x that is not 16-byte aligned or
-  // has odd length is iterated in a padded library copy.
-  const bool tma_engine = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && !persistent && !sm;
+  // The launched update kernels read x in 16-byte units, the bulk-copy ones whole units only: a
+  // caller's x that is not 16-byte aligned (for those: or has odd length) is iterated in a padded
+  // library copy.
+  const bool launched = !persistent && !sm;
+  const bool tma_engine = A->tma_ok && !(o->flags & PK_FLAG_NO_TMA) && launched;
   double* x_copy_back = nullptr;
-  if (tma_engine && (((uintptr_t)xd & 15) || (A->n & 1))) {
+  if ((launched && ((uintptr_t)xd & 15)) || (tma_engine && (A->n & 1))) {
     double* xi;
     if ((e = work_vec(A, 13, &xi))) return e;
     PK_CUDA(cudaMemcpyAsync(xi, xd, sizeof(double) * A->n, cudaMemcpyDeviceToDevice, s));
